@@ -674,18 +674,6 @@ int sq_append_kv(sq_cache* c, sq_seq seq, int32_t n_tokens, const void* k, const
     size_t n_ups = 0;  // of them, passed to the kernel
     rc = fence_taken_pages(c, plan.taken, stream);
     if (rc != SQ_OK) return undo(rc);
-    if (plan.cow) {
-        CowArgs ca;
-        ca.pool = c->pool;
-        ca.num_pages = g.num_pages;
-        ca.L = g.L; ca.Hkv = g.Hkv; ca.P = g.P; ca.D = g.D;
-        ca.src_page = plan.cow_old;
-        ca.dst_page = plan.cow_new;
-        ca.rows = plan.cow_rows;
-        ca.err = c->d_err;
-        cudaError_t e = launch_cow_copy(ca, c->num_sms, st);
-        if (e != cudaSuccess) return undo(cuda_status(e));
-    }
     // rows go to slot-space positions pos0 .. pos0 + n - 1 (the last page's
     // free slots, then the fresh pages)
     const int64_t end = (int64_t)plan.pos0 + plan.n_new;
@@ -708,8 +696,11 @@ int sq_append_kv(sq_cache* c, sq_seq seq, int32_t n_tokens, const void* k, const
         a.n_tok = (int32_t)(pe - pb);
         a.lens.n = 0;
         if (b == 0) n_ups = fill_lens(ups, 0, &a.lens);  // an in-page append is one launch
+        // the launch that writes the fresh copy's first rows also copies the old ones
+        a.cow = {0, 0, 0};
+        if (b == 0 && plan.cow) a.cow = {plan.cow_old, plan.cow_new, plan.cow_rows};
         a.err = c->d_err;
-        cudaError_t e = launch_append(a, c->num_sms, st);
+        cudaError_t e = launch_append(a, st);
         if (e != cudaSuccess) return undo(cuda_status(e));
     }
     note_writes(c, plan.pages.data(), plan.pages.size(), stream);
@@ -759,19 +750,6 @@ int sq_append_kv_batch(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, const vo
         plan_len_updates(c, seqs[i], plans[i], old_versions[i], st, &ups[i]);
     int rc = fence_taken_pages(c, taken, stream);
     if (rc != SQ_OK) return undo(n_seqs, rc);
-    for (int32_t i = 0; i < n_seqs; ++i) {
-        if (!plans[i].cow) continue;
-        CowArgs ca;
-        ca.pool = c->pool;
-        ca.num_pages = g.num_pages;
-        ca.L = g.L; ca.Hkv = g.Hkv; ca.P = g.P; ca.D = g.D;
-        ca.src_page = plans[i].cow_old;
-        ca.dst_page = plans[i].cow_new;
-        ca.rows = plans[i].cow_rows;
-        ca.err = c->d_err;
-        cudaError_t e = launch_cow_copy(ca, c->num_sms, st);
-        if (e != cudaSuccess) return undo(n_seqs, cuda_status(e));
-    }
     for (int32_t b = 0; b < n_seqs; b += kAppendBatchMax) {
         AppendBatchArgs a;
         a.pool = c->pool;
@@ -784,8 +762,10 @@ int sq_append_kv_batch(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, const vo
         a.n = std::min(kAppendBatchMax, n_seqs - b);
         AppendLens& l = a.lens;
         l.n = 0;
+        a.n_cow = 0;
         for (int32_t i = 0; i < a.n; ++i) {
             const AppendPlan& pl = plans[b + i];
+            if (pl.cow) a.cow[a.n_cow++] = {pl.cow_old, pl.cow_new, pl.cow_rows};
             a.page[i] = pl.pages[0];                 // the page holding slot position pos0
             a.slot[i] = pl.pos0 % g.P;
             // a sequence's plan updates go all into this launch, or none do
@@ -802,7 +782,7 @@ int sq_append_kv_batch(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, const vo
             }
         }
         a.err = c->d_err;
-        cudaError_t e = launch_append_batch(a, c->num_sms, st);
+        cudaError_t e = launch_append_batch(a, st);
         if (e != cudaSuccess) return undo(n_seqs, cuda_status(e));
     }
     {

@@ -92,7 +92,14 @@ cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
 cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStream_t st);
 
 // ---- append / copy-on-write / eviction --------------------------------------
-constexpr int kAppendMaxPages = 64;
+// Pages one append launch writes at most (their ids are launch arguments):
+// 32,768 tokens at 64-token pages, 4,096 at 8-token ones.
+constexpr int kAppendMaxPages = 512;
+
+// Copy-on-write of the first `rows` rows of a page, in every plane.
+struct CowCopy {
+    int32_t src_page, dst_page, rows;
+};
 
 // Words of cached decode plans that an append rewrites (in stream order, by
 // block 0): the row limit of the run holding the appended sequence's last
@@ -118,6 +125,8 @@ struct AppendArgs {
     int32_t n_pages;
     int32_t pages[kAppendMaxPages];
     AppendLens lens;
+    CowCopy cow;                // rows > 0: copied by this launch too
+    int32_t n_blocks;           // blocks that append (set by the launcher)
     int* err;
 };
 
@@ -136,14 +145,9 @@ struct AppendBatchArgs {
     int32_t page[kAppendBatchMax];
     int32_t slot[kAppendBatchMax];
     AppendLens lens;
-    int* err;
-};
-
-struct CowArgs {
-    __nv_bfloat16* pool;
-    int64_t num_pages;
-    int32_t L, Hkv, P, D;
-    int32_t src_page, dst_page, rows;
+    int32_t n_cow;              // copies made by this launch too
+    CowCopy cow[kAppendBatchMax];
+    int32_t n_blocks;           // blocks that append (set by the launcher)
     int* err;
 };
 
@@ -164,9 +168,8 @@ struct EvictArgs {
     int* err;
 };
 
-cudaError_t launch_append(const AppendArgs& a, int num_sms, cudaStream_t st);
-cudaError_t launch_append_batch(const AppendBatchArgs& a, int num_sms, cudaStream_t st);
-cudaError_t launch_cow_copy(const CowArgs& a, int num_sms, cudaStream_t st);
+cudaError_t launch_append(AppendArgs& a, cudaStream_t st);
+cudaError_t launch_append_batch(AppendBatchArgs& a, cudaStream_t st);
 // Shared memory of one eviction CTA for a tile size and ring depth (plus one
 // zero tile when the plan zeroes rows).
 int evict_smem_bytes(int tile_rows, int D, int stages, bool zero_tiles = false);
