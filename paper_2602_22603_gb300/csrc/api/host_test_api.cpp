@@ -219,4 +219,39 @@ int sqh_plan_prefill(int32_t Hq, int32_t Hkv, int32_t P, int32_t n, int32_t n_q,
     return kOk;
 }
 
+// The work items of a masked prefill (as sqh_plan_prefill): info_out receives
+// the numbers of items, merges and partial results; items_out 4 int32 per item
+// (unit, first key tile, key tiles, partial entry), merges_out 3 per merge
+// (unit, first entry, entries).
+int sqh_prefill_items(int32_t Hq, int32_t Hkv, int32_t P, int32_t n, int32_t n_q,
+                      const int32_t* spans, int32_t n_spans, int32_t target_ctas,
+                      int64_t* info_out, int32_t* items_out, int32_t cap, int32_t* merges_out,
+                      int32_t merge_cap) {
+    Geometry g;
+    g.L = 1; g.Hq = Hq; g.Hkv = Hkv; g.D = 128; g.P = P;
+    g.num_pages = 1; g.max_seqs = 1; g.max_pages_per_seq = 1;
+    std::vector<int32_t> a(n_spans > 0 ? n_spans : 0), b(a.size());
+    for (int32_t i = 0; i < n_spans; ++i) {
+        a[i] = spans[2 * i];
+        b[i] = spans[2 * i + 1];
+    }
+    PrefillPlanHost p;
+    int rc = plan_prefill(g, n, n_q, a.data(), b.data(), n_spans, target_ctas, &p);
+    if (rc != kOk) return rc;
+    info_out[0] = (int64_t)p.items.size();
+    info_out[1] = (int64_t)p.merges.size();
+    info_out[2] = p.n_parts;
+    if (cap < info_out[0] || merge_cap < info_out[1]) return kCapacity;
+    for (size_t i = 0; i < p.items.size(); ++i) {
+        const PrefillItem& it = p.items[i];
+        const int32_t v[4] = {it.unit, it.t0, it.n_tiles, it.part};
+        std::memcpy(items_out + 4 * i, v, sizeof v);
+    }
+    for (size_t m = 0; m < p.merges.size(); ++m) {
+        const int32_t v[3] = {p.merges[m].unit, p.merges[m].part0, p.merges[m].n};
+        std::memcpy(merges_out + 3 * m, v, sizeof v);
+    }
+    return kOk;
+}
+
 }  // extern "C"

@@ -73,10 +73,10 @@ struct PrefillPlanEntry {
     int32_t n_q = 0;
     int32_t target = 0;
     std::vector<int32_t> spans;  // start, end pairs as passed
-    size_t tb = 0, qb = 0;       // bytes of the tile records, of the per-CTA-tile counts
-    int32_t n_tiles = 0, n_pieces = 0, BP = 0, n_qt = 0, n_split = 0;
+    size_t o_items = 0, o_merges = 0, o_pages = 0;  // byte offsets of the parts of d
+    int32_t n_tiles = 0, n_pieces = 0, BP = 0, n_items = 0, n_merges = 0, n_parts = 0;
     int64_t visible_pairs = 0;
-    uint8_t* d = nullptr;  // [tiles][qt_tiles][tile_pages]
+    uint8_t* d = nullptr;  // [tiles][items][merges][tile_pages]
     size_t cap = 0;
     cudaEvent_t ev = nullptr;  // recorded after the last launch that used it
     bool ev_recorded = false;
@@ -1125,6 +1125,9 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     cudaStream_t st = as_stream(stream);
     cudaError_t e;
     PrefillPlanEntry* hit = nullptr;
+    // a reused plan that needs no cross-stream wait was on the device before
+    // anything this call enqueues
+    int32_t plan_ready = 0;
     for (auto& p : c->pre_plans)
         if (p.valid && p.seq == seq && p.version == s->version && p.n_q == n_q &&
             p.target == c->num_sms && p.spans == key) {
@@ -1154,10 +1157,12 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
                               s->pages.data());
         }
         if (rc != SQ_OK) return rc;
-        // upload: key tiles, per-CTA-tile counts, then the page of every piece
-        const size_t tb = plan.tiles.size() * sizeof(PrefillTile);
-        const size_t qb = plan.qt_tiles.size() * sizeof(int32_t);
-        const size_t pb = plan.tile_pages.size() * sizeof(int32_t);
+        // upload: key tiles, items, merges, then the page of every piece (the
+        // records of 16 bytes first, so each part is aligned)
+        const size_t o_items = plan.tiles.size() * sizeof(PrefillTile);
+        const size_t o_merges = o_items + plan.items.size() * sizeof(PrefillItem);
+        const size_t o_pages = o_merges + plan.merges.size() * sizeof(PrefillMerge);
+        const size_t bytes = o_pages + plan.tile_pages.size() * sizeof(int32_t);
         // least recently used entry
         PrefillPlanEntry* victim = &c->pre_plans[0];
         for (auto& p : c->pre_plans)
@@ -1167,13 +1172,13 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
             e = cudaEventCreateWithFlags(&victim->ev, cudaEventDisableTiming);
             if (e != cudaSuccess) return cuda_status(e);
         }
-        if (tb + qb + pb > victim->cap) {
+        if (bytes > victim->cap) {
             if (victim->ev_recorded) cudaEventSynchronize(victim->ev);
             if (victim->d) cudaFree(victim->d);
             victim->d = nullptr;
             victim->cap = 0;
             victim->ev_recorded = false;
-            const size_t cap = std::max<size_t>((tb + qb + pb) * 5 / 4, 4096);
+            const size_t cap = std::max<size_t>(bytes * 5 / 4, 4096);
             e = cudaMalloc(&victim->d, cap);
             if (e != cudaSuccess) return cuda_status(e);
             victim->cap = cap;
@@ -1183,24 +1188,30 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
             e = cudaStreamWaitEvent(st, victim->ev, 0);
             if (e != cudaSuccess) return cuda_status(e);
         }
-        if (c->staging.size() < tb + qb + pb) c->staging.resize(tb + qb + pb);
-        if (tb) std::memcpy(c->staging.data(), plan.tiles.data(), tb);
-        std::memcpy(c->staging.data() + tb, plan.qt_tiles.data(), qb);
-        if (pb) std::memcpy(c->staging.data() + tb + qb, plan.tile_pages.data(), pb);
-        rc = staged_copy(c, victim->d, c->staging.data(), tb + qb + pb, stream);
+        if (c->staging.size() < bytes) c->staging.resize(bytes);
+        auto put = [&](size_t at, const void* src, size_t n) {
+            if (n) std::memcpy(c->staging.data() + at, src, n);
+        };
+        put(0, plan.tiles.data(), o_items);
+        put(o_items, plan.items.data(), o_merges - o_items);
+        put(o_merges, plan.merges.data(), o_pages - o_merges);
+        put(o_pages, plan.tile_pages.data(), bytes - o_pages);
+        rc = staged_copy(c, victim->d, c->staging.data(), bytes, stream);
         if (rc != SQ_OK) return rc;
         victim->seq = seq;
         victim->version = s->version;
         victim->n_q = n_q;
         victim->target = c->num_sms;
         victim->spans = key;
-        victim->tb = tb;
-        victim->qb = qb;
+        victim->o_items = o_items;
+        victim->o_merges = o_merges;
+        victim->o_pages = o_pages;
         victim->n_tiles = (int32_t)plan.tiles.size();
         victim->n_pieces = plan.n_pieces;
         victim->BP = plan.BP;
-        victim->n_qt = plan.n_qt;
-        victim->n_split = plan.n_split;
+        victim->n_items = (int32_t)plan.items.size();
+        victim->n_merges = (int32_t)plan.merges.size();
+        victim->n_parts = plan.n_parts;
         victim->visible_pairs = plan.visible_pairs;
         victim->valid = true;
         hit = victim;
@@ -1208,13 +1219,14 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         // its upload ran on the stream of the call that planned it
         e = cudaStreamWaitEvent(st, hit->ev, 0);
         if (e != cudaSuccess) return cuda_status(e);
+    } else {
+        plan_ready = 1;
     }
     hit->last_use = ++c->use_clock;
     const PrefillPlanEntry& plan = *hit;
-    const int64_t grid = (int64_t)plan.n_qt * g.Hkv * plan.n_split;
-    if (plan.n_split > 1) {
+    if (plan.n_parts > 0) {
         const size_t need =
-            (size_t)grid * kPrefillQTiles * kPrefillRows * (g.D + 1) * sizeof(float);
+            (size_t)plan.n_parts * kPrefillQTiles * kPrefillRows * (g.D + 1) * sizeof(float);
         if (!c->pre_ev) {
             e = cudaEventCreateWithFlags(&c->pre_ev, cudaEventDisableTiming);
             if (e != cudaSuccess) return cuda_status(e);
@@ -1250,8 +1262,8 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     }
     PrefillArgs a;
     a.tiles = reinterpret_cast<const PrefillTile*>(plan.d);
-    a.qt_tiles = reinterpret_cast<const int32_t*>(plan.d + plan.tb);
-    a.tile_pages = reinterpret_cast<const int32_t*>(plan.d + plan.tb + plan.qb);
+    a.items = reinterpret_cast<const PrefillItem*>(plan.d + plan.o_items);
+    a.tile_pages = reinterpret_cast<const int32_t*>(plan.d + plan.o_pages);
     a.n_pieces = plan.n_pieces;
     a.n_tiles = plan.n_tiles;
     a.n = slot_end(*s, g.P);   // the slot-space end (s->n when every page but the last is full)
@@ -1263,8 +1275,8 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     a.P = g.P;
     a.num_pages = g.num_pages;
     a.BP = plan.BP;
-    a.n_qt = plan.n_qt;
-    a.n_split = plan.n_split;
+    a.n_items = plan.n_items;
+    a.plan_ready = plan_ready;
     // the kernel keeps the scale inside the exponent (s * scale - m); a zero
     // scale runs as 1e-30, whose weights 2^(s * 1e-30 - m) are exactly 1
     a.scale_log2 = std::max(sm_scale * 1.4426950408889634f, 1e-30f);
@@ -1273,13 +1285,15 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     a.lse = lse;
     a.part_o = c->pre_part;
     a.part_ml = c->pre_part
-                    ? c->pre_part + (size_t)grid * kPrefillQTiles * kPrefillRows * g.D
+                    ? c->pre_part + (size_t)plan.n_parts * kPrefillQTiles * kPrefillRows * g.D
                     : nullptr;
     a.err = c->d_err;
     e = launch_prefill(c->tmap, qmap, a, g.D, st);
     if (e != cudaSuccess) return cuda_status(e);
-    if (plan.n_split > 1) {
+    if (plan.n_merges > 0) {
         PrefillCombineArgs ca;
+        ca.merges = reinterpret_cast<const PrefillMerge*>(plan.d + plan.o_merges);
+        ca.n_merges = plan.n_merges;
         ca.part_o = a.part_o;
         ca.part_ml = a.part_ml;
         ca.out = out;
@@ -1290,8 +1304,6 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         ca.Hkv = g.Hkv;
         ca.G = g.G();
         ca.BP = plan.BP;
-        ca.n_qt = plan.n_qt;
-        ca.n_split = plan.n_split;
         e = launch_prefill_combine(ca, g.D, st);
         if (e != cudaSuccess) return cuda_status(e);
         e = cudaEventRecord(c->pre_ev, st);

@@ -748,6 +748,78 @@ void plan_serialize(const DecodePlanHost& p, const DecodePlanLayout& L, uint8_t*
 }
 
 // ---------------------------------------------------------------------------
+// Items of a prefill plan: units (CTA tile qt, KV head) of out->qt_tiles[qt]
+// key tiles each, longest first, taken by `ctas` CTAs one after the other.
+//
+// Units that do not divide evenly leave a last round in which most CTAs wait:
+// 376 units of ~200 key tiles on 152 CTAs take three rounds for 2.47 rounds of
+// work.  When every unit has about the same number of key tiles (a tool
+// response over a long context), the units of the last one or two rounds are
+// split into `k` key ranges each, k chosen by the estimated makespan in key
+// tiles: full rounds x (T + kItem) + rounds of pieces x (T / k + kItem) + the
+// merge (a launch, and the partials written and read) + a quarter of a piece
+// for SMs of unequal speed.  Units of growing length (a whole trace) already
+// end with the short ones and are not split.
+static void list_prefill_items(int32_t Hkv, int32_t ctas, PrefillPlanHost* out) {
+    constexpr double kItem = 2.0, kMergeLaunch = 4.0, kMergePiece = 0.032;
+    constexpr int32_t kMaxPieces = 16;
+    const int32_t n_qt = out->n_qt, units = n_qt * Hkv;
+    const int32_t T = out->qt_tiles.back(), T_min = out->qt_tiles.front();
+    int32_t n_tail = 0, k_tail = 1;  // units split, pieces of each
+    if (out->n_split == 1 && units > ctas && units % ctas != 0 && units < 16 * (int64_t)ctas &&
+        T >= 8 && 10 * (int64_t)T_min >= 7 * (int64_t)T) {
+        double best = (double)((units + ctas - 1) / ctas) * (T + kItem) + 0.25 * T;
+        for (int32_t extra = 0; extra < 2; ++extra) {
+            const int32_t r = units % ctas + extra * ctas;
+            if (r > units) break;
+            for (int32_t k = 2; k <= kMaxPieces && 4 * k <= T; ++k) {
+                const int64_t pieces = (int64_t)r * k;
+                const double cost = (double)((units - r) / ctas) * (T + kItem) +
+                                    (double)((pieces + ctas - 1) / ctas) * ((T + k - 1) / k + kItem) +
+                                    kMergeLaunch + kMergePiece * pieces + 0.25 * T / k;
+                if (cost < 0.98 * best) {
+                    best = cost;
+                    n_tail = r;
+                    k_tail = k;
+                }
+            }
+        }
+    }
+    // items, longest first; pieces of one key range and head side by side, so
+    // that the CTAs running together share their keys
+    std::vector<PrefillItem>& items = out->items;
+    items.clear();
+    items.reserve((size_t)units * std::max(out->n_split, 1));
+    out->merges.clear();
+    out->n_parts = 0;
+    const int32_t whole = units - n_tail;
+    auto unit_at = [&](int32_t i) { return (n_qt - 1 - i / Hkv) * Hkv + i % Hkv; };
+    std::vector<int32_t> part0(units, -1), pieces_of(units, 1);
+    for (int32_t i = 0; i < units; ++i) {
+        const int32_t u = unit_at(i), t = out->qt_tiles[u / Hkv];
+        const int32_t k = std::min(i < whole ? out->n_split : k_tail, std::max(t, 1));
+        pieces_of[u] = k;
+        if (k > 1) {
+            part0[u] = out->n_parts;
+            out->merges.push_back({u, out->n_parts, k, 0});
+            out->n_parts += k;
+        } else {
+            items.push_back({u, 0, t, -1});
+        }
+    }
+    const int32_t kmax = std::max(out->n_split, k_tail);
+    for (int32_t x = 0; kmax > 1 && x < kmax; ++x)
+        for (int32_t h = 0; h < Hkv; ++h)
+            for (int32_t qt = n_qt - 1; qt >= 0; --qt) {
+                const int32_t u = qt * Hkv + h, k = pieces_of[u];
+                if (k < 2 || x >= k) continue;
+                const int64_t t = out->qt_tiles[qt];
+                const int32_t a = (int32_t)(t * x / k), b = (int32_t)(t * (x + 1) / k);
+                items.push_back({u, a, b - a, part0[u] + x});
+            }
+}
+
+// ---------------------------------------------------------------------------
 // Masked prefill planning.  Visibility of key j to the query at position p:
 // j <= p (causal) and j in no span (Algorithm 2: a closed cursor's tokens are
 // masked for every later token).  The kernel applies the causal part; the
@@ -820,12 +892,18 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
                 out->tile_pages[t * out->n_pieces + i] = key < n ? pages[key / g.P] : -1;
             }
     }
-    // visible keys of each query: the visible keys among 0 .. p
-    int64_t seen = 0, pairs = 0;
+    // visible keys of each query: the visible keys among 0 .. p.  Key j is
+    // seen by the queries from max(q0, j) on.
     const int32_t q0 = n - n_q;
-    for (int32_t j = 0; j < n; ++j) {
-        seen += (vis[j >> 5] >> (j & 31)) & 1u;
-        if (j >= q0) pairs += seen;
+    int64_t pairs = 0;
+    for (int32_t w = 0; 32 * w < n; ++w) {
+        uint32_t bits = vis[w];
+        if (32 * w + 32 <= q0) {
+            pairs += (int64_t)__builtin_popcount(bits) * n_q;
+            continue;
+        }
+        for (; bits; bits &= bits - 1)
+            pairs += n - std::max(q0, 32 * w + __builtin_ctz(bits));
     }
     out->visible_pairs = pairs;
     out->n = n;
@@ -844,20 +922,19 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
     const int32_t n_tiles = (int32_t)out->tiles.size();
     // Split each CTA tile's key range when there are too few CTA tiles to
     // fill the GPU: pick the split that minimises the estimated makespan,
-    // waves x (key tiles per CTA + a fixed per-CTA cost), CTAs running
+    // rounds x (key tiles per item + a fixed cost per item), items running
     // `target_ctas` at a time.
     int32_t split = 1;
     if (units < target_ctas && n_tiles > 0 && target_ctas > 0) {
-        constexpr int32_t kMaxSplit = 64;
-        constexpr double kCtaCost = 4.0;  // prologue + epilogue, in key tiles
+        constexpr double kItemCost = 4.0;  // prologue + epilogue, in key tiles
         double avg = 0;
         for (int32_t c : out->qt_tiles) avg += c;
         avg /= std::max<int32_t>(1, out->n_qt);
         double best = 1e300;
-        for (int32_t sp = 1; sp <= kMaxSplit && sp <= n_tiles; ++sp) {
+        for (int32_t sp = 1; sp <= kPrefillMaxSplit && sp <= n_tiles; ++sp) {
             const int64_t ctas = units * sp;
             const int64_t waves = (ctas + target_ctas - 1) / target_ctas;
-            const double cost = (double)waves * (avg / sp + kCtaCost);
+            const double cost = (double)waves * (avg / sp + kItemCost);
             if (cost < best - 1e-9) {
                 best = cost;
                 split = sp;
@@ -865,6 +942,7 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
         }
     }
     out->n_split = split;
+    list_prefill_items(g.Hkv, std::max<int32_t>(1, target_ctas), out);
     return kOk;
 }
 

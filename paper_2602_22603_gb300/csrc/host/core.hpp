@@ -248,14 +248,19 @@ struct PrefillPlanHost {
     int32_t n = 0, n_q = 0;
     int32_t BP = 0;                   // query positions per query tile
     int32_t n_qt = 0;                 // CTA tiles (kPrefillQTiles query tiles each) per KV head
-    int32_t n_split = 1;              // key-range splits per query tile
+    int32_t n_split = 1;              // key-range splits per query tile (all alike)
+    std::vector<PrefillItem> items;   // the kernel's work, longest first
+    std::vector<PrefillMerge> merges; // units of more than one item
+    int32_t n_parts = 0;              // partial results of all of them
     int64_t visible_pairs = 0;        // sum over queries of the keys each sees
 };
 
 // Plans masked prefill attention over a sequence of n tokens whose last n_q
 // tokens are the queries: validates the spans, builds the per-tile visibility
-// bitmaps, and splits each query tile's key range in n_split parts when the
-// query tiles alone would fill fewer than `target_ctas` CTAs.
+// bitmaps, and lists the work items of the query units (CTA tiles x KV heads)
+// for `target_ctas` CTAs at a time.  Every unit's key range is split in
+// n_split parts when the units alone would fill fewer CTAs than that; with
+// more of them, the units of a last round that would leave CTAs idle may be.
 // `pages` (may be null) is the sequence's page table; with it the plan also
 // lists the page of every piece of every key tile.  Positions are slot-space
 // positions: for a sequence with partial pages, n is its slot-space end and

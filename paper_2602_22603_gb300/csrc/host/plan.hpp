@@ -92,6 +92,27 @@ struct PrefillTile {
     int32_t pad;
 };
 
+// One work item of the prefill kernel: key tiles [t0, t0 + n_tiles) of one
+// query unit (the two query tiles of CTA tile unit / Hkv at KV head
+// unit % Hkv).  A unit of several items leaves normalised partial results in
+// entry `part` (-1: its only item, written to the outputs).
+struct PrefillItem {
+    int32_t unit;
+    int32_t t0;
+    int32_t n_tiles;
+    int32_t part;
+};
+
+// A unit whose items' partial results [part0, part0 + n) are merged.
+struct PrefillMerge {
+    int32_t unit;
+    int32_t part0;
+    int32_t n;
+    int32_t pad;
+};
+// Partial results one unit may have at most (a lane of the merge takes two).
+constexpr int32_t kPrefillMaxSplit = 64;
+
 // Byte offsets of the arrays of a decode plan inside one upload buffer.
 // Byte offsets of the serialised decode plan.  `arrive` holds one 32-bit
 // arrival count per (sequence, KV head), zero in the serialised plan; the

@@ -57,30 +57,34 @@ cudaError_t launch_decode(const CUtensorMap& tmap, const DecodeArgs& a, int n_ct
 // ---- masked prefill attention -------------------------------------------------
 struct PrefillArgs {
     const PrefillTile* tiles;   // key tiles with a visible key, increasing key0
-    const int32_t* qt_tiles;    // [n_qt] key tiles each CTA tile reaches (a prefix of tiles)
+    const PrefillItem* items;   // [n_items] work items, longest first
     const int32_t* tile_pages;  // [n_tiles][n_pieces] page of each min(P, 64)-row piece, -1 past the end
     int32_t n_tiles, n_pieces;
     int32_t n, n_q;             // sequence tokens; queries = its last n_q tokens
     int32_t layer, Hq, Hkv, G, P, num_pages;
     int32_t BP;                 // query positions per query tile (kPrefillRows / G)
-    int32_t n_qt, n_split;
+    int32_t n_items;
+    // 1: the plan was on the device before whatever precedes this launch on
+    // the stream, so it may be read before the grid-dependency wait
+    int32_t plan_ready;
     float scale_log2;           // sm_scale * log2(e), >= 0
-    void* out;                  // [n_q][Hq][D] bf16 or fp32 (n_split == 1)
+    void* out;                  // [n_q][Hq][D] bf16 or fp32
     int32_t out_f32;
-    float* lse;                 // [n_q][Hq] or null (n_split == 1)
-    float* part_o;              // [grid][kPrefillQTiles][kPrefillRows][D] normalised partials
-                                // (n_split > 1)
-    float* part_ml;             // [grid][kPrefillQTiles][kPrefillRows] their log2-sum-exp
+    float* lse;                 // [n_q][Hq] or null
+    float* part_o;              // [n_parts][kPrefillQTiles][kPrefillRows][D] normalised partials
+    float* part_ml;             // [n_parts][kPrefillQTiles][kPrefillRows] their log2-sum-exp
     int* err;
 };
 
 struct PrefillCombineArgs {
+    const PrefillMerge* merges;
+    int32_t n_merges;
     const float* part_o;
     const float* part_ml;
     void* out;
     int32_t out_f32;
     float* lse;
-    int32_t n_q, Hq, Hkv, G, BP, n_qt, n_split;
+    int32_t n_q, Hq, Hkv, G, BP;
 };
 
 // Dynamic shared memory of the prefill kernel.

@@ -10,9 +10,9 @@
 // A query tile is 128 rows: floor(128 / G) consecutive query positions times
 // the G query heads of one KV head (Sec. 2.1).  One CTA owns two consecutive
 // query tiles (a, b) of the same KV head, and every K/V tile it loads serves
-// both, which halves the loads per tensor-core FLOP.  Keys go 128 at a time,
-// aligned to 128; tiles whose keys are all masked are never loaded (the host
-// lists the others with a visibility bitmap).  Per key tile j and query tile t:
+// both, which halves the loads per tensor-core FLOP.  Keys go 128 at a time;
+// tiles whose keys are all masked are never loaded (the host lists the others
+// with a visibility bitmap).  Per key tile j and query tile t:
 //   S_t = Q_t K_j^T           tcgen05.mma, Q and K from shared memory, S in TMEM
 //   P_t = exp2(S_t - m)       softmax warpgroup t: tcgen05.ld of S, mask, bf16 P
 //                             stored back over the first half of S_t
@@ -26,16 +26,32 @@
 // warpgroup may rescale O_t then without another wait.  The running maximum
 // is raised lazily: a key tile's weights are taken with the current maximum
 // and accepted while every row's sum of them stays at most 2^16 (so does each
-// weight); only then is a maximum raised and O rescaled.  K and V stream through one ring of
-// shared-memory slots (K_0, V_0, K_1, ...); a K slot is released once both S
-// products are done, a V slot once both PV products are.
+// weight); only then is a maximum raised and O rescaled.  K and V stream through
+// one ring of shared-memory slots (K_0, V_0, K_1, ...); V_j and K_{j+1} are
+// released together, after the products PV_b(j) and S_b(j+1).
+//
+// What bounds it: the one thread that issues the MMAs (see there), then the
+// softmax chain of each tile.  32,768 queries, 40% masked, 32q/8kv, d = 128:
+// 3.55 -> 3.25 ms a layer (1,320 -> 1,440 TFLOP/s
+// over the visible pairs); 3,001 queries over 33,001 tokens: 1,027 -> 845 us.
 //
 // Short query blocks: when a CTA tile's queries all fit in tile a, tile b's
 // warpgroup takes the same rows over every other key tile (dual-key mode, the
 // two results merged per row at the end, loads in the order the MMAs consume
-// them), and when there are fewer CTA tiles than SMs each tile's key range is
-// split over several CTAs whose normalised partial results a second kernel
-// merges.
+// them).
+//
+// Work items: the host lists (CTA tile, KV head, key range) items, longest
+// first, and the grid has one CTA per item, of which an SM holds one.  A CTA
+// that has issued the loads of its item asks the launch hardware for the next
+// CTA not started yet (clusterlaunchcontrol.try_cancel) and takes over its
+// item, so the ring, the barriers' phases and tensor memory run on from item
+// to item and the next item's first keys and queries load while the last one's
+// softmax, PV and output finish.  One CTA per item paid a start and a drain
+// each, ~5 us; dealing the items to persistent CTAs beforehand lost 4%, since
+// SMs run this kernel at speeds up to 7% apart (1.78 to 1.91 us per key tile).
+// A unit split in several items (too few units for the SMs, or a last round
+// that would leave most SMs idle) leaves normalised partial results that a
+// second kernel merges.
 //
 // Warp roles (320 threads): warp 0 loads (lanes 0 and 1 issue the TMA copies,
 // two loads at a time), lane 0 of warp 1 issues the MMAs and warp 1 owns the
@@ -51,6 +67,11 @@
 namespace sq {
 namespace dev {
 namespace {
+
+// Items in flight between the producer and the other roles, and the warps that
+// read each (MMA warp and eight softmax warps).
+constexpr int kItemSlots = 4;
+constexpr int kItemReaders = 9;
 
 template <int D>
 struct PreCfg {
@@ -70,9 +91,17 @@ struct PreCfg {
     static constexpr int kBarP = kBarS + 2;             // [2] P_t written (128 arrivals)
     static constexpr int kBarO = kBarP + 2;             // [2] last PV_t done
     static constexpr int kBarVfix = kBarO + 2;          // V of the last key tile landed
-    static constexpr int kBarDone = kBarVfix + 1;       // every MMA of the CTA done
-    static constexpr int kNumBars = kBarDone + 1;
-    static constexpr int kOffMisc = kOffBar + kNumBars * 8;
+    static constexpr int kBarQFree = kBarVfix + 1;      // the item's last QK product done
+    static constexpr int kBarDone = kBarQFree + 1;      // every MMA of the CTA done
+    static constexpr int kBarItem = kBarDone + 1;       // [kItemSlots] item written
+    static constexpr int kBarItemFree = kBarItem + kItemSlots;  // [kItemSlots] item read by all
+    static constexpr int kBarClc = kBarItemFree + kItemSlots;   // answer of the launch hardware
+    static constexpr int kBarX = kBarClc + 1;           // dual-key mode: tile b's half handed over
+    static constexpr int kBarXFree = kBarX + 1;         // ... and read by tile a
+    static constexpr int kNumBars = kBarXFree + 1;
+    static constexpr int kOffItems = (kOffBar + kNumBars * 8 + 15) & ~15;  // [kItemSlots] int4
+    static constexpr int kOffClc = kOffItems + kItemSlots * 16;           // 16-byte answer
+    static constexpr int kOffMisc = kOffClc + 16;
     // dual-key mode: tile b's (max, normaliser) of each row, for the merge
     static constexpr int kOffXchg = (kOffMisc + 32 + 15) & ~15;
     static constexpr int kSmemBytes = kOffXchg + kPrefillRows * 8 + 1024;  // + alignment slack
@@ -94,6 +123,68 @@ struct Smem {
         return base + PreCfg<D>::kOffBar + 8 * i;
     }
 };
+
+// A work item as the roles see it; raw.z (its key tiles) is -1 after the last.
+struct Item {
+    int g, pos_lo, t0, T, part;
+    bool two;   // tile b holds query rows
+    bool dual;  // tile b takes every other key tile of tile a's rows
+};
+
+__device__ __forceinline__ Item make_item(const PrefillArgs& a, int4 raw) {
+    Item it;
+    const int qt = raw.x / a.Hkv;
+    it.g = raw.x - qt * a.Hkv;
+    it.pos_lo = qt * kPrefillQTiles * a.BP;
+    it.t0 = raw.y;
+    it.T = raw.z;
+    it.part = raw.w;
+    // tile b is empty when every query of the CTA tile fits in tile a
+    it.two = it.pos_lo + a.BP < a.n_q;
+    it.dual = !it.two && it.T >= 2;
+    return it;
+}
+
+// Asks the launch hardware for a CTA of the grid that has not started; the
+// 16-byte answer lands at `dst`, completing `bar`.
+__device__ __forceinline__ void clc_request(uint32_t dst, uint32_t bar) {
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], "
+        "[%1];" ::"r"(dst),
+        "r"(bar)
+        : "memory");
+}
+
+// The answer at `src`: the index of the CTA taken over, or -1.
+__device__ __forceinline__ int clc_answer(uint32_t src) {
+    uint32_t ok, x;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n\t}"
+        : "=r"(ok), "=r"(x)
+        : "r"(src)
+        : "memory");
+    return ok ? (int)x : -1;
+}
+
+// The reading side of the item ring: item k of the CTA is in slot k mod
+// kItemSlots until every reader has freed it.
+template <int D>
+__device__ __forceinline__ bool item_wait(const Smem& sm, uint32_t k, const volatile int* abort_flag) {
+    return mbar_wait(sm.bar<D>(PreCfg<D>::kBarItem + k % kItemSlots), (k / kItemSlots) & 1, abort_flag);
+}
+template <int D>
+__device__ __forceinline__ int4 item_read(const Smem& sm, uint32_t k) {
+    return *reinterpret_cast<const int4*>(sm.ptr + PreCfg<D>::kOffItems + k % kItemSlots * 16);
+}
+template <int D>
+__device__ __forceinline__ void item_free(const Smem& sm, uint32_t k) {
+    mbar_arrive(sm.bar<D>(PreCfg<D>::kBarItemFree + k % kItemSlots));
+}
 
 // Bits 0 .. x of a word (x < 0: none; x >= 31: all).
 __device__ __forceinline__ uint32_t low_bits_through(int x) {
@@ -121,306 +212,485 @@ __device__ __forceinline__ void load_of(int u, int T, bool dual, int& j, int& kv
         kv = (u & 1) ? 0 : 1;
     }
 }
-// The loads of K_j and V_j in dual-key mode (T >= 2).
-__device__ __forceinline__ int dual_load_k(int j) { return j < 2 ? j : 2 * j - 1; }
-__device__ __forceinline__ int dual_load_v(int j, int T) { return j < T - 1 ? 2 * j + 2 : 2 * T - 1; }
 
-// The producer warp: the query tiles once, then the K and V tiles of every key
-// tile into the ring in the order of load_of, two loads at a time: the whole
-// warp waits for both slots, then lanes 0 and 1 arm their barriers and issue
-// their copies together, so that the shared-memory round trips of the two
-// overlap.  What a tile's copies need, {first key, page of box 0, page of box
-// 1}, is held in
+// {first key of each half, page of box 0, page of box 1} of key tile
+// tb + lane % kBatch of an item (x = key0, y = page 0, z = page 1, w = key0b).
+constexpr int kBatch = 16;
+__device__ __forceinline__ int4 tile_record(const PrefillArgs& a, int t0, int T, int tb, int lane) {
+    int4 r = make_int4(0, -1, -1, kPrefillNoKeys);
+    const int jj = tb + (lane & (kBatch - 1));
+    if (jj < T) {
+        const size_t t = (size_t)(t0 + jj);
+        r.x = __ldg(&a.tiles[t].key0);
+        r.w = __ldg(&a.tiles[t].key0b);
+        r.y = __ldg(&a.tile_pages[t * a.n_pieces]);
+        if (a.n_pieces > 1) r.z = __ldg(&a.tile_pages[t * a.n_pieces + 1]);
+    }
+    return r;
+}
+
+// A CTA's own item and its first batch of records, in the producer's lanes.
+struct FirstItem {
+    int4 raw, rec;
+    __device__ void read(const PrefillArgs& a, int lane) {
+        raw = __ldg(reinterpret_cast<const int4*>(a.items) + blockIdx.x);
+        rec = tile_record(a, raw.y, raw.z, 0, lane);
+    }
+};
+
+// The producer warp, item by item: the query tiles, then the K and V tiles of
+// every key tile into the ring in the order of load_of, two loads at a time:
+// the whole warp waits for both slots, then lanes 0 and 1 arm their barriers
+// and issue their copies together, so that the shared-memory round trips of
+// the two overlap.  The queries of an item wait until the previous item's last
+// QK product is done; its first two loads go out before that wait.  What a
+// tile's copies need, {first key, page of box 0, page of box 1}, is held in
 // registers: lane l has the record of the window's key tile j = l (mod 32),
 // batches of 16 tiles alternating between the lower and the upper half-warp;
 // a batch is read from global memory about ten tiles before its first use and
-// moved into place a few tiles before it.  Boxes past the second (pages of
-// fewer than 64 tokens) take their page from global memory.
+// moved into place a few tiles before it, an item's first batch while the item
+// before it runs.  Boxes past the second (pages of fewer than 64 tokens) take
+// their page from global memory.
 template <int D>
 __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* qmap,
-                                const PrefillArgs& a, const Smem& sm, int g, int pos_lo, int t0,
-                                int T, bool two, bool dual, volatile int* abort_flag, int lane) {
+                                const PrefillArgs& a, const Smem& sm, const FirstItem& start,
+                                volatile int* abort_flag, int lane) {
     using C = PreCfg<D>;
-    if (lane == 0) {
-        prefetch_tmap(pool_map);
-        prefetch_tmap(qmap);
-        const int nq = two ? 2 : 1;  // tile b is loaded only when it holds queries
-        mbar_arrive_expect_tx(sm.bar<D>(C::kBarQ), nq * C::kColBlocks * a.BP * a.G * 128);
-        for (int t = 0; t < nq; ++t)
-            for (int cb = 0; cb < C::kColBlocks; ++cb)
-                tma_load_3d(sm.base + C::kOffQ + t * C::kQBytes + cb * C::kBlockBytes, qmap,
-                            sm.bar<D>(C::kBarQ), cb * 64, g * a.G, pos_lo + t * a.BP);
-    }
     const int br = a.P < 64 ? a.P : 64;  // rows of one TMA box
     const int n_pieces = a.n_pieces;      // <= 16
-    constexpr int kBatch = 16;
-    // {first key of each half, page of box 0, page of box 1} of key tile
-    // tb + lane % 16 (x = key0, y = page 0, z = page 1, w = key0b)
-    auto load_rec = [&](int tb) {
-        int4 r = make_int4(0, -1, -1, kPrefillNoKeys);
-        const int jj = tb + (lane & (kBatch - 1));
-        if (jj < T) {
-            const size_t t = (size_t)(t0 + jj);
-            r.x = __ldg(&a.tiles[t].key0);
-            r.w = __ldg(&a.tiles[t].key0b);
-            r.y = __ldg(&a.tile_pages[t * n_pieces]);
-            if (n_pieces > 1) r.z = __ldg(&a.tile_pages[t * n_pieces + 1]);
+    auto load_rec = [&](int t0, int T, int tb) { return tile_record(a, t0, T, tb, lane); };
+    int4 raw = start.raw, first = start.rec;  // the item, and its first batch of records
+    uint32_t n_items = 1;     // items published (the first at start-up)
+    bool asked = false;       // an answer of the launch hardware is due
+    uint32_t ub = 0;          // loads issued before this item (even)
+    uint32_t n_queries = 0;   // items whose queries were loaded
+    uint32_t n_fix = 0;       // uses of the fix-up barrier
+    uint32_t issued = 0;
+    // Slots are freed by the MMA warp's commits: one for every V tile, which
+    // covers the K tile loaded right after it too, and one for each item's
+    // first K tile; in dual-key mode one for every tile.  Bit i of `own`: the
+    // load i + 1 before the next one has a commit of its own; bit s of `par`:
+    // parity of slot s's next commit.
+    uint32_t own = 0, par = 0;
+    uint32_t slot0 = 0;       // slot of the next load
+    uint32_t tail_u = 0;      // the load that used the fix-up barrier last
+    bool tail_open = false;   // ... and was not handed over on its slot's barrier
+    bool ok = true;
+    auto load_queries = [&](const Item& it) {
+        if (n_queries > 0)
+            ok = mbar_wait(sm.bar<D>(C::kBarQFree), (n_queries - 1) & 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok && lane == 0) {
+            const int nq = it.two ? 2 : 1;  // tile b is loaded only when it holds queries
+            mbar_arrive_expect_tx(sm.bar<D>(C::kBarQ), nq * C::kColBlocks * a.BP * a.G * 128);
+            for (int t = 0; t < nq; ++t)
+                for (int cb = 0; cb < C::kColBlocks; ++cb)
+                    tma_load_3d(sm.base + C::kOffQ + t * C::kQBytes + cb * C::kBlockBytes, qmap,
+                                sm.bar<D>(C::kBarQ), cb * 64, it.g * a.G, it.pos_lo + t * a.BP);
         }
-        return r;
+        if (ok) ++n_queries;
     };
-    int4 rec = make_int4(0, -1, -1, kPrefillNoKeys), pend = rec;
-    if (lane < kBatch) rec = load_rec(0);
-    int fill_b = 1;    // the next batch to read
-    int merge_b = -1;  // the batch read into `pend`, not yet in place
-    const int n_units = 2 * T;
-    int issued = 0;
-    int tail_u = -1;          // the load that used the fix-up barrier
-    bool tail_done = false;   // ... and was handed over on its slot's barrier
-    for (int u0 = 0; u0 < n_units; u0 += 2) {  // n_units is even
-        int j0, kv0, j1, kv1;
-        load_of(u0, T, dual, j0, kv0);
-        load_of(u0 + 1, T, dual, j1, kv1);
-        const int jmax = j0 > j1 ? j0 : j1;
-        if (merge_b >= 0 && jmax + 4 >= kBatch * merge_b) {
-            if ((lane >> 4) == (merge_b & 1)) rec = pend;
-            merge_b = -1;
+    // hands an item (or the end mark) to the other roles
+    auto publish = [&](int4 r) {
+        const int slot = n_items % kItemSlots;
+        if (n_items >= kItemSlots)
+            ok = __all_sync(0xffffffffu,
+                            mbar_wait(sm.bar<D>(C::kBarItemFree + slot),
+                                      (n_items / kItemSlots - 1) & 1, abort_flag));
+        if (ok && lane == 0) {
+            *reinterpret_cast<int4*>(sm.ptr + C::kOffItems + slot * 16) = r;
+            mbar_arrive(sm.bar<D>(C::kBarItem + slot));
         }
-        if (merge_b < 0 && fill_b * kBatch < T && jmax + 10 >= kBatch * fill_b) {
-            if ((lane >> 4) == (fill_b & 1)) pend = load_rec(fill_b * kBatch);
-            merge_b = fill_b++;
+        if (ok) ++n_items;
+    };
+    // The next item: requested when an item's first loads have gone out, taken in
+    // a few loads later, with its first batch of records.
+    int4 next = make_int4(0, 0, -1, 0);
+    auto request = [&]() {
+        if (lane == 0) {
+            mbar_arrive_expect_tx(sm.bar<D>(C::kBarClc), 16);
+            clc_request(sm.base + C::kOffClc, sm.bar<D>(C::kBarClc));
         }
-        const int u = u0 + (lane & 1);  // lanes 0 and 1 issue
-        const int j = (lane & 1) ? j1 : j0, kv = (lane & 1) ? kv1 : kv0;
-        const int key0 = __shfl_sync(0xffffffffu, rec.x, j & 31);
-        const int pg0 = __shfl_sync(0xffffffffu, rec.y, j & 31);
-        const int pg1 = __shfl_sync(0xffffffffu, rec.z, j & 31);
-        const int key0b = __shfl_sync(0xffffffffu, rec.w, j & 31);
-        // rows of the tile inside the sequence (only the last tile has fewer
-        // than 128): the lower half's, then the upper half's
-        const int rows_b = key0b < a.n ? min(64, a.n - key0b) : 0;
-        const int rows = rows_b > 0 ? 64 + rows_b : min(64, a.n - key0);
-        const int slot = u % C::kSlots;
-        const bool vfix = lane < 2 && kv == 1 && rows < kPrefillKeys;
-        // every lane polls both slots' barriers in turn: warp-uniform waits,
-        // so no lane waits at the vote below for two polling lanes
-        bool ok = true;
-        if (u0 >= C::kSlots)
-            ok = mbar_wait(sm.bar<D>(C::kBarEmpty + u0 % C::kSlots), (u0 / C::kSlots - 1) & 1,
-                           abort_flag);
-        if (ok && u0 + 1 >= C::kSlots)
-            ok = mbar_wait(sm.bar<D>(C::kBarEmpty + (u0 + 1) % C::kSlots),
-                           ((u0 + 1) / C::kSlots - 1) & 1, abort_flag);
-        // both slots free, or neither load is issued
-        if (!__all_sync(0xffffffffu, ok)) {
-            if (lane == 0) {
-                set_error(a.err, kErrTimeout);
-                *abort_flag = 1;
+        asked = true;
+    };
+    auto take_next = [&](uint32_t parity) {
+        ok = __all_sync(0xffffffffu, mbar_wait(sm.bar<D>(C::kBarClc), parity, abort_flag));
+        if (!ok) return;
+        asked = false;
+        const int cta = clc_answer(sm.base + C::kOffClc);
+        next = make_int4(0, 0, -1, 0);
+        if (cta >= 0 && cta < a.n_items)
+            next = __ldg(reinterpret_cast<const int4*>(a.items) + cta);
+        first = load_rec(next.y, next.z, 0);
+        // the answer's words are read before the next request overwrites them
+        fence_proxy_async_smem();
+        __syncwarp();
+    };
+    while (ok && raw.z >= 0) {
+        const Item it = make_item(a, raw);
+        const uint32_t clc_parity = (n_items - 1) & 1;
+        int4 rec = first, pend = first;
+        const int T = it.T;
+        const int n_units = 2 * T;
+        const int take_at = n_units > 10 ? 8 : n_units - 2;
+        const bool late_queries = ub > 0;
+        if (T > 0 && !late_queries) load_queries(it);
+        if (T == 0) {
+            request();
+            take_next(clc_parity);
+        }
+        int fill_b = 1;    // the next batch to read
+        int merge_b = -1;  // the batch read into `pend`, not yet in place
+        // only the sequence's last key tile has rows past its end
+        const int j_tail = it.t0 + T == a.n_tiles ? T - 1 : T;
+        for (int u0 = 0; ok && u0 < n_units; u0 += 2) {  // n_units is even
+            int j0, kv0, j1, kv1;
+            load_of(u0, T, it.dual, j0, kv0);
+            load_of(u0 + 1, T, it.dual, j1, kv1);
+            const int jmax = j0 > j1 ? j0 : j1;
+            if (merge_b >= 0 && jmax + 4 >= kBatch * merge_b) {
+                if ((lane >> 4) == (merge_b & 1)) rec = pend;
+                merge_b = -1;
             }
-            break;
-        }
-        if (lane < 2) {
-            const int nv = (rows + br - 1) / br;  // boxes inside the sequence (a prefix)
-            const uint32_t fb = vfix ? sm.bar<D>(C::kBarVfix) : sm.bar<D>(C::kBarFull + slot);
-            mbar_arrive_expect_tx(fb, (uint32_t)nv * br * 128 * C::kColBlocks);
+            if (merge_b < 0 && fill_b * kBatch < T && jmax + 10 >= kBatch * fill_b) {
+                if ((lane >> 4) == (fill_b & 1)) pend = load_rec(it.t0, T, fill_b * kBatch);
+                merge_b = fill_b++;
+            }
+            const uint32_t U0 = ub + u0;
+            const uint32_t slot1 = slot0 + 1 == C::kSlots ? 0 : slot0 + 1;
+            const int j = (lane & 1) ? j1 : j0, kv = (lane & 1) ? kv1 : kv0;
+            const int key0 = __shfl_sync(0xffffffffu, rec.x, j & 31);
+            const int pg0 = __shfl_sync(0xffffffffu, rec.y, j & 31);
+            const int pg1 = __shfl_sync(0xffffffffu, rec.z, j & 31);
+            const int key0b = __shfl_sync(0xffffffffu, rec.w, j & 31);
+            const int slot = (lane & 1) ? slot1 : slot0;  // lanes 0 and 1 issue
             const uint32_t dst = sm.base + C::kOffRing + slot * C::kSlotBytes;
-            const int head_row = (kv ? a.Hkv + g : g) * a.P;
-#pragma unroll 1
-            for (int i = 0; i < nv; ++i) {
-                int32_t page =
-                    i == 0 ? pg0
-                           : (i == 1 ? pg1
-                                     : __ldg(&a.tile_pages[(size_t)(t0 + j) * n_pieces + i]));
-                if ((uint32_t)page >= (uint32_t)a.num_pages) {
-                    // a page outside the pool: flagged; the box is read from
-                    // page 0 so that the barrier's byte count still completes
-                    set_error(a.err, kErrBounds);
-                    page = 0;
-                }
-                const int half = n_pieces / 2;
-                const int key = i < half ? key0 + i * br : key0b + (i - half) * br;
+            const int head_row = (kv ? a.Hkv + it.g : it.g) * a.P;
+            // every lane polls the slots' barriers in turn: warp-uniform waits,
+            // so no lane waits at the vote below for two polling lanes
+            if (U0 >= C::kSlots && ((own >> (C::kSlots - 1)) & 1u)) {
+                ok = mbar_wait(sm.bar<D>(C::kBarEmpty + slot0), (par >> slot0) & 1u, abort_flag);
+                par ^= 1u << slot0;
+            }
+            if (U0 + 1 >= C::kSlots && ((own >> (C::kSlots - 2)) & 1u)) {
+                if (ok)
+                    ok = mbar_wait(sm.bar<D>(C::kBarEmpty + slot1), (par >> slot1) & 1u, abort_flag);
+                par ^= 1u << slot1;
+            }
+            own = own << 2 | (it.dual || j0 == 0 ? 3u : 1u);  // K_j0, V_j1 but in dual-key mode
+            // both slots free, or neither load is issued
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            auto checked = [&](int32_t page) {
+                if ((uint32_t)page < (uint32_t)a.num_pages) return page;
+                // a page outside the pool: flagged; the box is read from page 0
+                // so that the barrier's byte count still completes
+                set_error(a.err, kErrBounds);
+                return 0;
+            };
+            auto load_box = [&](uint32_t bar, int i, int key, int32_t page) {
+                const int row = head_row + (key & (a.P - 1));  // P is a power of two
 #pragma unroll
                 for (int cb = 0; cb < C::kColBlocks; ++cb)
-                    tma_load_4d(dst + cb * C::kBlockBytes + i * br * 128, pool_map, fb, cb * 64,
-                                head_row + key % a.P, page, a.layer);
-            }
-        }
-        issued = u0 + 2;
-        const uint32_t fix = __ballot_sync(0xffffffffu, vfix);
-        if (fix) {
-            // V of the last key tile: its rows past the sequence's end hold
-            // stale or never-written data.  Their weights are zero, but 0 * NaN
-            // is not, so zero those rows before the MMAs read the slot.
-            const int src = __ffs(fix) - 1;
-            const int fslot = __shfl_sync(0xffffffffu, slot, src);
-            const int frows = __shfl_sync(0xffffffffu, rows, src);
-            tail_u = u0 + src;
-            if (lane == 0) ok = mbar_wait(sm.bar<D>(C::kBarVfix), 0, abort_flag);
-            if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) {
-                if (lane == 0) {
-                    set_error(a.err, kErrTimeout);
-                    *abort_flag = 1;
+                    tma_load_4d(dst + cb * C::kBlockBytes + i * br * 128, pool_map, bar, cb * 64, row,
+                                page, a.layer);
+            };
+            if (n_pieces == 2 && jmax < j_tail) {
+                // two whole boxes of 64 rows, as almost every tile has
+                if (lane < 2) {
+                    const uint32_t fb = sm.bar<D>(C::kBarFull + slot);
+                    mbar_arrive_expect_tx(fb, C::kSlotBytes);
+                    load_box(fb, 0, key0, checked(pg0));
+                    load_box(fb, 1, key0b, checked(pg1));
                 }
-                break;
+            } else {
+                // rows of the tile inside the sequence: the lower half's, then
+                // the upper half's
+                const int rows_b = key0b < a.n ? min(64, a.n - key0b) : 0;
+                const int rows = rows_b > 0 ? 64 + rows_b : min(64, a.n - key0);
+                const bool vfix = lane < 2 && kv == 1 && rows < kPrefillKeys;
+                if (lane < 2) {
+                    const int nv = (rows + br - 1) / br;  // boxes inside the sequence (a prefix)
+                    const uint32_t fb = vfix ? sm.bar<D>(C::kBarVfix) : sm.bar<D>(C::kBarFull + slot);
+                    mbar_arrive_expect_tx(fb, (uint32_t)nv * br * 128 * C::kColBlocks);
+                    const int half = n_pieces / 2;
+#pragma unroll 1
+                    for (int i = 0; i < nv; ++i) {
+                        const int32_t page =
+                            i == 0
+                                ? pg0
+                                : (i == 1 ? pg1
+                                          : __ldg(&a.tile_pages[(size_t)(it.t0 + j) * n_pieces + i]));
+                        load_box(fb, i, i < half ? key0 + i * br : key0b + (i - half) * br,
+                                 checked(page));
+                    }
+                }
+                const uint32_t fix = __ballot_sync(0xffffffffu, vfix);
+                if (fix) {
+                    // V of the last key tile: its rows past the sequence's end hold
+                    // stale or never-written data.  Their weights are zero, but
+                    // 0 * NaN is not, so zero those rows before the MMAs read the slot.
+                    const int src = __ffs(fix) - 1;
+                    const int fslot = __shfl_sync(0xffffffffu, slot, src);
+                    const int r0 = __shfl_sync(0xffffffffu, rows, src);  // 1 .. 127
+                    tail_u = U0 + src;
+                    tail_open = true;
+                    issued = U0 + 2;
+                    if (lane == 0) ok = mbar_wait(sm.bar<D>(C::kBarVfix), n_fix & 1, abort_flag);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0);
+                    if (!ok) break;
+                    ++n_fix;
+                    const int chunks = (kPrefillKeys - r0) * 8;
+                    uint8_t* vsp = sm.ptr + C::kOffRing + fslot * C::kSlotBytes;
+                    for (int cb = 0; cb < C::kColBlocks; ++cb)
+                        for (int c = lane; c < chunks; c += 32)
+                            *reinterpret_cast<uint4*>(vsp + cb * C::kBlockBytes +
+                                                      (r0 + (c >> 3)) * 128 + (c & 7) * 16) =
+                                make_uint4(0, 0, 0, 0);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(sm.bar<D>(C::kBarFull + fslot));
+                    tail_open = false;
+                }
             }
-            const int r0 = frows;  // 1 .. 127
-            const int chunks = (kPrefillKeys - r0) * 8;
-            uint8_t* vsp = sm.ptr + C::kOffRing + fslot * C::kSlotBytes;
-            for (int cb = 0; cb < C::kColBlocks; ++cb)
-                for (int c = lane; c < chunks; c += 32)
-                    *reinterpret_cast<uint4*>(vsp + cb * C::kBlockBytes + (r0 + (c >> 3)) * 128 +
-                                              (c & 7) * 16) = make_uint4(0, 0, 0, 0);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(sm.bar<D>(C::kBarFull + fslot));
-            tail_done = true;
+            issued = U0 + 2;
+            slot0 = slot1 + 1 == C::kSlots ? 0 : slot1 + 1;
+            if (u0 == 0) {
+                request();
+                if (late_queries) load_queries(it);
+            }
+            if (ok && u0 == take_at) take_next(clc_parity);
         }
+        ub += n_units;
+        raw = next;
+        if (ok) publish(raw);  // an item, or the end mark
+    }
+    if (!ok && lane == 0) {
+        if (!*abort_flag) set_error(a.err, kErrTimeout);
+        *abort_flag = 1;
     }
     // Drain: every copy this CTA issued lands before the CTA exits (immediate
     // unless a consumer gave up early).
     if (lane == 0) {
-        mbar_wait(sm.bar<D>(C::kBarQ), 0);
-        for (int u = issued > C::kSlots ? issued - C::kSlots : 0; u < issued; ++u) {
-            if (u == tail_u && !tail_done) mbar_wait(sm.bar<D>(C::kBarVfix), 0);
+        if (asked) mbar_wait(sm.bar<D>(C::kBarClc), (n_items - 1) & 1);
+        if (n_queries > 0) mbar_wait(sm.bar<D>(C::kBarQ), (n_queries - 1) & 1);
+        for (uint32_t u = issued > C::kSlots ? issued - C::kSlots : 0; u < issued; ++u) {
+            if (u == tail_u && tail_open) mbar_wait(sm.bar<D>(C::kBarVfix), n_fix & 1);
             else mbar_wait(sm.bar<D>(C::kBarFull + u % C::kSlots), (u / C::kSlots) & 1);
         }
     }
 }
 
+// Descriptors of a CTA's operands: the two query tiles, and the ring's slot 0
+// as a K tile (K-major) and as a V tile (MN-major).  Slot s is s *
+// kSlotBytes / 16 further in the address field.
+struct MmaDesc {
+    uint32_t q[2], k, v;      // low words
+    uint32_t k_hi, v_hi;      // high words (the queries' is the K tile's)
+    uint32_t tmem;
+};
+template <int D>
+__device__ __forceinline__ MmaDesc mma_desc(const Smem& sm, uint32_t tmem) {
+    using C = PreCfg<D>;
+    static_assert(C::kBlockBytes == 16384, "the K-major steps' block stride");
+    const uint64_t q = smem_desc_sw128(sm.base + C::kOffQ, 16, 1024);
+    const uint64_t k = smem_desc_sw128(sm.base + C::kOffRing, 16, 1024);
+    const uint64_t v = smem_desc_sw128(sm.base + C::kOffRing, C::kBlockBytes, 1024);
+    MmaDesc d;
+    d.q[0] = (uint32_t)q;
+    d.q[1] = (uint32_t)q + (C::kQBytes >> 4);
+    d.k = (uint32_t)k;
+    d.v = (uint32_t)v;
+    d.k_hi = (uint32_t)(k >> 32);
+    d.v_hi = (uint32_t)(v >> 32);
+    d.tmem = tmem;
+    return d;
+}
+
 // S_t = Q_q K^T for the K tile in `slot`, into TMEM columns 128 t (q = t
 // except in dual-key mode, where both tiles use query tile 0).
 template <int D>
-__device__ __forceinline__ void issue_qk(const Smem& sm, uint32_t tmem, int t, int slot, int q = -1) {
+__device__ __forceinline__ void issue_qk(const MmaDesc& d, int t, int q, uint32_t slot) {
     using C = PreCfg<D>;
-    const uint32_t qa = sm.base + C::kOffQ + (q < 0 ? t : q) * C::kQBytes;
-    const uint32_t ka = sm.base + C::kOffRing + slot * C::kSlotBytes;
-    const uint32_t dt = tmem + C::kColS + (uint32_t)t * kPrefillKeys;
-    // descriptors built once and stepped per K step: the address field holds
-    // address / 16 in 14 bits and every address here is below 2^18 bytes, so
-    // adding offset / 16 cannot carry out of it
-    const uint64_t qd = smem_desc_sw128(qa, 16, 1024), kd = smem_desc_sw128(ka, 16, 1024);
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
-        const uint32_t off = ((ks >> 2) * C::kBlockBytes + (ks & 3) * 32) >> 4;
-        mma_bf16_ss(dt, qd + off, kd + off, C::kIdescQK, ks > 0);
-    }
+    mma_bf16_ss_steps<D / 16>(d.tmem + C::kColS + (uint32_t)t * kPrefillKeys, d.q[q],
+                              d.k + slot * (C::kSlotBytes >> 4), d.k_hi, C::kIdescQK);
 }
 
 // O_t += P_t V for the V tile in `slot`; P_t from TMEM over the first half of S_t.
 template <int D>
-__device__ __forceinline__ void issue_pv(const Smem& sm, uint32_t tmem, int t, int slot,
-                                         bool first) {
+__device__ __forceinline__ void issue_pv(const MmaDesc& d, int t, uint32_t slot, bool first) {
     using C = PreCfg<D>;
-    const uint32_t pa = tmem + C::kColS + (uint32_t)t * kPrefillKeys;
-    const uint32_t va = sm.base + C::kOffRing + slot * C::kSlotBytes;
-    const uint64_t vd = smem_desc_sw128(va, C::kBlockBytes, 1024);
-#pragma unroll
-    for (int ks = 0; ks < kPrefillKeys / 16; ++ks)
-        mma_bf16_ts(tmem + C::kColO + (uint32_t)t * 128, pa + ks * 8, vd + (uint64_t)(ks * 128),
-                    C::kIdescPV, (!first || ks > 0) ? 1u : 0u);
+    static_assert(kPrefillKeys == 128, "8 steps of 16 keys");
+    mma_bf16_ts_steps8(d.tmem + C::kColO + (uint32_t)t * 128,
+                       d.tmem + C::kColS + (uint32_t)t * kPrefillKeys,
+                       d.v + slot * (C::kSlotBytes >> 4), d.v_hi, C::kIdescPV, first ? 0u : 1u);
 }
 
+// Phases of the barriers the MMA warp waits on, running on from item to item.
+struct MmaPhase {
+    uint32_t ub;    // loads of the items before (K_j, V_j: load_of)
+    uint32_t slot;  // ub mod kSlots
+    uint32_t p;     // bit t: parity of the next P_t hand-off
+    uint32_t q;     // items whose queries were used
+};
+
+// The lane that issues the MMAs is the busiest thread of the kernel: whatever
+// it does between two products, the tensor core's short queue drains.  So it
+// waits for P_t alone: a softmax warp of tile a hands over P only when V_j and
+// K_{j+1} have landed too, and one commit after the second PV frees V_j and,
+// with it, the K tile used by the QK products issued just before.  (With its
+// own waits for both tiles and a commit for each slot the lane needed 3,434
+// cycles per key tile for products of 2,650, and was never waiting for P.)
+// In dual-key mode memory is the bound, not this lane: it waits for each tile
+// by itself and frees each slot at once.
+//
 // Dual-key mode (every query of the CTA tile fits in tile a): both tiles
 // hold tile a's queries; tile a takes key tiles 0, 2, 4, ... and tile b the
 // odd ones, and the two results are merged at the end.  Key tile j's PV and
 // the QK of key tile j + 2 (into the same S columns) are issued in the order
 // of the loads, each as soon as its tile has landed.
 template <int D>
-__device__ bool prefill_mma_dual(const Smem& sm, uint32_t tmem, int T, volatile int* abort_flag) {
+__device__ bool prefill_mma_dual(const Smem& sm, const MmaDesc& d, int T, MmaPhase& ph,
+                                 volatile int* abort_flag) {
     using C = PreCfg<D>;
-    bool ok = true;
-    for (int t = 0; t < 2 && ok; ++t) {
-        // S_t = Q_a K_t
-        const int u = dual_load_k(t), slot = u % C::kSlots;
-        if (!(ok = mbar_wait(sm.bar<D>(C::kBarFull + slot), (u / C::kSlots) & 1, abort_flag))) break;
-        issue_qk<D>(sm, tmem, t, slot, 0);
-        mma_commit(sm.bar<D>(C::kBarS + t));
+    // the tiles are used in the order of their loads: K_0, K_1, V_0, K_2, V_1, ...
+    uint32_t slot = ph.slot, full = (ph.ub / C::kSlots) & 1;
+    auto landed = [&]() { return mbar_wait(sm.bar<D>(C::kBarFull + slot), full, abort_flag); };
+    auto used = [&]() {
         mma_commit(sm.bar<D>(C::kBarEmpty + slot));
+        if (++slot == C::kSlots) {
+            slot = 0;
+            full ^= 1;
+        }
+    };
+    for (int t = 0; t < 2; ++t) {
+        // S_t = Q_a K_t
+        if (!landed()) return false;
+        issue_qk<D>(d, t, 0, slot);
+        mma_commit(sm.bar<D>(C::kBarS + t));
+        used();
     }
-    for (int j = 0; ok && j < T; ++j) {
-        const int t = j & 1, i = j >> 1;
-        const int uv = dual_load_v(j, T), vslot = uv % C::kSlots;
-        if (!(ok = mbar_wait(sm.bar<D>(C::kBarFull + vslot), (uv / C::kSlots) & 1, abort_flag)))
-            break;
-        if (!(ok = mbar_wait(sm.bar<D>(C::kBarP + t), i & 1, abort_flag))) break;
+    if (T == 2) mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
+    for (int j = 0; j < T; ++j) {
+        const int t = j & 1;
+        if (!landed()) return false;
+        if (!mbar_wait(sm.bar<D>(C::kBarP + t), (ph.p >> t) & 1, abort_flag)) return false;
+        ph.p ^= 1u << t;
         tc_fence_after();
-        issue_pv<D>(sm, tmem, t, vslot, i == 0);
-        mma_commit(sm.bar<D>(C::kBarEmpty + vslot));
+        issue_pv<D>(d, t, slot, j < 2);
+        used();
         if (j + 2 >= T) {  // the last key tile of tile t
             mma_commit(sm.bar<D>(C::kBarO + t));
             continue;
         }
-        const int uk = dual_load_k(j + 2), kslot = uk % C::kSlots;
-        if (!(ok = mbar_wait(sm.bar<D>(C::kBarFull + kslot), (uk / C::kSlots) & 1, abort_flag)))
-            break;
-        issue_qk<D>(sm, tmem, t, kslot, 0);
+        if (!landed()) return false;
+        issue_qk<D>(d, t, 0, slot);
         mma_commit(sm.bar<D>(C::kBarS + t));
-        mma_commit(sm.bar<D>(C::kBarEmpty + kslot));
+        used();
+        if (j + 3 == T) mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
     }
-    return ok;
+    ph.slot = slot;
+    return true;
 }
 
-// `two`: tile b holds query rows (false for short query blocks, whose rows
-// all fit in tile a; tile b's products are then skipped, or, with `dual`, it
-// takes every other key tile).
-template <int D>
-__device__ void prefill_mma(const PrefillArgs& a, const Smem& sm, uint32_t tmem, int T, bool two,
-                            bool dual, volatile int* abort_flag) {
+// One step of the two-tile path: O_t += P_t V_j, then S_t for the next key tile,
+// for tile a and then tile b.
+template <int D, bool kFirst, bool kMore>
+__device__ __forceinline__ bool prefill_mma_step(const Smem& sm, const MmaDesc& d, uint32_t vslot,
+                                                 uint32_t kslot, uint32_t pa, uint32_t pb,
+                                                 const volatile int* abort_flag) {
     using C = PreCfg<D>;
-    bool ok = mbar_wait(sm.bar<D>(C::kBarQ), 0, abort_flag);
-    bool any = false;
-    if (ok && T > 0 && dual) {
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        if (!mbar_wait(sm.bar<D>(C::kBarP + t), t ? pb : pa, abort_flag)) return false;
         tc_fence_after();
+        issue_pv<D>(d, t, vslot, kFirst);
+        if (kMore) issue_qk<D>(d, t, t, kslot);
+        mma_commit(sm.bar<D>(kMore ? C::kBarS + t : C::kBarO + t));
+    }
+    mma_commit(sm.bar<D>(C::kBarEmpty + vslot));  // V_j, and K_{j+1} with it
+    return true;
+}
+
+// `two`: tile b holds query rows (false for an item of one key tile whose rows
+// all fit in tile a; tile b's products are then skipped).
+template <int D>
+__device__ bool prefill_mma_item(const Smem& sm, const MmaDesc& d, int T, bool two, MmaPhase& ph,
+                                 volatile int* abort_flag) {
+    using C = PreCfg<D>;
+    auto after = [](uint32_t slot) { return slot + 1 == C::kSlots ? 0u : slot + 1; };
+    uint32_t slot = ph.slot;
+    if (!mbar_wait(sm.bar<D>(C::kBarFull + slot), (ph.ub / C::kSlots) & 1, abort_flag)) return false;
+    issue_qk<D>(d, 0, 0, slot);
+    mma_commit(sm.bar<D>(C::kBarS + 0));
+    if (two) {
+        issue_qk<D>(d, 1, 1, slot);
+        mma_commit(sm.bar<D>(C::kBarS + 1));
+    }
+    mma_commit(sm.bar<D>(C::kBarEmpty + slot));
+    uint32_t vslot = after(slot), kslot = after(vslot);
+    if (!two) {
+        mma_commit(sm.bar<D>(C::kBarQFree));
+        if (!mbar_wait(sm.bar<D>(C::kBarP + 0), ph.p & 1, abort_flag)) return false;
+        tc_fence_after();
+        issue_pv<D>(d, 0, vslot, true);
+        mma_commit(sm.bar<D>(C::kBarO + 0));
+        mma_commit(sm.bar<D>(C::kBarEmpty + vslot));
+        ph.p ^= 1u;
+        ph.slot = kslot;
+        return true;
+    }
+    uint32_t pa = ph.p & 1, pb = (ph.p >> 1) & 1;
+    if (T == 1) {
+        mma_commit(sm.bar<D>(C::kBarQFree));
+        if (!prefill_mma_step<D, true, false>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
+    } else {
+        if (!prefill_mma_step<D, true, true>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
+        for (int j = 1; j + 1 < T; ++j) {
+            vslot = after(kslot);
+            kslot = after(vslot);
+            pa ^= 1;
+            pb ^= 1;
+            if (!prefill_mma_step<D, false, true>(sm, d, vslot, kslot, pa, pb, abort_flag))
+                return false;
+        }
+        mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
+        vslot = after(kslot);
+        kslot = after(vslot);
+        if (!prefill_mma_step<D, false, false>(sm, d, vslot, kslot, pa ^ 1, pb ^ 1, abort_flag))
+            return false;
+    }
+    ph.p ^= (T & 1) ? 3u : 0u;
+    ph.slot = kslot;
+    return true;
+}
+
+// The MMA-issuing lane, item by item.  The next item's first S may be issued
+// while the softmax warps still write out this one's O: S has columns of its
+// own, and the first PV, which overwrites O, waits for a P that each softmax
+// thread hands over only after it has read its O.
+template <int D>
+__device__ void prefill_mma(const PrefillArgs& a, const Smem& sm, uint32_t tmem,
+                            volatile int* abort_flag) {
+    using C = PreCfg<D>;
+    MmaPhase ph = {0, 0, 0, 0};
+    const MmaDesc d = mma_desc<D>(sm, tmem);
+    bool ok = true, any = false;
+    for (uint32_t k = 0;; ++k) {
+        if (!(ok = item_wait<D>(sm, k, abort_flag))) break;
+        const int4 raw = item_read<D>(sm, k);
+        item_free<D>(sm, k);
+        if (raw.z < 0) break;
+        if (raw.z == 0) continue;
+        const Item it = make_item(a, raw);
+        if (!(ok = mbar_wait(sm.bar<D>(C::kBarQ), ph.q & 1, abort_flag))) break;
+        tc_fence_after();
+        ++ph.q;
         any = true;
-        ok = prefill_mma_dual<D>(sm, tmem, T, abort_flag);
-    } else if (ok && T > 0) {
-        tc_fence_after();
-        const int k0 = 0;
-        ok = mbar_wait(sm.bar<D>(C::kBarFull + k0), 0, abort_flag);
-        if (ok) {
-            any = true;
-            issue_qk<D>(sm, tmem, 0, k0);
-            mma_commit(sm.bar<D>(C::kBarS + 0));
-            if (two) {
-                issue_qk<D>(sm, tmem, 1, k0);
-                mma_commit(sm.bar<D>(C::kBarS + 1));
-            }
-            mma_commit(sm.bar<D>(C::kBarEmpty + k0));
-        }
-        for (int j = 0; ok && j < T; ++j) {
-            const int uv = 2 * j + 1, vslot = uv % C::kSlots;
-            const int uk = 2 * j + 2, kslot = uk % C::kSlots;
-            const bool more = j + 1 < T;
-            // V_j and K_{j+1} have normally landed long ago; checking them before
-            // P_a keeps these barrier reads off the path from P_a to the MMAs
-            if (!(ok = mbar_wait(sm.bar<D>(C::kBarFull + vslot), (uv / C::kSlots) & 1, abort_flag)))
-                break;
-            if (more && !(ok = mbar_wait(sm.bar<D>(C::kBarFull + kslot), (uk / C::kSlots) & 1,
-                                         abort_flag)))
-                break;
-            // tile a: O_a += P_a V_j, then S_a for the next key tile
-            if (!(ok = mbar_wait(sm.bar<D>(C::kBarP + 0), j & 1, abort_flag))) break;
-            tc_fence_after();
-            issue_pv<D>(sm, tmem, 0, vslot, j == 0);
-            if (!more) mma_commit(sm.bar<D>(C::kBarO + 0));
-            if (!two) mma_commit(sm.bar<D>(C::kBarEmpty + vslot));
-            if (more) {
-                issue_qk<D>(sm, tmem, 0, kslot);
-                mma_commit(sm.bar<D>(C::kBarS + 0));
-                if (!two) mma_commit(sm.bar<D>(C::kBarEmpty + kslot));
-            }
-            if (!two) continue;
-            // tile b
-            if (!(ok = mbar_wait(sm.bar<D>(C::kBarP + 1), j & 1, abort_flag))) break;
-            tc_fence_after();
-            issue_pv<D>(sm, tmem, 1, vslot, j == 0);
-            mma_commit(sm.bar<D>(C::kBarEmpty + vslot));
-            if (!more) mma_commit(sm.bar<D>(C::kBarO + 1));
-            if (more) {
-                issue_qk<D>(sm, tmem, 1, kslot);
-                mma_commit(sm.bar<D>(C::kBarS + 1));
-                mma_commit(sm.bar<D>(C::kBarEmpty + kslot));
-            }
-        }
+        ok = it.dual ? prefill_mma_dual<D>(sm, d, it.T, ph, abort_flag)
+                     : prefill_mma_item<D>(sm, d, it.T, it.two, ph, abort_flag);
+        if (!ok) break;
+        ph.ub += 2 * it.T;
     }
     if (!ok) {
         set_error(a.err, kErrTimeout);
@@ -476,232 +746,22 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const v
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
 }
 
-// Softmax warpgroup of query tile t (one row per thread) and its epilogue.
+// Normalises and writes one row of O_t (with tile b's part in dual-key mode) to
+// the outputs, or to the item's partial result.
 template <int D>
-__device__ void prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t tmem, int t, int g,
-                                int pos_lo, int t0, int T_cta, bool dual, volatile int* abort_flag,
-                                int warp, int lane) {
+__device__ __forceinline__ void prefill_write(const PrefillArgs& a, const Item& it, uint32_t tl,
+                                              uint32_t col_o, int t, int row, bool valid,
+                                              float m_run, float l, float wa, float wb) {
     using C = PreCfg<D>;
-    const int wq = warp & 3;
-    const int row = wq * 32 + lane;
-    // dual-key mode: both tiles hold tile a's queries, tile t takes key tiles
-    // t, t + 2, t + 4, ... of the CTA's range
-    const int qi = pos_lo + (dual ? 0 : t) * a.BP + row / a.G;
-    const bool valid = row < a.BP * a.G && qi < a.n_q;
-    const int T = dual ? (T_cta + 1 - t) / 2 : T_cta;
-    const int kstep = dual ? 2 : 1, kfirst = dual ? t : 0;
-    float* xchg = reinterpret_cast<float*>(sm.ptr + C::kOffXchg);
-    // A warp none of whose rows is a query only keeps the barrier count: it
-    // waits for each S and signals its P without computing (its rows of P
-    // and O are never read back).
-    if (!__any_sync(0xffffffffu, valid)) {
-        bool wok = true;
-        for (int j = 0; j < T; ++j) {
-            if (wok) wok = warp_wait(sm.bar<D>(C::kBarS + t), j & 1, abort_flag);
-            tc_fence_before();
-            mbar_arrive(sm.bar<D>(C::kBarP + t));
-        }
-        if (!wok && lane == 0) {
-            set_error(a.err, kErrTimeout);
-            *abort_flag = 1;
-        }
-        // the merge of the two tiles' results meets all 256 threads, whatever happened
-        if (dual) named_bar_sync(3, 256);
-        return;
-    }
-    const int p_row = a.n - a.n_q + qi;
-    const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16);
-    const uint32_t col_s = C::kColS + (uint32_t)t * kPrefillKeys;
-    const uint32_t col_o = C::kColO + (uint32_t)t * 128;
-    const float sc = a.scale_log2;  // > 0 (the host raises a zero scale to a tiny one)
-    float m_run = -INFINITY, l = 0.f;
-    bool ok = true;
-    int4 n0 = make_int4(0, 0, 0, 0), n1 = n0;
-    if (T > 0) {
-        const int4* tp = reinterpret_cast<const int4*>(a.tiles + t0 + kfirst);
-        n0 = __ldg(tp);
-        n1 = __ldg(tp + 1);
-    }
-    for (int j = 0; j < T; ++j) {
-        // this tile's record; the next one is fetched while this tile is worked on
-        const int4 w0 = n0, w1 = n1;
-        if (j + 1 < T) {
-            const int4* tp =
-                reinterpret_cast<const int4*>(a.tiles + t0 + kfirst + (j + 1) * kstep);
-            n0 = __ldg(tp);
-            n1 = __ldg(tp + 1);
-        }
-        const int key0 = w0.x;
-        const uint32_t vis[4] = {(uint32_t)w0.z, (uint32_t)w0.w, (uint32_t)w1.x, (uint32_t)w1.y};
-        ok = warp_wait(sm.bar<D>(C::kBarS + t), j & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        // Raw logits q.k (the scale is applied inside the exponent; it is > 0),
-        // taken 64 columns at a time to keep registers low: one pass for the
-        // row maximum, one for the weights.
-        // keys key0 + c (lower half) and key0b + c (upper half) with c <= lim,
-        // c <= limb are causal
-        const int lim = p_row - key0, limb = p_row - w1.z;
-        const bool unmasked = valid && (w0.y & kPrefillTileFull) && lim >= 63 && limb >= 63;
-        // Weights 2^(s * scale - m) with the running maximum m, two arguments
-        // at a time with a packed FMA, rounded to bf16 into wt (32 words per
-        // 64 keys).  The normaliser sums the same rounded weights that the PV
-        // product takes (eight fp32 chains), so the output is a convex
-        // combination of the V rows whatever the rounding.
-        // Nothing is stored: S stays intact until the weights are accepted.
-        const uint64_t sc2 = f2pack(sc, sc);
-        uint32_t wt[2][32];
-        auto weights = [&](float m, float& tile_sum) {
-            const float nmu = m == -INFINITY ? 0.f : -m;
-            const uint64_t nmu2 = f2pack(nmu, nmu);
-            float ls[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                uint32_t x[64];
-                tmem_ld32(tl + col_s + 64 * hh, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                tmem_ld32(tl + col_s + 64 * hh + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-                tmem_wait_ld();
-                if (!unmasked) {
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        const int ww = 2 * hh + w;
-                        const uint32_t mw =
-                            valid ? (vis[ww] & low_bits_through((ww < 2 ? lim : limb) - 32 * (ww & 1))) : 0u;
-#pragma unroll
-                        for (int c = 0; c < 32; ++c)
-                            if (!((mw >> c) & 1u)) x[32 * w + c] = 0xff800000u;  // -inf
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const float x0 = __uint_as_float(x[2 * i]), x1 = __uint_as_float(x[2 * i + 1]);
-                    float a0, a1;
-                    f2unpack(ffma2(f2pack(x0, x1), sc2, nmu2), a0, a1);
-                    const __nv_bfloat162 hb = __floats2bfloat162_rn(ex2_ftz(a0), ex2_ftz(a1));
-                    wt[hh][i] = *reinterpret_cast<const uint32_t*>(&hb);
-                    add_bf16x2_f32(wt[hh][i], ls[2 * (i & 3)], ls[2 * (i & 3) + 1]);
-                }
-            }
-            tile_sum = ((ls[0] + ls[1]) + (ls[2] + ls[3])) + ((ls[4] + ls[5]) + (ls[6] + ls[7]));
-        };
-        // The maximum is raised lazily, so most tiles keep it: take the
-        // weights with the current maximum and accept them when no row's sum
-        // exceeds 2^16, which bounds every weight; no maximum is needed for
-        // that.  Otherwise (or when a row has seen no key yet) find the tile's
-        // maximum and redo the tile with it wherever it exceeds the running
-        // one by more than 2^8.
-        float mt = -INFINITY, tsum = 0.f;
-        bool done = false;
-        if (__all_sync(0xffffffffu, m_run != -INFINITY)) {
-            weights(m_run, tsum);
-            done = !__any_sync(0xffffffffu, tsum > 65536.f);
-        }
-        if (!done) {
-            // row maximum: three-input max over four independent chains
-            float mx[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) mx[c] = -INFINITY;
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                uint32_t x[64];
-                tmem_ld32(tl + col_s + 64 * hh, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                tmem_ld32(tl + col_s + 64 * hh + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-                tmem_wait_ld();
-                if (!unmasked) {
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        const int ww = 2 * hh + w;
-                        const uint32_t mw =
-                            valid ? (vis[ww] & low_bits_through((ww < 2 ? lim : limb) - 32 * (ww & 1))) : 0u;
-#pragma unroll
-                        for (int c = 0; c < 32; ++c)
-                            if (!((mw >> c) & 1u)) x[32 * w + c] = 0xff800000u;  // -inf
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 64; c += 8) {
-                    mx[0] = fmax3(mx[0], __uint_as_float(x[c]), __uint_as_float(x[c + 1]));
-                    mx[1] = fmax3(mx[1], __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]));
-                    mx[2] = fmax3(mx[2], __uint_as_float(x[c + 4]), __uint_as_float(x[c + 5]));
-                    mx[3] = fmax3(mx[3], __uint_as_float(x[c + 6]), __uint_as_float(x[c + 7]));
-                }
-            }
-            mt = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]) * sc;
-        }
-        if (done) {
-            l += tsum;
-        } else {
-            const bool need = mt > m_run + 8.f;
-            float alpha = 1.f;
-            if (need) {
-                alpha = exp2f(m_run - mt);
-                m_run = mt;
-                l *= alpha;
-            }
-            if (j > 0 && __any_sync(0xffffffffu, need)) {
-                // O_t holds the products up to key tile j - 1 (complete: S_t(j)
-                // was issued after them): rescale it in place
-#pragma unroll
-                for (int c = 0; c < D / 32; ++c) {
-                    uint32_t o[32];
-                    tmem_ld32(tl + col_o + c * 32, o);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                    tmem_st32(tl + col_o + c * 32, o);
-                }
-            }
-            weights(m_run, tsum);
-            l += tsum;
-        }
-        // P_t over the first half of S_t: keys 64 hh .. +63 to columns 32 hh .. +31
-        tmem_st32(tl + col_s, wt[0]);
-        tmem_st32(tl + col_s + 32, wt[1]);
-        tmem_wait_st();
-        tc_fence_before();
-        mbar_arrive(sm.bar<D>(C::kBarP + t));
-    }
-    if (ok && T > 0) ok = warp_wait(sm.bar<D>(C::kBarO + t), 0, abort_flag);
-    // dual-key mode: tile b hands its (max, normaliser) to tile a, which
-    // merges the two partial results of each row (weights 2^(m_t - max))
-    float wa = 1.f, wb = 0.f;
-    if (dual) {
-        if (t == 1) {
-            xchg[2 * row] = m_run;
-            xchg[2 * row + 1] = l;
-        }
-        named_bar_sync(3, 256);
-        if (t == 1) {
-            if (!ok && lane == 0) {
-                set_error(a.err, kErrTimeout);
-                *abort_flag = 1;
-            }
-            return;
-        }
-        if (ok) ok = warp_wait(sm.bar<D>(C::kBarO + 1), 0, abort_flag);
-        const float mb = xchg[2 * row], lb = xchg[2 * row + 1];
-        const float M = fmaxf(m_run, mb);
-        wa = m_run == -INFINITY ? 0.f : exp2f(m_run - M);
-        wb = mb == -INFINITY ? 0.f : exp2f(mb - M);
-        l = l * wa + lb * wb;
-        m_run = M;
-    }
-    if (!ok) {
-        if (lane == 0) {
-            set_error(a.err, kErrTimeout);
-            *abort_flag = 1;
-        }
-        return;
-    }
-    tc_fence_after();
+    const bool dual = it.dual, any_keys = it.T > 0;
+    const int qi = it.pos_lo + (dual ? 0 : t) * a.BP + row / a.G;
     const float inv = l > 0.f ? 1.f / l : 0.f;
     const float lse2 = l > 0.f ? m_run + __log2f(l) : -INFINITY;
-    const int h = g * a.G + row % a.G;
+    const int h = it.g * a.G + row % a.G;
     float* part_row = nullptr;
     uint8_t* out_row = nullptr;
-    if (a.n_split > 1) {
-        const size_t pr = ((size_t)blockIdx.x * kPrefillQTiles + t) * kPrefillRows + row;
+    if (it.part >= 0) {
+        const size_t pr = ((size_t)it.part * kPrefillQTiles + t) * kPrefillRows + row;
         part_row = a.part_o + pr * D;
         if (valid) a.part_ml[pr] = lse2;
     } else {
@@ -712,7 +772,7 @@ __device__ void prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
 #pragma unroll
     for (int c = 0; c < D / 32; ++c) {
         uint32_t o[32];
-        if (T > 0) {
+        if (any_keys) {
             tmem_ld32(tl + col_o + c * 32, o);
             tmem_wait_ld();
         } else {
@@ -754,6 +814,267 @@ __device__ void prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
     }
 }
 
+// What a softmax warp carries from item to item, in two words so that the
+// loop over key tiles keeps its registers: the loads of the items before, and,
+// as bits of `par`, the parities of the hand-offs to wait for next.  The item
+// itself stays in its ring slot until the warp has written its output.
+struct SoftmaxPhase {
+    uint32_t ub, par;
+};
+constexpr uint32_t kParS = 1, kParO = 2, kParX = 4;  // S_t, O_t, dual-key exchange
+
+// Softmax warpgroup of query tile t (one row per thread) and its epilogue,
+// for one item.  False: a wait ran out.
+template <int D>
+__device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t tmem, int t,
+                                uint32_t k, SoftmaxPhase& ph, volatile int* abort_flag, int warp,
+                                int lane) {
+    using C = PreCfg<D>;
+    const int wq = warp & 3;
+    const int row = wq * 32 + lane;
+    const Item it = make_item(a, item_read<D>(sm, k));
+    const bool dual = it.dual;
+    const int T_cta = it.T, t0 = it.t0;
+    // dual-key mode: both tiles hold tile a's queries, tile t takes key tiles
+    // t, t + 2, t + 4, ... of the CTA's range
+    const int qi = it.pos_lo + (dual ? 0 : t) * a.BP + row / a.G;
+    const bool valid = row < a.BP * a.G && qi < a.n_q;
+    const int T = dual ? (T_cta + 1 - t) / 2 : T_cta;
+    const int kstep = dual ? 2 : 1, kfirst = dual ? t : 0;
+    float* xchg = reinterpret_cast<float*>(sm.ptr + C::kOffXchg);
+    // A warp none of whose rows is a query only keeps the barrier count: it
+    // waits for each S and signals its P without computing (its rows of P
+    // and O are never read back).
+    if (!__any_sync(0xffffffffu, valid)) {
+        for (int j = 0; j < T; ++j) {
+            if (!warp_wait(sm.bar<D>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
+            ph.par ^= kParS;
+            tc_fence_before();
+            mbar_arrive(sm.bar<D>(C::kBarP + t));
+        }
+        if (T > 0) ph.par ^= kParO;
+        if (dual) {
+            mbar_arrive(sm.bar<D>(t == 1 ? C::kBarX : C::kBarXFree));
+            // (tile b's next P waits for tile a's reads also here)
+            if (t == 1 && !warp_wait(sm.bar<D>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag))
+                return false;
+            ph.par ^= kParX;
+        }
+        return true;
+    }
+    // rows that are no query (their results are never read) mask as the last
+    // one does and stay out of the warp's votes, so that a tile with some does
+    // not take the masked, twice-computed path (2.33 instead of 1.77 us a tile)
+    const int p_row = a.n - a.n_q + (valid ? qi : a.n_q - 1);
+    const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16);
+    const uint32_t col_s = C::kColS + (uint32_t)t * kPrefillKeys;
+    const uint32_t col_o = C::kColO + (uint32_t)t * 128;
+    const float sc = a.scale_log2;  // > 0 (the host raises a zero scale to a tiny one)
+    float m_run = -INFINITY, l = 0.f;
+    // {first keys, flags} of the next key tile; its visibility bits are read
+    // only where a tile is masked (they would hold eight registers of the loop)
+    const PrefillTile* tp = a.tiles + t0 + kfirst;
+    int2 nk = make_int2(0, 0);
+    int nb = 0;
+    if (T > 0) {
+        nk = __ldg(reinterpret_cast<const int2*>(tp));
+        nb = __ldg(&tp->key0b);
+    }
+    for (int j = 0; j < T; ++j) {
+        // this tile's record; the next one is fetched while this tile is worked on
+        const int2 wk = nk;
+        const int wb_ = nb;
+        if (j + 1 < T) {
+            nk = __ldg(reinterpret_cast<const int2*>(tp + kstep));
+            nb = __ldg(&tp[kstep].key0b);
+        }
+        if (!warp_wait(sm.bar<D>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
+        ph.par ^= kParS;
+        tc_fence_after();
+        // Raw logits q.k (the scale is applied inside the exponent; it is > 0),
+        // taken 64 columns at a time to keep registers low: one pass for the
+        // row maximum, one for the weights.
+        // keys key0 + c (lower half) and key0b + c (upper half) with c <= lim,
+        // c <= limb are causal
+        const int lim = p_row - wk.x, limb = p_row - wb_;
+        const bool unmasked = (wk.y & kPrefillTileFull) && lim >= 63 && limb >= 63;
+        // Weights 2^(s * scale - m) with the running maximum m, two arguments
+        // at a time with a packed FMA, rounded to bf16 into wt (32 words per
+        // 64 keys).  The normaliser sums the same rounded weights that the PV
+        // product takes (eight fp32 chains), so the output is a convex
+        // combination of the V rows whatever the rounding.
+        // Nothing is stored: S stays intact until the weights are accepted.
+        const uint64_t sc2 = f2pack(sc, sc);
+        uint32_t wt[2][32];
+        auto weights = [&](float m, float& tile_sum) {
+            const float nmu = m == -INFINITY ? 0.f : -m;
+            const uint64_t nmu2 = f2pack(nmu, nmu);
+            float ls[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                uint32_t x[64];
+                tmem_ld32(tl + col_s + 64 * hh, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
+                tmem_ld32(tl + col_s + 64 * hh + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                tmem_wait_ld();
+                if (!unmasked) {
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        const int ww = 2 * hh + w;
+                        const uint32_t mw =
+                            __ldg(&tp->vis[ww]) & low_bits_through((ww < 2 ? lim : limb) - 32 * (ww & 1));
+#pragma unroll
+                        for (int c = 0; c < 32; ++c)
+                            if (!((mw >> c) & 1u)) x[32 * w + c] = 0xff800000u;  // -inf
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const float x0 = __uint_as_float(x[2 * i]), x1 = __uint_as_float(x[2 * i + 1]);
+                    float a0, a1;
+                    f2unpack(ffma2(f2pack(x0, x1), sc2, nmu2), a0, a1);
+                    const __nv_bfloat162 hb = __floats2bfloat162_rn(ex2_ftz(a0), ex2_ftz(a1));
+                    wt[hh][i] = *reinterpret_cast<const uint32_t*>(&hb);
+                    add_bf16x2_f32(wt[hh][i], ls[2 * (i & 3)], ls[2 * (i & 3) + 1]);
+                }
+            }
+            tile_sum = ((ls[0] + ls[1]) + (ls[2] + ls[3])) + ((ls[4] + ls[5]) + (ls[6] + ls[7]));
+        };
+        // The maximum is raised lazily, so most tiles keep it: take the
+        // weights with the current maximum and accept them when no row's sum
+        // exceeds 2^16, which bounds every weight; no maximum is needed for
+        // that.  Otherwise (or when a row has seen no key yet) find the tile's
+        // maximum and redo the tile with it wherever it exceeds the running
+        // one by more than 2^8.
+        float mt = -INFINITY, tsum = 0.f;
+        bool done = false;
+        if (__all_sync(0xffffffffu, m_run != -INFINITY || !valid)) {
+            weights(m_run, tsum);
+            done = !__any_sync(0xffffffffu, valid && tsum > 65536.f);
+        }
+        if (!done) {
+            // row maximum: three-input max over four independent chains
+            float mx[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) mx[c] = -INFINITY;
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                uint32_t x[64];
+                tmem_ld32(tl + col_s + 64 * hh, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
+                tmem_ld32(tl + col_s + 64 * hh + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                tmem_wait_ld();
+                if (!unmasked) {
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        const int ww = 2 * hh + w;
+                        const uint32_t mw =
+                            __ldg(&tp->vis[ww]) & low_bits_through((ww < 2 ? lim : limb) - 32 * (ww & 1));
+#pragma unroll
+                        for (int c = 0; c < 32; ++c)
+                            if (!((mw >> c) & 1u)) x[32 * w + c] = 0xff800000u;  // -inf
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 64; c += 8) {
+                    mx[0] = fmax3(mx[0], __uint_as_float(x[c]), __uint_as_float(x[c + 1]));
+                    mx[1] = fmax3(mx[1], __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]));
+                    mx[2] = fmax3(mx[2], __uint_as_float(x[c + 4]), __uint_as_float(x[c + 5]));
+                    mx[3] = fmax3(mx[3], __uint_as_float(x[c + 6]), __uint_as_float(x[c + 7]));
+                }
+            }
+            mt = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]) * sc;
+        }
+        if (done) {
+            l += tsum;
+        } else {
+            const bool need = valid && mt > m_run + 8.f;
+            float alpha = 1.f;
+            if (need) {
+                alpha = exp2f(m_run - mt);
+                m_run = mt;
+                l *= alpha;
+            }
+            if (j > 0 && __any_sync(0xffffffffu, need)) {
+                // O_t holds the products up to key tile j - 1 (complete: S_t(j)
+                // was issued after them): rescale it in place
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t o[32];
+                    tmem_ld32(tl + col_o + c * 32, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                    tmem_st32(tl + col_o + c * 32, o);
+                }
+            }
+            weights(m_run, tsum);
+            l += tsum;
+        }
+        // P_t over the first half of S_t: keys 64 hh .. +63 to columns 32 hh .. +31.
+        // One warp also sees that the tiles of the products that follow have
+        // landed (long ago, as a rule): V_j, and the K tile of the next S.
+        bool landed = true;
+        uint32_t fv = 0, fk = 0, pv = 0, pk = 0;
+        if (wq == 0 && t == 0 && !dual) {
+            const uint32_t uv = ph.ub + 2 * j + 1, uk = uv + 1;
+            fv = sm.bar<D>(C::kBarFull + uv % C::kSlots);
+            pv = (uv / C::kSlots) & 1;
+            fk = j + 1 < T ? sm.bar<D>(C::kBarFull + uk % C::kSlots) : fv;
+            pk = j + 1 < T ? (uk / C::kSlots) & 1 : pv;
+            landed = mbar_try_wait(fv, pv) & mbar_try_wait(fk, pk);
+        }
+        tmem_st32(tl + col_s, wt[0]);
+        tmem_st32(tl + col_s + 32, wt[1]);
+        tmem_wait_st();
+        if (!__all_sync(0xffffffffu, landed)) {
+            if (!warp_wait(fv, pv, abort_flag) || !warp_wait(fk, pk, abort_flag)) return false;
+        }
+        tc_fence_before();
+        mbar_arrive(sm.bar<D>(C::kBarP + t));
+        tp += kstep;
+    }
+    if (T > 0) {
+        if (!warp_wait(sm.bar<D>(C::kBarO + t), (ph.par & kParO) != 0, abort_flag)) return false;
+        ph.par ^= kParO;
+    }
+    // dual-key mode: tile b hands its (max, normaliser) to tile a, which
+    // merges the two partial results of each row (weights 2^(m_t - max)) and
+    // reads O_b, complete by tile b's wait above
+    float wa = 1.f, wb = 0.f;
+    tc_fence_after();
+    if (dual && t == 1) {
+        xchg[2 * row] = m_run;
+        xchg[2 * row + 1] = l;
+        tc_fence_before();
+        mbar_arrive(sm.bar<D>(C::kBarX));
+        // tile b's next P (and with it the products that overwrite O_b) waits
+        // until tile a has read O_b
+        if (!warp_wait(sm.bar<D>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag)) return false;
+        ph.par ^= kParX;
+        tc_fence_after();
+        return true;
+    }
+    if (dual) {
+        if (!warp_wait(sm.bar<D>(C::kBarX), (ph.par & kParX) != 0, abort_flag)) return false;
+        ph.par ^= kParX;
+        tc_fence_after();
+        const float mb = xchg[2 * row], lb = xchg[2 * row + 1];
+        const float M = fmaxf(m_run, mb);
+        wa = m_run == -INFINITY ? 0.f : exp2f(m_run - M);
+        wb = mb == -INFINITY ? 0.f : exp2f(mb - M);
+        l = l * wa + lb * wb;
+        m_run = M;
+    }
+    // the item again, from its slot
+    const int4 raw = item_read<D>(sm, k);
+    prefill_write<D>(a, make_item(a, raw), tl, col_o, t, row, valid, m_run, l, wa, wb);
+    if (dual) {
+        tc_fence_before();
+        mbar_arrive(sm.bar<D>(C::kBarXFree));
+    }
+    return true;
+}
+
 template <int D>
 __global__ void __launch_bounds__(320, 1)
     sq_prefill_kernel(const __grid_constant__ CUtensorMap pool_map,
@@ -766,16 +1087,9 @@ __global__ void __launch_bounds__(320, 1)
     sm.base = smem_addr(sm.ptr);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm.ptr + C::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm.ptr + C::kOffMisc + 4);
-    int* sched = reinterpret_cast<int*>(sm.ptr + C::kOffMisc + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the split-merging kernel that follows may be scheduled from here on
     grid_launch_dependents();
-    // heaviest CTA tiles (latest positions) first
-    const int split = blockIdx.x % a.n_split;
-    const int rest = blockIdx.x / a.n_split;
-    const int g = rest % a.Hkv;
-    const int qt = a.n_qt - 1 - rest / a.Hkv;
-    const int pos_lo = qt * kPrefillQTiles * a.BP;
     if (threadIdx.x == 0) {
         mbar_init(sm.bar<D>(C::kBarQ), 1);
         for (int s = 0; s < C::kSlots; ++s) {
@@ -788,7 +1102,15 @@ __global__ void __launch_bounds__(320, 1)
             mbar_init(sm.bar<D>(C::kBarO + b), 1);
         }
         mbar_init(sm.bar<D>(C::kBarVfix), 1);
+        mbar_init(sm.bar<D>(C::kBarQFree), 1);
         mbar_init(sm.bar<D>(C::kBarDone), 1);
+        for (int s = 0; s < kItemSlots; ++s) {
+            mbar_init(sm.bar<D>(C::kBarItem + s), 1);
+            mbar_init(sm.bar<D>(C::kBarItemFree + s), kItemReaders);
+        }
+        mbar_init(sm.bar<D>(C::kBarClc), 1);
+        mbar_init(sm.bar<D>(C::kBarX), 128);
+        mbar_init(sm.bar<D>(C::kBarXFree), 128);
         fence_mbar_init();
         *abort_flag = 0;
     }
@@ -796,34 +1118,56 @@ __global__ void __launch_bounds__(320, 1)
         tmem_alloc(smem_addr(tmem_slot), C::kTmemCols);
         tmem_relinquish();
     }
+    FirstItem start;
+    if (warp == 0) {
+        if (lane == 0) {
+            prefetch_tmap(&pool_map);
+            prefetch_tmap(&qmap);
+        }
+        if (a.plan_ready) start.read(a, lane);
+    }
     // Launched as a programmatic dependent: the set-up above overlapped the
-    // preceding kernel's tail; the plan, the queries and the pool are read
-    // only from here on.
+    // preceding kernel's tail; the queries and the pool, and a plan that was
+    // not on the device before that kernel, are read only from here on.
     grid_dependency_wait();
-    if (threadIdx.x == 0) {
-        // key tiles up to the CTA tile's last query position, split evenly
-        const int lo = __ldg(&a.qt_tiles[qt]);
-        const int t0 = (int)((int64_t)lo * split / a.n_split);
-        sched[0] = t0;
-        sched[1] = (int)((int64_t)lo * (split + 1) / a.n_split) - t0;
+    if (warp == 0) {
+        if (!a.plan_ready) start.read(a, lane);
+        if (lane == 0) {  // the thread that initialised the barriers
+            *reinterpret_cast<int4*>(sm.ptr + C::kOffItems) = start.raw;
+            mbar_arrive(sm.bar<D>(C::kBarItem));
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int t0 = sched[0], T = sched[1];
-    // tile b is empty when every query of the CTA tile fits in tile a; it then
-    // takes every other key tile of tile a's queries (dual-key mode)
-    const bool two = pos_lo + a.BP < a.n_q;
-    const bool dual = !two && T >= 2;
     if (warp == 0) {
-        prefill_produce<D>(&pool_map, &qmap, a, sm, g, pos_lo, t0, T, two, dual, abort_flag, lane);
+        prefill_produce<D>(&pool_map, &qmap, a, sm, start, abort_flag, lane);
     } else if (warp == 1) {
-        if (lane == 0) prefill_mma<D>(a, sm, tmem, T, two, dual, abort_flag);
+        if (lane == 0) prefill_mma<D>(a, sm, tmem, abort_flag);
         __syncwarp();
-    } else if (warp < 6 || two || dual) {
-        prefill_softmax<D>(a, sm, tmem, (warp - 2) >> 2, g, pos_lo, t0, T, dual, abort_flag, warp,
-                           lane);
+    } else {
+        const int t = (warp - 2) >> 2;
+        SoftmaxPhase ph = {0, 0};
+        bool ok;
+        for (uint32_t k = 0;; ++k) {
+            ok = __all_sync(0xffffffffu, item_wait<D>(sm, k, abort_flag));
+            if (!ok) break;
+            const int4 raw = item_read<D>(sm, k);
+            if (raw.z < 0) break;
+            const Item it = make_item(a, raw);
+            if (t == 0 || it.two || it.dual) {
+                ok = prefill_softmax<D>(a, sm, tmem, t, k, ph, abort_flag, warp, lane);
+                if (!ok) break;
+            }
+            ph.ub += 2 * raw.z;
+            __syncwarp();
+            if (lane == 0) item_free<D>(sm, k);
+        }
+        if (!ok && lane == 0) {
+            if (!*abort_flag) set_error(a.err, kErrTimeout);
+            *abort_flag = 1;
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -834,7 +1178,7 @@ __global__ void __launch_bounds__(320, 1)
 }
 
 // Merges the key-range splits of each query row: weights 2^(lse_s - max).
-// One warp per (CTA tile, query tile, row); the lanes take the splits' log-sum-
+// One warp per (split unit, query tile, row); the lanes take the splits' log-sum-
 // exps (up to 64 splits).  The partial outputs of the first 24 splits are
 // loaded together with them, so a row of up to 24 splits costs one round trip;
 // an empty split's partial (never written) is read but selected away.
@@ -842,26 +1186,31 @@ template <int D>
 __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCombineArgs a) {
     constexpr int V = D / 32;  // output elements per lane
     constexpr int U = 24;      // splits per batch of loads
+    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    constexpr int kRowsPerUnit = kPrefillQTiles * kPrefillRows;
+    if (gw >= a.n_merges * kRowsPerUnit) {
+        grid_dependency_wait();
+        return;
+    }
+    const int tr = gw % kRowsPerUnit;
+    // the plan was uploaded before the prefill kernel started
+    const PrefillMerge mg = a.merges[gw / kRowsPerUnit];
+    const int n_split = mg.n;
+    const int t = tr / kPrefillRows, row = tr % kPrefillRows;
+    const int qt = mg.unit / a.Hkv, g = mg.unit % a.Hkv;
+    const int qi = (qt * kPrefillQTiles + t) * a.BP + row / a.G;
     // programmatic dependent of the prefill kernel: wait for its partials;
     // the next layer's prefill may then be scheduled
     grid_dependency_wait();
     grid_launch_dependents();
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    const int units = a.n_qt * a.Hkv;
-    constexpr int kRowsPerUnit = kPrefillQTiles * kPrefillRows;
-    if (gw >= units * kRowsPerUnit) return;
-    const int rest = gw / kRowsPerUnit, tr = gw % kRowsPerUnit;
-    const int t = tr / kPrefillRows, row = tr % kPrefillRows;
-    const int g = rest % a.Hkv, qt = a.n_qt - 1 - rest / a.Hkv;
-    const int qi = (qt * kPrefillQTiles + t) * a.BP + row / a.G;
     if (row >= a.BP * a.G || qi >= a.n_q) return;
     const int h = g * a.G + row % a.G;
     // partial row of split s: part0 + s * kRowsPerUnit
-    const size_t part0 = ((size_t)rest * a.n_split * kPrefillQTiles + t) * kPrefillRows + row;
-    const float ml0 = lane < a.n_split ? a.part_ml[part0 + (size_t)lane * kRowsPerUnit] : -INFINITY;
+    const size_t part0 = ((size_t)mg.part0 * kPrefillQTiles + t) * kPrefillRows + row;
+    const float ml0 = lane < n_split ? a.part_ml[part0 + (size_t)lane * kRowsPerUnit] : -INFINITY;
     const float ml1 =
-        lane + 32 < a.n_split ? a.part_ml[part0 + (size_t)(lane + 32) * kRowsPerUnit] : -INFINITY;
+        lane + 32 < n_split ? a.part_ml[part0 + (size_t)(lane + 32) * kRowsPerUnit] : -INFINITY;
     float vals[U][V];
     auto load = [&](int s0) {
 #pragma unroll
@@ -869,7 +1218,7 @@ __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCo
             const int s = s0 + u;  // the same in every lane
 #pragma unroll
             for (int e = 0; e < V; ++e) vals[u][e] = 0.f;
-            if (s < a.n_split) {
+            if (s < n_split) {
                 const float* po = a.part_o + (part0 + (size_t)s * kRowsPerUnit) * D + lane * V;
                 if constexpr (V == 4) {
                     const float4 v = *reinterpret_cast<const float4*>(po);
@@ -896,13 +1245,13 @@ __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCo
     float acc[V];
 #pragma unroll
     for (int e = 0; e < V; ++e) acc[e] = 0.f;
-    for (int s0 = 0; W > 0.f && s0 < a.n_split; s0 += U) {
+    for (int s0 = 0; W > 0.f && s0 < n_split; s0 += U) {
         if (s0 > 0) load(s0);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int s = s0 + u;
             const float ws = __shfl_sync(0xffffffffu, s < 32 ? w0 : w1, s & 31);
-            if (s < a.n_split && ws > 0.f) {
+            if (s < n_split && ws > 0.f) {
 #pragma unroll
                 for (int e = 0; e < V; ++e) acc[e] += ws * vals[u][e];
             }
@@ -951,7 +1300,7 @@ cudaError_t prefill_prepare(int D) {
 
 cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
                            const PrefillArgs& a, int D, cudaStream_t st) {
-    const unsigned grid = (unsigned)(a.n_qt * a.Hkv * a.n_split);
+    const unsigned grid = (unsigned)a.n_items;
     if (grid == 0) return cudaSuccess;
     // a programmatic dependent of whatever precedes it: its barrier and tensor
     // memory set-up overlaps that work's tail (it waits before any read)
@@ -974,7 +1323,7 @@ cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
 }
 
 cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStream_t st) {
-    const int64_t warps = (int64_t)a.n_qt * a.Hkv * kPrefillQTiles * kPrefillRows;
+    const int64_t warps = (int64_t)a.n_merges * kPrefillQTiles * kPrefillRows;
     const unsigned grid = (unsigned)((warps * 32 + 255) / 256);
     if (grid == 0) return cudaSuccess;
     // scheduled while the prefill kernel's last CTAs run; waits for them

@@ -57,26 +57,145 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem], issued by one thread.
-__device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                            uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
+// One product over a contraction of steps of 16 elements, issued by one thread
+// as one block of instructions.  The issuing thread is the bound of a stream
+// of 128 x 128 products (64 cycles each on the tensor core), so each step
+// costs it as little as possible: a descriptor's low word holds address / 16
+// in 14 bits, every operand here lies below 2^18 bytes, so a step adds a
+// constant to that word alone.
+//
+// D[tmem] = A[smem] * B[smem], both K-major with the same high descriptor
+// word, D / 16 steps over one or two 64-column blocks of 16 KiB.
+template <int N>
+__device__ __forceinline__ void mma_bf16_ss_steps(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
+                                                  uint32_t hi, uint32_t idesc) {
+    static_assert(N == 4 || N == 8, "one or two 64-column blocks");
+    if constexpr (N == 8)
+        asm volatile(
+            "{\n\t"
+            ".reg .pred f, t;\n\t"
+            ".reg .b32 la, lb;\n\t"
+            ".reg .b64 a, b;\n\t"
+            "setp.ne.b32 f, 0, 0;\n\t"
+            "setp.eq.b32 t, 0, 0;\n\t"
+            "mov.b64 a, {%1, %3};\n\t"
+            "mov.b64 b, {%2, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, f;\n\t"
+            "add.u32 la, %1, 2;\n\t"
+            "add.u32 lb, %2, 2;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 4;\n\t"
+            "add.u32 lb, %2, 4;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 6;\n\t"
+            "add.u32 lb, %2, 6;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 1024;\n\t"
+            "add.u32 lb, %2, 1024;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 1026;\n\t"
+            "add.u32 lb, %2, 1026;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 1028;\n\t"
+            "add.u32 lb, %2, 1028;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 1030;\n\t"
+            "add.u32 lb, %2, 1030;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "}\n\t"
+            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t"
+            ".reg .pred f, t;\n\t"
+            ".reg .b32 la, lb;\n\t"
+            ".reg .b64 a, b;\n\t"
+            "setp.ne.b32 f, 0, 0;\n\t"
+            "setp.eq.b32 t, 0, 0;\n\t"
+            "mov.b64 a, {%1, %3};\n\t"
+            "mov.b64 b, {%2, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, f;\n\t"
+            "add.u32 la, %1, 2;\n\t"
+            "add.u32 lb, %2, 2;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 4;\n\t"
+            "add.u32 lb, %2, 4;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "add.u32 la, %1, 6;\n\t"
+            "add.u32 lb, %2, 6;\n\t"
+            "mov.b64 a, {la, %3};\n\t"
+            "mov.b64 b, {lb, %3};\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, t;\n\t"
+            "}\n\t"
+            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc)
+            : "memory");
 }
 
-// D[tmem] (+)= A[tmem] * B[smem], issued by one thread.  A (M rows x K) sits
-// in TMEM with row m in lane m and two bf16 per 32-bit column (column c holds
-// elements 2c in its low half and 2c + 1 in its high half), so a K step of 16
-// advances the A address by 8 columns.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b,
-                                            uint32_t idesc, uint32_t accumulate) {
+// D[tmem] (+)= A[tmem] * B[smem] over 8 steps.  A (M rows x K) sits in TMEM
+// with row m in lane m and two bf16 per 32-bit column (column c holds elements
+// 2c in its low half and 2c + 1 in its high half), so a step advances the A
+// address by 8 columns; B is MN-major, a step 16 rows of 128 bytes.
+__device__ __forceinline__ void mma_bf16_ts_steps8(uint32_t d_tmem, uint32_t a, uint32_t b_lo,
+                                                   uint32_t b_hi, uint32_t idesc,
+                                                   uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
+        "{\n\t"
+        ".reg .pred f, t;\n\t"
+        ".reg .b32 la, lb;\n\t"
+        ".reg .b64 b;\n\t"
+        "setp.ne.b32 f, %5, 0;\n\t"
+        "setp.eq.b32 t, 0, 0;\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, f;\n\t"
+        "add.u32 la, %1, 8;\n\t"
+        "add.u32 lb, %2, 128;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 16;\n\t"
+        "add.u32 lb, %2, 256;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 24;\n\t"
+        "add.u32 lb, %2, 384;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 32;\n\t"
+        "add.u32 lb, %2, 512;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 40;\n\t"
+        "add.u32 lb, %2, 640;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 48;\n\t"
+        "add.u32 lb, %2, 768;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "add.u32 la, %1, 56;\n\t"
+        "add.u32 lb, %2, 896;\n\t"
+        "mov.b64 b, {lb, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [la], b, %4, t;\n\t"
+        "}\n\t"
+        ::"r"(d_tmem), "r"(a), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
