@@ -159,11 +159,18 @@ int64_t sqh_peak_live_pages(void* c) { return static_cast<HostCache*>(c)->peak_l
 int32_t sqh_evict_tile_rows(int32_t P, int32_t D) { return evict_tile_rows_for(P, D); }
 int32_t sqh_evict_stages(int64_t planes, int32_t num_sms) { return evict_stages_for(planes, num_sms); }
 
+// `sqh_decode_costs` sets the units' start-up costs of the plans that follow
+// (negative: the library's own).
+static int32_t g_unit_cost = kUnitCostStages, g_short_cost = kUnitCostStages;
+void sqh_decode_costs(int32_t unit, int32_t small) {
+    g_unit_cost = unit < 0 ? kDecodeUnitCost : unit;
+    g_short_cost = small < 0 ? kDecodeShortUnitCost : small;
+}
 int sqh_plan_decode(void* c, const int32_t* handles, int32_t n, int32_t n_ctas,
                     int64_t* layout_out, uint8_t* buf, int64_t buf_bytes) {
     HostCache* hc = static_cast<HostCache*>(c);
     DecodePlanHost p;
-    int rc = plan_decode(*hc, handles, n, n_ctas, &p);
+    int rc = plan_decode(*hc, handles, n, n_ctas, &p, g_unit_cost, g_short_cost);
     if (rc != kOk) return rc;
     DecodePlanLayout L = plan_layout(p, n, hc->geom().Hkv);
     int64_t v[17] = {L.segs, L.items, L.cta_begin, L.page_ids, L.comb_off, L.arrive, L.total,

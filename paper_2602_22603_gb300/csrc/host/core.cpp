@@ -513,7 +513,7 @@ void evict_chunks(const std::vector<int32_t>& window_tile, int32_t n_tiles, int3
 // decode planning
 
 int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
-                int32_t n_ctas, DecodePlanHost* out) {
+                int32_t n_ctas, DecodePlanHost* out, int32_t unit_cost, int32_t short_cost) {
     *out = DecodePlanHost();
     const Geometry& g = c.geom();
     if (n_seqs < 1 || !handles || n_ctas < 1) return kInvalidArg;
@@ -630,8 +630,8 @@ int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
     }
 
     // (segment, head) units and an even split of their cost over the
-    // persistent CTAs.  On the cost line a unit occupies kUnitCostStages
-    // (its start-up) followed by its stages; an item is the overlap of a
+    // persistent CTAs.  On the cost line a unit occupies its start-up cost
+    // followed by its stages; an item is the overlap of a
     // CTA's share with a unit's stages.  Units go family by family, head by
     // head, each family's segments in tree order: a fork's own short tail
     // follows the shared prefix of the same head, so it lands in the CTA that
@@ -655,15 +655,17 @@ int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
     }
     std::vector<int64_t> unit_start;  // where the unit's stages begin on the cost line
     std::vector<int64_t> unit_end;
-    int64_t total = 0;
+    int64_t total = 0, stages = 0;
     for (size_t v = 0; v < unit_seg.size(); ++v) {
-        total += kUnitCostStages;
+        const int32_t n = ceil_div(out->segs[unit_seg[v]].n_tok, kStageTokens);
+        total += n <= kShortUnitStages ? short_cost : unit_cost;
         unit_start.push_back(total);
-        total += ceil_div(out->segs[unit_seg[v]].n_tok, kStageTokens);
+        total += n;
+        stages += n;
         unit_end.push_back(total);
     }
     const int64_t n_units = (int64_t)unit_start.size();
-    const int32_t ctas = (int32_t)std::min<int64_t>(n_ctas, total - n_units * kUnitCostStages);
+    const int32_t ctas = (int32_t)std::min<int64_t>(n_ctas, stages);
     out->n_ctas = ctas;
     out->cta_begin.resize(ctas + 1);
     int64_t u = 0;
@@ -671,7 +673,7 @@ int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
         const int64_t b = total * cta / ctas, e = total * (cta + 1) / ctas;
         out->cta_begin[cta] = (int32_t)out->items.size();
         while (u < n_units && unit_end[u] <= b) ++u;
-        for (int64_t v = u; v < n_units && unit_start[v] - kUnitCostStages < e; ++v) {
+        for (int64_t v = u; v < n_units && (v == 0 ? 0 : unit_end[v - 1]) < e; ++v) {
             const int64_t lo = std::max(b, unit_start[v]), hi = std::min(e, unit_end[v]);
             if (hi <= lo) continue;
             DecodeItem it;

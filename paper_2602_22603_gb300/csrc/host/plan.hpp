@@ -11,13 +11,24 @@ namespace sq {
 constexpr int kRowsPerTile = 16;
 // Tokens of K/V one pipeline stage of the decode kernel holds.
 constexpr int kStageTokens = 64;
-// Consumer warps of the decode kernel; each owns kStageTokens / 4 tokens.
-constexpr int kDecodeConsumerWarps = 4;
+// Consumer warps of the decode kernel: two groups that take alternate stages,
+// four warps each, kStageTokens / 4 tokens of a stage per warp.
+constexpr int kDecodeGroups = 2;
+constexpr int kDecodeConsumerWarps = 4 * kDecodeGroups;
 // Fixed cost of starting a work unit, in stages: its query reload and its
 // item-end merge.  The planner balances stages plus this cost per unit, so a
 // CTA that gets many short units (e.g. the few-token tails of several forks)
 // is not the one every other CTA waits for.
 constexpr int kUnitCostStages = 2;
+// The costs the decode calls plan with.  A stage passes in 0.7 us; a unit's
+// start and end hide behind the stages of its neighbours unless it is a stage
+// or two long.  Measured, us per pass for costs (2, 2) (4, 4) (4, 8) (6, 6):
+// 36 short sequences x 8 layers 379 376 376 383; four agents with forks and
+// their one-stage tails x 8 layers 384 377 371 372; an agent turn 2,624 2,549
+// 2,514 2,513; one 32k sequence x 32 layers 809 805 805 802.
+constexpr int kShortUnitStages = 2;
+constexpr int kDecodeUnitCost = 4;
+constexpr int kDecodeShortUnitCost = 8;
 
 // A run of logical pages read once for a group of sequences that hold the
 // same physical pages there (a main thread and its forks, Sec. 3.4).

@@ -11,27 +11,39 @@
 // group of sequences holds in common (a main thread and its forked auxiliary
 // threads, Sec. 3.4) is one segment; a (segment, KV head) pair is a list of
 // 64-token stages; the stages of all pairs are dealt evenly to persistent
-// CTAs.  Each CTA streams its stages through a TMA + mbarrier ring in shared
-// memory; each of four consumer warps owns 16 tokens of a stage and keeps an
+// CTAs, one per SM.
+//
+// A CTA has two consumer groups of four warps, each with a producer warp and a
+// TMA + mbarrier ring of its own (2 x 96 KiB in flight per SM); the groups take
+// alternate stages.  A consumer warp owns 16 tokens of a stage and keeps an
 // online-softmax partial (max, sum, unnormalised output) for up to 16 query
-// rows — the G heads of every sequence in the group, so a shared page is read
-// from HBM once for all of them.
+// rows - the G heads of every sequence in the segment's group, so a shared page
+// is read from HBM once for all of them.  At an item's end the consumers leave
+// their rows in shared memory and go on; two closing warps add them, write the
+// item's partial and merge what it completes.
+//
+// What bounds it: HBM in long calls (the read probe's rate at 128k); in short
+// ones the chain after the last stage (add, partial, arrival, merge, ~6 us) and
+// the start.  Two CTAs per SM with the same ring space, each closing its items
+// itself, left twice the entries per run and stalled at every item's end.  Per
+// call at 32q/8kv, d = 128, before and after: one sequence of 32,768 tokens
+// 27.5 and 25.1 us, 36 sequences of 250 .. 6,000 tokens 51.4 and 47.0 us, four
+// agents and their forks at 20,000 .. 60,000 tokens with partial pages 54.6 and
+// 46.4 us; eight of 131,072 and their forks 604 us either way.
 //
 // Merge: an item leaves one partial (max, sum, unnormalised output) per group
 // member, in that (sequence, KV head)'s contiguous run of entries; a member
-// whose run is this one item gets its normalised output directly.  After its
-// last item a CTA counts its arrivals on each (sequence, KV head) it touched;
-// the CTA that brings a count to the number of entries merges that run
-// (max of the maxima, weights 2^(m - M)) and writes the normalised output.
-// Counts are zero in every uploaded plan and the completing arrival resets
-// its count, so every call starts from zero.
+// whose run is this one item gets its normalised output directly.  After an
+// item a CTA counts its arrival on each of the item's runs; the CTA that brings
+// a count to the number of entries merges that run (max of the maxima, weights
+// 2^(m - M)) and writes the normalised output.  Counts are zero in every
+// uploaded plan and the merger resets its count, so every call starts from
+// zero.
 //
 // Start-up: the kernel is a programmatic dependent of whatever precedes it.
-// When the plan was already on the device (a reused plan), the producer reads
-// its item range and first stages into registers and prefetches those stages
-// into L2 before the dependency wait; the K/V rows themselves reach shared
-// memory only after the wait, through L2, which holds whatever the preceding
-// kernel wrote to them.
+// When the plan was already on the device (a reused plan), every role reads its
+// first items before the dependency wait, and stages in pages that no running
+// work writes are loaded before it.
 //
 // Page fills: after a ragged eviction a page may hold fewer rows than it has
 // slots (its rows first, then zeros or rows once appended).  Stages are in
@@ -58,17 +70,30 @@ struct DecCfg {
     static constexpr int kBlockBytes = kStageTokens * 128;       // one column block of a tile
     static constexpr int kTileBytes = kColBlocks * kBlockBytes;  // K (or V) of one stage
     static constexpr int kStageBytes = 2 * kTileBytes;
-    static constexpr int kStages = (D == 128) ? 3 : 6;
-    static constexpr int kThreads = (kDecodeConsumerWarps + 1) * 32;
-    // item-end merge of the four consumer warps: per-warp row max / sum,
-    // and one 16-row output tile
-    static constexpr int kMergeStride = D + 8;  // floats per merge row (padded: fewer bank conflicts)
-    static constexpr int kMergeBytes = 2 * kDecodeConsumerWarps * kRowsPerTile * 4 +
-                                       kRowsPerTile * kMergeStride * 4 + kRowsPerTile * 4;
-    // + 1024 alignment slack + 256 for the mbarriers and flags
-    static constexpr int kSmemBytes = kStages * kStageBytes + kMergeBytes + 1024 + 256;
+    static constexpr int kStages = (D == 128) ? 3 : 6;           // per group: 96 KiB in flight
+    static constexpr int kConsumers = kDecodeConsumerWarps * 32;
+    static constexpr int kRingBytes = kDecodeGroups * kStages * kStageBytes;
+    // warps: consumers, a producer per group, two that close items
+    static constexpr int kClosers = 64;
+    static constexpr int kThreads = kConsumers + kDecodeGroups * 32 + kClosers;
+    static constexpr int kOffBars = kRingBytes;
+    // barriers: per group full [kStages], empty [kStages]; then the three of the
+    // items' ends; then the abort flag
+    static constexpr int kBarOut = kDecodeGroups * 2 * kStages;  // a pass's rows are written
+    static constexpr int kBarOutFree = kBarOut + 1;              // ... and read
+    static constexpr int kBarRuns = kBarOut + 2;                 // the last item's runs are listed
+    static constexpr int kOffRed = kOffBars + 256;
+    // item ends: per-warp row max / sum, eight rows of every warp's output, and
+    // the runs an item completed
+    static constexpr int kPassRows = 8;
+    static constexpr int kOffRuns = kOffRed + 2 * kDecodeConsumerWarps * kRowsPerTile * 4;
+    static constexpr int kOffOut = kOffRuns + 256;
+    static constexpr int kOutBytes = kDecodeConsumerWarps * kPassRows * D * 4;
+    static constexpr int kSmemBytes = kOffOut + kOutBytes + 1024;  // + alignment slack
     static constexpr int kNT = D / 8;   // 8-wide output column tiles
     static constexpr int kKS = D / 16;  // 16-deep contraction steps
+    static_assert(kSmemBytes <= 232448 && kOffOut % 16 == 0, "shared memory");
+    static_assert((kBarRuns + 1) * 8 + 4 <= 256, "mbarriers");
 };
 
 __device__ __forceinline__ uint32_t ld_u32(const __nv_bfloat16* p) {
@@ -80,236 +105,221 @@ __device__ __forceinline__ float bf16x2_sum(uint32_t v) {
     return __uint_as_float(v << 16) + __uint_as_float(v & 0xffff0000u);
 }
 
-// ---- start-up work before the grid-dependency wait --------------------------
-constexpr int kPrefetchStages = 4;  // stages prefetched into L2
-constexpr int kFastStages = 3;      // stages whose coordinates are kept in registers
+// ---- producers: one warp per group issues the TMA loads of its stages --------
+// The groups take alternate stages of the CTA, each through a ring of its own.
+// The warp walks its stages in order; the page of the next stage is read while
+// the current one waits for its slot.  Whole-page stages (P >= 64) are issued by
+// lane 0; with smaller pages each lane issues one box (page, column block, K or
+// V).
+template <int D>
+struct Producer {
+    using C = DecCfg<D>;
+    const CUtensorMap* tmap;
+    const DecodeArgs& a;
+    uint8_t* ring;      // the group's slots
+    uint64_t* bars;     // the group's barriers: full [kStages], empty [kStages]
+    volatile int* abort_flag;
+    int group, lane;
+    // this lane's box within a stage of small pages
+    int box_page, box_cb, box_kv;
+    // the current stage: stage s of item it (it0 .. it1), and its lane's page
+    int it, it1, s, s1, head, page_off, n_pages;
+    int32_t pid;      // -1: no box for this lane
+    int slot;
+    uint32_t phase;   // parity of the slot's use
+    uint32_t issued, issued_phase;  // per-slot bits of the last issue
+    bool first;       // the CTA's first stage has not gone out yet
 
-// The coordinates of a CTA's first stages (whole-page stages only, P >= 64):
-// the producer issues their loads right after the wait, without re-reading the
-// plan there.
-struct FastStart {
-    int n;                       // stages read (0: none)
-    int early;                   // of them, issued before the grid-dependency wait
-    int it, s;                   // where the producer continues
-    int32_t row[kFastStages];    // K row coordinate head * P + row0 (V: + Hkv * P)
-    int32_t pid[kFastStages];
-};
-
-__device__ __forceinline__ void fast_start(const DecodeArgs& a, int it0, int it1, FastStart& fs) {
-    const int P = a.P;
-    int it = it0, s = 0, s1 = 0, head = 0, page_off = 0;
-    if (it < it1) {
+    __device__ void init() {
+        box_cb = lane % C::kColBlocks;
+        box_kv = (lane / C::kColBlocks) % 2;
+        box_page = a.P < kStageTokens ? lane / (2 * C::kColBlocks) : 0;
+        it = a.cta_begin[blockIdx.x];
+        it1 = a.cta_begin[blockIdx.x + 1];
+        slot = 0;
+        phase = 0;
+        issued = issued_phase = 0;
+        first = group == 0;
+        if (it < it1) {
+            open_item();
+            s += group;
+            settle();
+        }
+    }
+    __device__ bool more() const { return it < it1; }
+    __device__ void open_item() {
         const DecodeItem* item = a.items + it;
+        const DecodeSeg* seg = a.segs + item->seg;
         s = item->s0;
         s1 = item->s1;
         head = item->head;
-        page_off = a.segs[item->seg].page_off;
+        page_off = seg->page_off;
+        n_pages = seg->n_pages;
     }
-    fs.n = 0;
-#pragma unroll
-    for (int k = 0; k < kFastStages; ++k) {
-        while (it < it1 && s >= s1) {
-            if (++it < it1) {
-                const DecodeItem* item = a.items + it;
-                s = item->s0;
-                s1 = item->s1;
-                head = item->head;
-                page_off = a.segs[item->seg].page_off;
-            }
+    // Carries a stage past the item's end into the items that follow.
+    __device__ void settle() {
+        while (s >= s1) {
+            const int over = s - s1;
+            if (++it == it1) return;
+            open_item();
+            s += over;
         }
-        if (it < it1) {
-            const int tok0 = s * kStageTokens;
-            fs.pid[k] = a.page_ids[page_off + tok0 / P];
-            fs.row[k] = head * P + tok0 % P;
-            fs.n = k + 1;
-            ++s;
-        }
+        const int pi = s * kStageTokens / a.P + box_page;
+        const int per = a.P < kStageTokens ? kStageTokens / a.P : 1;
+        pid = box_page < per && pi < n_pages ? a.page_ids[page_off + pi] : -1;
     }
-    fs.it = it;
-    fs.s = s;
-}
-
-template <int D>
-__device__ void prefetch_first_stages(const CUtensorMap* tmap, const DecodeArgs& a, int it0,
-                                      int it1) {
-    const int P = a.P;
-    const int pages_per_stage = P < kStageTokens ? kStageTokens / P : 1;
-    int n = 0;
-    for (int it = it0; it < it1 && n < kPrefetchStages; ++it) {
-        const DecodeItem* item = a.items + it;
-        const int head = item->head, s1 = item->s1;
-        const DecodeSeg* seg = a.segs + item->seg;
-        const int page_off = seg->page_off, n_pages = seg->n_pages;
-        for (int s = item->s0; s < s1 && n < kPrefetchStages; ++s, ++n) {
-            const int tok0 = s * kStageTokens;
-            const int pi0 = tok0 / P;
-            const int row0 = P > kStageTokens ? (tok0 % P) : 0;
-            const int np = P >= kStageTokens ? 1 : min(pages_per_stage, n_pages - pi0);
-            for (int k = 0; k < np; ++k) {
-                const int32_t p = a.page_ids[page_off + pi0 + k];
-                if ((uint32_t)p >= (uint32_t)a.num_pages) continue;  // reported by the producer
-                for (int cb = 0; cb < DecCfg<D>::kColBlocks; ++cb) {
-                    tma_prefetch_l2_4d(tmap, cb * 64, head * P + row0, p, a.layer);
-                    tma_prefetch_l2_4d(tmap, cb * 64, (a.Hkv + head) * P + row0, p, a.layer);
-                }
-            }
-        }
+    __device__ int row(int kv) const {
+        const int row0 = a.P > kStageTokens ? (s * kStageTokens) & (a.P - 1) : 0;
+        return (kv ? a.Hkv + head : head) * a.P + row0;
     }
-}
-
-// ---- producer: one thread issues the TMA loads of every stage -------------
-// Issues the loads of fast stage k (whole-page stage, ring slot k).
-template <int D>
-__device__ __forceinline__ void issue_fast_stage(const CUtensorMap* tmap, const DecodeArgs& a,
-                                                 const FastStart& fs, int k, uint8_t* smem,
-                                                 uint64_t* bars) {
-    using C = DecCfg<D>;
-    const uint32_t bytes = (uint32_t)kStageTokens * 128u * C::kColBlocks * 2u;
-    const uint32_t full = smem_addr(&bars[k]);
-    const int32_t p = fs.pid[k];
-    if ((uint32_t)p < (uint32_t)a.num_pages) {
-        mbar_arrive_expect_tx(full, bytes);
-        const uint32_t dk = smem_addr(smem + k * C::kStageBytes);
-#pragma unroll
-        for (int cb = 0; cb < C::kColBlocks; ++cb) {
-            tma_load_4d(dk + cb * C::kBlockBytes, tmap, full, cb * 64, fs.row[k], p, a.layer);
-            tma_load_4d(dk + cb * C::kBlockBytes + C::kTileBytes, tmap, full, cb * 64,
-                        fs.row[k] + a.Hkv * a.P, p, a.layer);
-        }
-    } else {
-        set_error(a.err, kErrBounds);
-        mbar_arrive(full);
-    }
-}
-
-template <int D>
-__device__ void produce(const CUtensorMap* tmap, const DecodeArgs& a, int it0, int it1,
-                        const FastStart& fs, uint8_t* smem, uint64_t* bars,
-                        volatile int* abort_flag) {
-    using C = DecCfg<D>;
-    const int P = a.P;
-    const int box_rows = P < kStageTokens ? P : kStageTokens;
-    const int pages_per_stage = P < kStageTokens ? kStageTokens / P : 1;
-    const uint32_t box_bytes = (uint32_t)box_rows * 128u;
-    int slot = 0;
-    uint32_t phase = 0;
-    uint32_t issued = 0, issued_phase = 0;  // per-slot bits of the last issue
-    bool ok = true;
-    int it_start = it0, s_start = -1;       // -1: the item's first stage
-    if (fs.n > 0) {
-        // the first stages, from registers (whole-page stages; fresh slots);
-        // the first fs.early of them were issued before the dependency wait
-#pragma unroll
-        for (int k = 0; k < kFastStages; ++k) {
-            if (k < fs.n) {
-                if (k >= fs.early) issue_fast_stage<D>(tmap, a, fs, k, smem, bars);
-                issued |= 1u << k;
-            }
-        }
-        slot = fs.n;
-        if (slot == C::kStages) {
+    __device__ void advance() {
+        first = false;
+        if (++slot == C::kStages) {
             slot = 0;
-            phase = 1;
+            phase ^= 1;
         }
-        it_start = fs.it;
-        s_start = fs.s;
+        s += kDecodeGroups;
+        settle();
     }
-    for (int it = it_start; it < it1 && ok; ++it) {
-        const DecodeItem item = a.items[it];
-        const DecodeSeg* seg = a.segs + item.seg;
-        const int page_off = seg->page_off, n_pages = seg->n_pages;
-        for (int s = (it == it_start && s_start >= 0) ? s_start : item.s0; s < item.s1; ++s) {
-            const uint32_t full = smem_addr(&bars[slot]);
-            const uint32_t empty = smem_addr(&bars[C::kStages + slot]);
-            if (!mbar_wait(empty, phase ^ 1, abort_flag)) {
-                if (!*abort_flag) set_error(a.err, kErrTimeout);
-                *abort_flag = 1;
-                ok = false;
-                break;
-            }
-            if (*abort_flag) {
-                ok = false;
-                break;
-            }
-            if ((int)blockIdx.x == a.debug_drop_cta && it == it0 && s == item.s0) {
-                // test hook: leave this stage unsignalled (the consumers'
-                // bounded wait runs out; nothing is in flight for it)
-                if (++slot == C::kStages) {
-                    slot = 0;
-                    phase ^= 1;
-                }
-                continue;
-            }
-            const int tok0 = s * kStageTokens;
-            const int pi0 = tok0 / P;
-            const int row0 = P > kStageTokens ? (tok0 % P) : 0;
-            const int np = P >= kStageTokens ? 1 : min(pages_per_stage, n_pages - pi0);
-            int32_t pid[kStageTokens / 8];
-            uint32_t vmask = 0;
-            for (int k = 0; k < np; ++k) {
-                const int32_t p = a.page_ids[page_off + pi0 + k];
-                pid[k] = p;
-                if ((uint32_t)p < (uint32_t)a.num_pages) vmask |= 1u << k;
-                else set_error(a.err, kErrBounds);
-            }
-            const uint32_t bytes = (uint32_t)__popc(vmask) * box_bytes * C::kColBlocks * 2u;
-            uint8_t* stage = smem + slot * C::kStageBytes;
-            if (bytes == 0) {
-                mbar_arrive(full);
-            } else {
-                mbar_arrive_expect_tx(full, bytes);
-                for (int k = 0; k < np; ++k) {
-                    if (!((vmask >> k) & 1u)) continue;
+    // Issues the current stage into its (free) slot.
+    __device__ void issue() {
+        const uint32_t full = smem_addr(&bars[slot]);
+        const uint32_t dst = smem_addr(ring) + slot * C::kStageBytes;
+        if (a.P >= kStageTokens) {
+            if (lane == 0) {
+                if ((uint32_t)pid < (uint32_t)a.num_pages) {
+                    mbar_arrive_expect_tx(full, C::kStageBytes);
+                    const int rk = row(0), rv = row(1);
+#pragma unroll
                     for (int cb = 0; cb < C::kColBlocks; ++cb) {
-                        const uint32_t dk =
-                            smem_addr(stage + cb * C::kBlockBytes + k * box_rows * 128);
-                        tma_load_4d(dk, tmap, full, cb * 64, item.head * P + row0, pid[k],
-                                    a.layer);
-                        tma_load_4d(dk + C::kTileBytes, tmap, full, cb * 64,
-                                    (a.Hkv + item.head) * P + row0, pid[k], a.layer);
+                        tma_load_4d(dst + cb * C::kBlockBytes, tmap, full, cb * 64, rk, pid, a.layer);
+                        tma_load_4d(dst + cb * C::kBlockBytes + C::kTileBytes, tmap, full, cb * 64, rv,
+                                    pid, a.layer);
                     }
+                } else {
+                    set_error(a.err, kErrBounds);
+                    mbar_arrive(full);
                 }
             }
-            issued |= 1u << slot;
-            issued_phase = (issued_phase & ~(1u << slot)) | (phase << slot);
-            if (++slot == C::kStages) {
-                slot = 0;
-                phase ^= 1;
+        } else {
+            const bool valid = pid >= 0 && pid < a.num_pages;
+            if (pid < -1 || pid >= a.num_pages) set_error(a.err, kErrBounds);
+            const uint32_t n = __popc(__ballot_sync(0xffffffffu, valid));
+            if (lane == 0) {
+                if (n) mbar_arrive_expect_tx(full, n * a.P * 128u);
+                else mbar_arrive(full);
+            }
+            __syncwarp();
+            if (valid)
+                tma_load_4d(dst + box_kv * C::kTileBytes + box_cb * C::kBlockBytes +
+                                box_page * a.P * 128,
+                            tmap, full, box_cb * 64, row(box_kv), pid, a.layer);
+        }
+        issued |= 1u << slot;
+        issued_phase = (issued_phase & ~(1u << slot)) | (phase << slot);
+    }
+    // Before the grid-dependency wait (a plan that was on the device): stages in
+    // pages that no running work writes are loaded, up to the ring's depth, and
+    // the first few of the others prefetched into L2.
+    __device__ void early() {
+        if ((int)blockIdx.x == a.debug_drop_cta) return;
+        int n = 0;
+        if (a.kv_early && a.P >= kStageTokens) {
+            for (; n < C::kStages && more(); ++n) {
+                bool unsafe = false;
+                for (int u = lane; u < a.n_unsafe; u += 32) unsafe |= a.unsafe[u] == pid;
+                if (__any_sync(0xffffffffu, unsafe)) break;
+                issue();
+                advance();
             }
         }
+        // (the walk goes on from here after the wait: look ahead on a copy)
+        Producer ahead = *this;
+        for (; n < kPrefetchStages && ahead.more(); ++n) {
+            if (ahead.pid >= 0 && ahead.pid < a.num_pages && (a.P < kStageTokens || lane < 2 * C::kColBlocks))
+                tma_prefetch_l2_4d(tmap, box_cb * 64, ahead.row(box_kv), ahead.pid, a.layer);
+            ahead.advance();
+        }
     }
-    if (!ok) {
-        // Leave only after every copy already issued has landed (bounded).
-        for (int sl = 0; sl < C::kStages; ++sl)
-            if ((issued >> sl) & 1u)
-                mbar_wait(smem_addr(&bars[sl]), (issued_phase >> sl) & 1u);
+    static constexpr int kPrefetchStages = 4;
+    __device__ void run() {
+        bool ok = true;
+        while (more()) {
+            const uint32_t empty = smem_addr(&bars[C::kStages + slot]);
+            ok = __all_sync(0xffffffffu, mbar_wait(empty, phase ^ 1, abort_flag));
+            if (!ok) break;
+            // test hook: leave this stage unsignalled (the consumers' bounded wait
+            // runs out; nothing is in flight for it)
+            if (!(first && (int)blockIdx.x == a.debug_drop_cta)) issue();
+            advance();
+        }
+        if (!ok && lane == 0) {
+            if (!*abort_flag) set_error(a.err, kErrTimeout);
+            *abort_flag = 1;
+            // Leave only after every copy already issued has landed (bounded).
+            for (int sl = 0; sl < C::kStages; ++sl)
+                if ((issued >> sl) & 1u)
+                    mbar_wait(smem_addr(&bars[sl]), (issued_phase >> sl) & 1u);
+        }
+        __syncwarp();
     }
+};
+
+// ---- consumers: two groups of four warps, 16 tokens of a stage per warp ------
+// The groups take alternate stages of the CTA.  Every consumer warp runs every
+// item and reaches every named barrier of every item, also after a wait ran
+// out (it then skips the work only), so the barriers never miss a participant.
+
+// What a consumer lane needs of an item before its first stage; read one item
+// ahead.  (The token count and the members' limits are not among it: an append
+// may rewrite them in a plan that is on the device, so they are read after the
+// dependency wait.)
+struct ItemHead {
+    int seg, head, s0, s1, n_grp, seq0, seq1;
+    __device__ void read(const DecodeArgs& a, int it, int j0, int j1) {
+        const DecodeItem* item = a.items + it;
+        seg = item->seg;
+        head = item->head;
+        s0 = item->s0;
+        s1 = item->s1;
+        const DecodeSeg* sg = a.segs + seg;
+        n_grp = sg->n_grp;
+        seq0 = sg->grp_seq[j0];  // (entries past n_grp are zero)
+        seq1 = sg->grp_seq[j1];
+    }
+};
+
+// One fp32 row of the item-end merge: eight-float blocks XORed with the row, so
+// that the eight rows of a warp's store hit different banks.
+template <int D>
+__device__ __forceinline__ int out_pos(int row, int col) {
+    return row * D + ((((col >> 3) ^ row) & (D / 8 - 1)) << 3) + (col & 7);
 }
 
-// ---- consumers: four warps, 16 tokens of every stage each ------------------
-// Every consumer warp runs every item and every stage and reaches every
-// named barrier of every item, also after a wait ran out (it then skips the
-// work only), so the barriers never miss a participant.
 template <int D>
-__device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, uint64_t* bars,
-                        volatile int* abort_flag, float* merge, int warp, int lane) {
+__device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, uint8_t* smem,
+                        uint64_t* all_bars, volatile int* abort_flag, int warp, int lane) {
     using C = DecCfg<D>;
     const int gid = lane >> 2, tig = lane & 3;
     const int r0 = gid, r1 = gid + 8;
     const int mi = lane >> 3, rr = lane & 7;
-    float* red_m = merge;                                          // [4][16]
-    float* red_l = merge + kDecodeConsumerWarps * kRowsPerTile;    // [4][16]
-    float* red_o = merge + 2 * kDecodeConsumerWarps * kRowsPerTile;  // [16][kMergeStride]
-    float* red_sum = red_o + kRowsPerTile * C::kMergeStride;          // [16] merged row sums
+    const int group = warp >> 2, w4 = warp & 3;
+    const int G = a.G;
+    const int j0 = r0 / G, j1 = r1 / G;
+    uint64_t* bars = all_bars + group * 2 * C::kStages;
+    float* red_m = reinterpret_cast<float*>(smem + C::kOffRed);     // [8][16]
+    float* red_l = red_m + kDecodeConsumerWarps * kRowsPerTile;     // [8][16]
+    float* red_o = reinterpret_cast<float*>(smem + C::kOffOut);     // [8][8][D], out_pos
+    uint32_t n_pass = 0;  // item-end passes so far
+    uint8_t* ring = smem + group * C::kStages * C::kStageBytes;  // the group's slots
     int slot = 0;
     uint32_t phase = 0;
+    int skip = group;   // stages to the group's next one
     bool dead = false;  // warp-uniform: a wait ran out or the CTA aborted
     for (int it = it0; it < it1; ++it) {
-        const DecodeItem item = a.items[it];
+        const ItemHead item = next;
         const DecodeSeg* seg = a.segs + item.seg;
-        const int G = a.G;
-        const int n_grp = seg->n_grp;
-        const int j0 = r0 / G, j1 = r1 / G;
+        const int n_grp = item.n_grp;
         const bool v0 = j0 < n_grp, v1 = j1 < n_grp;
         const int lim0 = v0 ? seg->grp_lim[j0] : 0;
         const int lim1 = v1 ? seg->grp_lim[j1] : 0;
@@ -318,9 +328,9 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
         uint32_t qa[C::kKS][4];
         {
             const __nv_bfloat16* q0 =
-                a.q + ((size_t)(v0 ? seg->grp_seq[j0] : 0) * a.Hq + item.head * G + r0 % G) * D;
+                a.q + ((size_t)(v0 ? item.seq0 : 0) * a.Hq + item.head * G + r0 % G) * D;
             const __nv_bfloat16* q1 =
-                a.q + ((size_t)(v1 ? seg->grp_seq[j1] : 0) * a.Hq + item.head * G + r1 % G) * D;
+                a.q + ((size_t)(v1 ? item.seq1 : 0) * a.Hq + item.head * G + r1 % G) * D;
 #pragma unroll
             for (int kk = 0; kk < C::kKS; ++kk) {
                 const int c = kk * 16 + tig * 2;
@@ -330,12 +340,14 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
                 qa[kk][3] = v1 ? ld_u32(q1 + c + 8) : 0u;
             }
         }
+        if (it + 1 < it1) next.read(a, it + 1, j0, j1);
         float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
         float o[C::kNT][4];
 #pragma unroll
         for (int nd = 0; nd < C::kNT; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
 
-        for (int s = item.s0; s < item.s1; ++s) {
+        int s = item.s0 + skip;
+        for (; s < item.s1; s += kDecodeGroups) {
             const uint32_t full = smem_addr(&bars[slot]);
             const uint32_t empty = smem_addr(&bars[C::kStages + slot]);
             // Pages a ragged eviction left partial: bit r of vm says whether
@@ -347,7 +359,7 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
                 // P is a power of two >= 8 and the 16 rows start at a multiple
                 // of 16: one page holds them all (P >= 16), or two (P = 8)
                 const int P = a.P;
-                const int t0 = s * kStageTokens + warp * 16;  // segment slot position
+                const int t0 = s * kStageTokens + w4 * 16;  // segment slot position
                 const int pq = t0 >> (__ffs(P) - 1);
                 const int f0 = pq < seg->n_pages ? __ldg(&a.page_fill[seg->page_off + pq]) : 0;
                 if (P >= 16) {
@@ -368,16 +380,16 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
                 }
             }
             if (!dead) {
-                const uint32_t kb = smem_addr(smem + slot * C::kStageBytes);
+                const uint32_t kb = smem_addr(ring + slot * C::kStageBytes);
                 const uint32_t vb = kb + C::kTileBytes;
-                const int tbase = s * kStageTokens + warp * 16;  // segment-relative
+                const int tbase = s * kStageTokens + w4 * 16;  // segment-relative
 
                 // S = Q K^T over this warp's 16 tokens (two n8 tiles)
                 float sc[2][4];
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
                 {
-                    const int t = warp * 16 + (mi >> 1) * 8 + rr;
+                    const int t = w4 * 16 + (mi >> 1) * 8 + rr;
                     const uint32_t row = kb + t * 128;
                     const int sw = t & 7;
 #pragma unroll
@@ -448,9 +460,9 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
                     const int first = max(0, n_tok - tbase);
                     const int per_row = C::kColBlocks * 8;  // 16-byte chunks per row
                     const int total = (16 - first) * per_row;
-                    uint8_t* vgen = smem + slot * C::kStageBytes + C::kTileBytes;
+                    uint8_t* vgen = ring + slot * C::kStageBytes + C::kTileBytes;
                     for (int idx = lane; idx < total; idx += 32) {
-                        const int row = warp * 16 + first + idx / per_row;
+                        const int row = w4 * 16 + first + idx / per_row;
                         const int rem = idx % per_row;
                         *reinterpret_cast<uint4*>(vgen + (rem >> 3) * C::kBlockBytes + row * 128 +
                                                   (rem & 7) * 16) = make_uint4(0, 0, 0, 0);
@@ -460,7 +472,7 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
 
                 // O += P V (V^T fragments through ldmatrix.trans)
                 {
-                    const int t = warp * 16 + (mi & 1) * 8 + rr;
+                    const int t = w4 * 16 + (mi & 1) * 8 + rr;
                     const uint32_t row = vb + t * 128;
                     const int sw = t & 7;
 #pragma unroll
@@ -482,141 +494,67 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, uint8_t* smem, ui
                 phase ^= 1;
             }
         }
+        skip = s - item.s1;
 
-        // close the item: merge the four warps' (m, l, o) in shared memory,
-        // then write one partial (unnormalised o, m, l) for the item
+        // Leave the item's rows to the closing warps, eight at a time, and go on
+        // with the next item: nothing here waits for the other consumers.
         l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
         l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
         l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
         l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-        if (tig == 0) {
-            red_m[warp * kRowsPerTile + r0] = dead ? -INFINITY : m0;
-            red_m[warp * kRowsPerTile + r1] = dead ? -INFINITY : m1;
-            red_l[warp * kRowsPerTile + r0] = dead ? 0.f : l0;
-            red_l[warp * kRowsPerTile + r1] = dead ? 0.f : l1;
-        }
-        named_bar_sync(1, kDecodeConsumerWarps * 32);
-        float M0 = -INFINITY, M1 = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kDecodeConsumerWarps; ++w) {
-            M0 = fmaxf(M0, red_m[w * kRowsPerTile + r0]);
-            M1 = fmaxf(M1, red_m[w * kRowsPerTile + r1]);
-        }
-        const float Ms0 = M0 == -INFINITY ? 0.f : M0, Ms1 = M1 == -INFINITY ? 0.f : M1;
-        const float f0 = dead ? 0.f : exp2f(m0 - Ms0), f1 = dead ? 0.f : exp2f(m1 - Ms1);
-        // the merged tile: member j's G rows, plus their (M, L), go to its
-        // partial entry; a member whose run is this item alone gets its
-        // normalised output instead
         const int rows = n_grp * G;
-        const int32_t* ent = a.items[it].ent;
-        const int sole = a.items[it].sole;
-        constexpr int kVecRow = D / 4;  // float4 per row
-        if (threadIdx.x < rows) {
-            const int r = threadIdx.x;
-            float M = -INFINITY;
+        for (int rb = 0; rb < rows; rb += C::kPassRows, ++n_pass) {
+            // the previous pass's rows have been read
+            if (!dead && n_pass > 0) {
+                const bool ok =
+                    mbar_wait(smem_addr(&all_bars[C::kBarOutFree]), (n_pass - 1) & 1, abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0 && !*abort_flag) set_error(a.err, kErrTimeout);
+                    *abort_flag = 1;
+                    dead = true;
+                }
+            }
+            if (dead) continue;
+            const int r = rb + gid;  // this lane's row of the pass: r0, then r1
+            if (tig == 0) {
+                red_m[warp * kRowsPerTile + r] = rb ? m1 : m0;
+                red_l[warp * kRowsPerTile + r] = rb ? l1 : l0;
+            }
+            if (r < rows) {
+                float* wo = red_o + warp * C::kPassRows * D;
 #pragma unroll
-            for (int w = 0; w < kDecodeConsumerWarps; ++w) M = fmaxf(M, red_m[w * kRowsPerTile + r]);
-            const float Ms = M == -INFINITY ? 0.f : M;
-            float L = 0.f;
-#pragma unroll
-            for (int w = 0; w < kDecodeConsumerWarps; ++w)
-                L += red_l[w * kRowsPerTile + r] * exp2f(red_m[w * kRowsPerTile + r] - Ms);
-            red_sum[r] = L;
-            if (!((sole >> (r / G)) & 1))
-                *reinterpret_cast<float4*>(a.part_ml + ((size_t)ent[r / G] * G + r % G) * 4) =
-                    make_float4(M, L, 0.f, 0.f);
+                for (int nd = 0; nd < C::kNT; ++nd)
+                    *reinterpret_cast<float2*>(wo + out_pos<D>(gid, nd * 8 + tig * 2)) =
+                        rb ? make_float2(o[nd][2], o[nd][3]) : make_float2(o[nd][0], o[nd][1]);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&all_bars[C::kBarOut]));
         }
-        // one row's float4 of the merged tile to its destination (read after
-        // a barrier that follows the red_sum writes)
-        auto put = [&](int r, int c4, float4 v) {
-            const int j = r / G;
-            if ((sole >> j) & 1) {
-                const float inv = 1.f / red_sum[r];
-                const size_t ob =
-                    ((size_t)seg->grp_seq[j] * a.Hq + item.head * G + r % G) * D + c4 * 4;
-                if (a.out_f32) {
-                    *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + ob) =
-                        make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
-                } else {
-                    uint2 u;
-                    u.x = pack_bf16x2(v.x * inv, v.y * inv);
-                    u.y = pack_bf16x2(v.z * inv, v.w * inv);
-                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + ob) = u;
-                }
-            } else {
-                float* po = a.part_o + ((size_t)ent[j] * G + r % G) * D;
-                reinterpret_cast<float4*>(po)[c4] = v;
-            }
-        };
-        if (it + 1 == it1) {
-            // The CTA's last item: every warp is past its last stage (the
-            // barrier above) and no copy is pending, so the ring is free.
-            // Each warp leaves its rows there; all threads add the four.
-            float* wo = reinterpret_cast<float*>(smem) + warp * kRowsPerTile * C::kMergeStride;
-#pragma unroll
-            for (int nd = 0; nd < C::kNT; ++nd) {
-                *reinterpret_cast<float2*>(wo + r0 * C::kMergeStride + nd * 8 + tig * 2) =
-                    dead ? make_float2(0.f, 0.f) : make_float2(o[nd][0] * f0, o[nd][1] * f0);
-                *reinterpret_cast<float2*>(wo + r1 * C::kMergeStride + nd * 8 + tig * 2) =
-                    dead ? make_float2(0.f, 0.f) : make_float2(o[nd][2] * f1, o[nd][3] * f1);
-            }
-            named_bar_sync(1, kDecodeConsumerWarps * 32);
-            const float* ro = reinterpret_cast<const float*>(smem);
-            for (int v = threadIdx.x; v < rows * kVecRow; v += kDecodeConsumerWarps * 32) {
-                const int r = v / kVecRow, c4 = v % kVecRow;
-                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int w = 0; w < kDecodeConsumerWarps; ++w) {
-                    const float4 x = *reinterpret_cast<const float4*>(
-                        ro + (w * kRowsPerTile + r) * C::kMergeStride + c4 * 4);
-                    sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
-                }
-                put(r, c4, sum);
-            }
-        } else {
-            // the ring is still in use: the four warps add in turn into one tile
-            for (int w = 0; w < kDecodeConsumerWarps; ++w) {
-                if (w == warp) {
-#pragma unroll
-                    for (int nd = 0; nd < C::kNT; ++nd) {
-                        float2* p0 = reinterpret_cast<float2*>(red_o + r0 * C::kMergeStride + nd * 8 + tig * 2);
-                        float2* p1 = reinterpret_cast<float2*>(red_o + r1 * C::kMergeStride + nd * 8 + tig * 2);
-                        float2 a0 = dead ? make_float2(0.f, 0.f) : make_float2(o[nd][0] * f0, o[nd][1] * f0);
-                        float2 a1 = dead ? make_float2(0.f, 0.f) : make_float2(o[nd][2] * f1, o[nd][3] * f1);
-                        if (w > 0) {
-                            const float2 b0 = *p0, b1 = *p1;
-                            a0.x += b0.x; a0.y += b0.y;
-                            a1.x += b1.x; a1.y += b1.y;
-                        }
-                        *p0 = a0;
-                        *p1 = a1;
-                    }
-                }
-                named_bar_sync(1, kDecodeConsumerWarps * 32);
-            }
-            for (int v = threadIdx.x; v < rows * kVecRow; v += kDecodeConsumerWarps * 32) {
-                const int r = v / kVecRow, c4 = v % kVecRow;
-                put(r, c4, *reinterpret_cast<const float4*>(red_o + r * C::kMergeStride + c4 * 4));
-            }
-        }
-        // the merge buffers are rewritten by the next item only after every
-        // warp has copied them out
-        named_bar_sync(1, kDecodeConsumerWarps * 32);
     }
 }
 
-// ---- arrivals and the merge of finished (sequence, KV head) runs -----------
+// ---- item ends: arrivals and the merge of finished (sequence, KV head) runs ---
+// Two warps close the items while the consumers stream the next ones: they add
+// the consumer warps' rows (weights 2^(m_w - M), warps in order), write the
+// item's partials or outputs, arrive on the runs it belongs to and merge those
+// it completes.  (With the consumers doing this between items, a batch of 36
+// short sequences, ~3 items per CTA, stalled at every end: 51 us per call
+// against TODO.)  The runs that the CTA's last item completes are merged by the
+// consumers, which have nothing else to do by then.
+//
 // The arrival word of a run holds two counts.  Its low half counts the items
 // that finished (a relaxed add, the claim); the claim that brings it to the
 // run's length makes its CTA the merger.  Every other CTA then publishes its
 // partial with a release add to the high half, and the merger, instead of
 // releasing its own partial first (a GPU-scope fence on its critical path),
-// waits with acquire loads until the high half counts the other entries; its
-// own partial it reads back within the CTA.  The merger sets the word back to
-// zero.  Every CTA claims once per (item, group member), also after a wait ran
-// out, so every call leaves every word at zero, and a plan upload writes
-// zeros; the word therefore always starts a call at zero.  A run holds at
-// most 65,535 entries (the planner's limit), so the halves never carry.
+// waits with acquire loads until the high half counts the other entries (their
+// claims came first, so their releases are under way: the wait depends on
+// nothing this CTA still has to do); its own partial it reads back within the
+// CTA.  The merger sets the word back to zero.  Every CTA claims once per
+// (item, group member), also after a wait ran out, so every call leaves every
+// word at zero, and a plan upload writes zeros; the word therefore always
+// starts a call at zero.  A run holds at most 65,535 entries (the planner's
+// limit), so the halves never carry.
 
 // GPU-scope atomics of the arrival protocol.
 __device__ __forceinline__ unsigned atom_add_relaxed_gpu(unsigned* p, unsigned v) {
@@ -633,238 +571,336 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     return v;
 }
 
-// Up to 4 output float4 per thread per round; a round stages whole runs
-// (several when they fit) or one chunk of a long run.
-constexpr int kMergeOuts = 4;
-
-// Stages entries [c0, c0 + cn) of run r (first entry e0) at `dst`:
-// [cn][G][D] outputs, then [cn][G] (m, l, -, -) records.
-template <int D>
-__device__ __forceinline__ void stage_run(const DecodeArgs& a, uint32_t dst, int e0, int c0, int cn,
-                                          int tid) {
-    const int G = a.G;
-    const int nv_o = cn * G * (D / 4);
-    const float* so = a.part_o + (size_t)(e0 + c0) * G * D;
-    for (int v = tid; v < nv_o; v += kDecodeConsumerWarps * 32) cp_async_16(dst + v * 16, so + v * 4);
-    const float* sm = a.part_ml + (size_t)(e0 + c0) * G * 4;
-    const uint32_t dm = dst + nv_o * 16;
-    for (int v = tid; v < cn * G; v += kDecodeConsumerWarps * 32) cp_async_16(dm + v * 16, sm + v * 4);
+// Four consecutive output elements from element `at`: v * inv.
+__device__ __forceinline__ void write_out(const DecodeArgs& a, size_t at, const float4& v, float inv) {
+    if (a.out_f32) {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + at) =
+            make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+    } else {
+        uint2 u;
+        u.x = pack_bf16x2(v.x * inv, v.y * inv);
+        u.y = pack_bf16x2(v.z * inv, v.w * inv);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + at) = u;
+    }
 }
 
-template <int D>
-__device__ void arrive_and_merge(const DecodeArgs& a, int it0, int it1, uint8_t* ring, int* smem_i,
-                                 int warp) {
-    using C = DecCfg<D>;
-    constexpr int kT = kDecodeConsumerWarps * 32;
-    constexpr int kVec = D / 4;                       // float4 per output row
-    const int tid = threadIdx.x;
+// (max, sum, weighted output) of one output float4.
+struct MergeAcc {
+    float M, L;
+    float4 o;
+    __device__ void clear() {
+        M = -INFINITY;
+        L = 0.f;
+        o = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __device__ void rescale(float to) {  // to >= M
+        const float sc = exp2f(M - (to == -INFINITY ? 0.f : to));
+        L *= sc;
+        o.x *= sc; o.y *= sc; o.z *= sc; o.w *= sc;
+        M = to;
+    }
+    __device__ void add(float w, float l, const float4& v) {
+        L += w * l;
+        o.x += w * v.x; o.y += w * v.y; o.z += w * v.z; o.w += w * v.w;
+    }
+};
+
+// One run completed by an item: its (sequence, KV head), entries [e0, e0 + n).
+struct RunRef {
+    int key, e0, n;
+};
+
+// A run's entries are added in two shares (the even and the odd ones), each in
+// order, whoever merges it: the result does not depend on which CTA, or which
+// of its warps, completes the run.  The entries come straight from L2, kBatch
+// at a time.
+template <int D, int kBatch>
+__device__ __forceinline__ MergeAcc merge_batches(const DecodeArgs& a, const RunRef& run, int row,
+                                                  int c4, int share) {
     const int G = a.G;
-    const int outs_run = G * kVec;                    // output float4 of one run (<= 512)
-    const int ent_bytes = G * (D * 4 + 16);           // one staged entry
-    const int cap = C::kStages * C::kStageBytes / ent_bytes;  // entries per round (>= 11)
-    const uint32_t ring_s = smem_addr(ring);
-    int* n_last = smem_i;
-    int* l_key = smem_i + 1;        // completed runs: key, first entry, entries
-    int* l_e0 = l_key + kT;
-    int* l_n = l_e0 + kT;
-    int total = 0;
-    for (int it = it0; it < it1; ++it) total += a.segs[a.items[it].seg].n_grp;
-    for (int rb = 0; rb < total; rb += kT) {
-        if (tid == 0) *n_last = 0;
-        named_bar_sync(1, kT);
-        int key = -1;
-        for (int it = it0, p = 0; it < it1 && p <= rb + tid; ++it) {
-            const DecodeItem* item = a.items + it;
-            const DecodeSeg* seg = a.segs + item->seg;
-            const int j = rb + tid - p;
-            if (j < seg->n_grp && !((item->sole >> j) & 1)) key = seg->grp_seq[j] * a.Hkv + item->head;
-            p += seg->n_grp;
-        }
-        if (key >= 0) {
-            const int e0 = a.comb_off[key], n = a.comb_off[key + 1] - e0;
-            // claim; a CTA that does not complete the run releases its
-            // partials (written before the barrier above) to the merger, which
-            // acquires every other entry's before its reads (its own were
-            // written within the CTA)
-            const unsigned old = atom_add_relaxed_gpu(a.arrive + key, 1u);
-            const bool merger = (old & 0xffffu) + 1u == (unsigned)n;
-            if (!merger) {
-                red_add_release_gpu(a.arrive + key, 0x10000u);
+    const float* po = a.part_o + ((size_t)run.e0 * G + row) * D + c4 * 4;
+    const float* pm = a.part_ml + ((size_t)run.e0 * G + row) * 4;
+    MergeAcc acc;
+    acc.clear();
+    for (int e = share; e < run.n; e += 2 * kBatch) {
+        float2 ml[kBatch];
+        float4 o[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int x = e + 2 * u;
+            if (x < run.n) {
+                ml[u] = __ldcg(reinterpret_cast<const float2*>(pm + (size_t)x * G * 4));
+                o[u] = __ldcg(reinterpret_cast<const float4*>(po + (size_t)x * G * D));
             } else {
-                const uint64_t t0 = globaltimer_ns();
-                for (uint32_t spin = 1;; ++spin) {
-                    if ((ld_acquire_gpu(a.arrive + key) >> 16) == (unsigned)(n - 1)) break;
-                    if ((spin & 31) == 0 && globaltimer_ns() - t0 > kWaitLimitNs) {
-                        set_error(a.err, kErrTimeout);
-                        break;
-                    }
+                ml[u] = make_float2(-INFINITY, 0.f);
+                o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        float bm = acc.M;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) bm = fmaxf(bm, ml[u].x);
+        acc.rescale(bm);
+        const float bs = bm == -INFINITY ? 0.f : bm;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) acc.add(exp2f(ml[u].x - bs), ml[u].y, o[u]);
+    }
+    return acc;
+}
+
+// Long runs (one sequence spread over the GPU: ~19 entries per run) want every
+// load in one round trip; short ones little besides their few entries.
+template <int D>
+__device__ __forceinline__ MergeAcc merge_share(const DecodeArgs& a, const RunRef& run, int row,
+                                                int c4, int share) {
+    return run.n <= 8 ? merge_batches<D, 4>(a, run, row, c4, share)
+                      : merge_batches<D, 12>(a, run, row, c4, share);
+}
+
+// Adds the second share to the first and writes the normalised output.
+template <int D>
+__device__ __forceinline__ void merge_finish(const DecodeArgs& a, const RunRef& run, int row, int c4,
+                                             MergeAcc x, const MergeAcc& y) {
+    const float bm = fmaxf(x.M, y.M);
+    x.rescale(bm);
+    x.add(exp2f(y.M - (bm == -INFINITY ? 0.f : bm)), y.L, y.o);
+    const int i = run.key / a.Hkv, h = (run.key % a.Hkv) * a.G + row;
+    write_out(a, ((size_t)i * a.Hq + h) * D + c4 * 4, x.o, 1.f / x.L);
+}
+
+// The closing warps (et: thread 0 .. 63 of them).
+template <int D>
+__device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem, uint64_t* bars,
+                            volatile int* abort_flag, int et) {
+    using C = DecCfg<D>;
+    constexpr int kVec = D / 4;  // float4 per output row
+    const int G = a.G, lane = et & 31;
+    const float* red_m = reinterpret_cast<const float*>(smem + C::kOffRed);
+    const float* red_l = red_m + kDecodeConsumerWarps * kRowsPerTile;
+    const float* red_o = reinterpret_cast<const float*>(smem + C::kOffOut);
+    int* n_runs = reinterpret_cast<int*>(smem + C::kOffRuns);
+    RunRef* runs = reinterpret_cast<RunRef*>(n_runs + 4);
+    uint32_t n_pass = 0;
+    bool dead = false;  // warp-uniform
+    for (int it = it0; it < it1; ++it) {
+        // read while the item is streamed
+        const DecodeItem* item = a.items + it;
+        const DecodeSeg* seg = a.segs + item->seg;
+        const int head = item->head, sole = item->sole, n_grp = seg->n_grp;
+        const int rows = n_grp * G;
+        // the arrival of this lane's group member (first warp)
+        int key = -1;
+        RunRef mine{-1, 0, 0};
+        if (et < n_grp && !((sole >> et) & 1)) {
+            key = seg->grp_seq[et] * a.Hkv + head;
+            mine.key = key;
+            mine.e0 = a.comb_off[key];
+            mine.n = a.comb_off[key + 1] - mine.e0;
+        }
+        for (int rb = 0; rb < rows; rb += C::kPassRows, ++n_pass) {
+            if (!dead) {
+                const bool ok = mbar_wait(smem_addr(&bars[C::kBarOut]), n_pass & 1, abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0 && !*abort_flag) set_error(a.err, kErrTimeout);
+                    *abort_flag = 1;
+                    dead = true;
                 }
             }
-            if (merger) {
-                a.arrive[key] = 0u;
-                const int k = atomicAdd(n_last, 1);
-                l_key[k] = key;
-                l_e0[k] = e0;
-                l_n[k] = n;
+            if (dead) continue;
+            const int n_out = min(rows - rb, (int)C::kPassRows) * kVec;
+            for (int v = et; v < n_out; v += C::kClosers) {
+                const int pr = v / kVec, c4 = v % kVec, r = rb + pr;
+                float M = -INFINITY;
+#pragma unroll
+                for (int w = 0; w < kDecodeConsumerWarps; ++w)
+                    M = fmaxf(M, red_m[w * kRowsPerTile + r]);
+                const float Ms = M == -INFINITY ? 0.f : M;
+                float L = 0.f;
+                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int w = 0; w < kDecodeConsumerWarps; ++w) {
+                    const float f = exp2f(red_m[w * kRowsPerTile + r] - Ms);
+                    L += red_l[w * kRowsPerTile + r] * f;
+                    const float4 x = *reinterpret_cast<const float4*>(
+                        red_o + w * C::kPassRows * D + out_pos<D>(pr, c4 * 4));
+                    sum.x += x.x * f; sum.y += x.y * f; sum.z += x.z * f; sum.w += x.w * f;
+                }
+                // a member whose run is this item alone gets its normalised output
+                const int j = r / G;
+                if ((sole >> j) & 1) {
+                    write_out(a, ((size_t)seg->grp_seq[j] * a.Hq + head * G + r % G) * D + c4 * 4, sum,
+                              1.f / L);
+                } else {
+                    const size_t pe = (size_t)item->ent[j] * G + r % G;
+                    *reinterpret_cast<float4*>(a.part_o + pe * D + c4 * 4) = sum;
+                    if (c4 == 0)
+                        *reinterpret_cast<float4*>(a.part_ml + pe * 4) = make_float4(M, L, 0.f, 0.f);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&bars[C::kBarOutFree]));
+        }
+        // both warps' partials are written (and the list of the item before read)
+        named_bar_sync(3, C::kClosers);
+        if (et < 32) {
+            bool merger = false;
+            if (key >= 0) {
+                const unsigned old = atom_add_relaxed_gpu(a.arrive + key, 1u);
+                merger = (old & 0xffffu) + 1u == (unsigned)mine.n;
+                if (!merger) {
+                    red_add_release_gpu(a.arrive + key, 0x10000u);
+                } else {
+                    const uint64_t t0 = globaltimer_ns();
+                    for (uint32_t spin = 1;; ++spin) {
+                        if ((ld_acquire_gpu(a.arrive + key) >> 16) == (unsigned)(mine.n - 1)) break;
+                        if ((spin & 31) == 0 && globaltimer_ns() - t0 > kWaitLimitNs) {
+                            set_error(a.err, kErrTimeout);
+                            break;
+                        }
+                    }
+                    a.arrive[key] = 0u;
+                }
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, merger);
+            if (merger) runs[__popc(mask & ((1u << lane) - 1u))] = mine;
+            if (lane == 0) *n_runs = __popc(mask);
+            __syncwarp();
+        }
+        if (it + 1 == it1) {
+            if (et == 0) mbar_arrive(smem_addr(&bars[C::kBarRuns]));
+            break;
+        }
+        named_bar_sync(3, C::kClosers);
+        const int n = *reinterpret_cast<volatile int*>(n_runs);
+        for (int q = 0; q < n; ++q) {
+            const RunRef run = runs[q];
+            for (int x = et; x < G * kVec; x += C::kClosers) {
+                const int row = x / kVec, c4 = x % kVec;
+                const MergeAcc s0 = merge_share<D>(a, run, row, c4, 0);
+                merge_finish<D>(a, run, row, c4, s0, merge_share<D>(a, run, row, c4, 1));
+            }
+        }
+    }
+}
+
+// The runs of the CTA's last item, by the consumers: a thread per share of an
+// output, the second shares through shared memory.
+template <int D>
+__device__ void merge_last_runs(const DecodeArgs& a, uint8_t* smem, uint64_t* bars,
+                                volatile int* abort_flag, int lane) {
+    using C = DecCfg<D>;
+    constexpr int kT = C::kConsumers, kVec = D / 4;
+    const int tid = threadIdx.x;
+    const int outs = a.G * kVec;  // of one run, <= 512
+    const int* n_runs = reinterpret_cast<const int*>(smem + C::kOffRuns);
+    volatile int* failed = const_cast<volatile int*>(n_runs + 1);
+    const RunRef* runs = reinterpret_cast<const RunRef*>(n_runs + 4);
+    const bool ok = mbar_wait(smem_addr(&bars[C::kBarRuns]), 0, abort_flag);
+    if (!ok) {
+        if (!*abort_flag) set_error(a.err, kErrTimeout);
+        *abort_flag = 1;
+        *failed = 1;
+    }
+    named_bar_sync(1, kT);  // from here on every consumer sees the same
+    const int n = *failed ? 0 : *reinterpret_cast<const volatile int*>(n_runs);
+    // (the item-end rows have been read: their buffer takes the shares)
+    float4* x_o = reinterpret_cast<float4*>(smem + C::kOffOut);
+    float2* x_ml = reinterpret_cast<float2*>(x_o + kT);
+    static_assert(kT * 24 <= C::kOutBytes, "shares");
+    // kT / 2 outputs at a time
+    for (int b = 0; b < n * outs; b += kT / 2) {
+        const int x = b + tid % (kT / 2), share = tid / (kT / 2);
+        const bool on = x < n * outs;
+        MergeAcc acc;
+        RunRef run{};
+        int row = 0, c4 = 0;
+        if (on) {
+            run = runs[x / outs];
+            row = x % outs / kVec;
+            c4 = x % kVec;
+            acc = merge_share<D>(a, run, row, c4, share);
+            if (share) {
+                x_o[tid] = acc.o;
+                x_ml[tid] = make_float2(acc.M, acc.L);
             }
         }
         named_bar_sync(1, kT);
-        const int nl = *reinterpret_cast<volatile int*>(n_last);
-        for (int k = 0; k < nl;) {
-            // whole runs while they fit, else chunks of the one run
-            int k1 = k, ents = 0;
-            while (k1 < nl && ents + l_n[k1] <= cap && (k1 - k + 1) * outs_run <= kMergeOuts * kT)
-                ents += l_n[k1++];
-            const bool chunked = k1 == k;
-            if (chunked) k1 = k + 1;
-            const int n_chunk = chunked ? l_n[k] : 0;
-            float Mr[kMergeOuts], Lr[kMergeOuts], acc[kMergeOuts][4];
-#pragma unroll
-            for (int r = 0; r < kMergeOuts; ++r) {
-                Mr[r] = -INFINITY;
-                Lr[r] = 0.f;
-                acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
-            }
-            for (int c0 = 0; c0 < (chunked ? n_chunk : 1); c0 += cap) {
-                const int cn_chunk = chunked ? min(cap, n_chunk - c0) : 0;
-                // stage
-                uint32_t off = 0;
-                for (int q = k; q < k1; ++q) {
-                    const int cn = chunked ? cn_chunk : l_n[q];
-                    stage_run<D>(a, ring_s + off, l_e0[q], chunked ? c0 : 0, cn, tid);
-                    off += cn * ent_bytes;
-                }
-                cp_async_commit();
-                cp_async_wait<0>();
-                named_bar_sync(1, kT);
-                // merge this thread's outputs
-#pragma unroll
-                for (int r = 0; r < kMergeOuts; ++r) {
-                    const int o = tid + r * kT;
-                    if (o >= (k1 - k) * outs_run) continue;
-                    const int q = k + o / outs_run;
-                    const int row = (o % outs_run) / kVec, c4 = o % kVec;
-                    uint32_t base = 0;
-                    for (int t = k; t < q; ++t) base += l_n[t] * ent_bytes;
-                    const int cn = chunked ? cn_chunk : l_n[q];
-                    const float4* so = reinterpret_cast<const float4*>(ring + base);
-                    const float4* sm = so + cn * G * kVec;
-                    float bm = Mr[r];
-#pragma unroll 4
-                    for (int e = 0; e < cn; ++e) bm = fmaxf(bm, sm[e * G + row].x);
-                    const float bs = bm == -INFINITY ? 0.f : bm;
-                    const float sc = exp2f(Mr[r] - bs);
-                    Lr[r] *= sc;
-                    acc[r][0] *= sc; acc[r][1] *= sc; acc[r][2] *= sc; acc[r][3] *= sc;
-#pragma unroll 4
-                    for (int e = 0; e < cn; ++e) {
-                        const float4 ml = sm[e * G + row];
-                        const float w = exp2f(ml.x - bs);
-                        Lr[r] += w * ml.y;
-                        const float4 v = so[(e * G + row) * kVec + c4];
-                        acc[r][0] += w * v.x; acc[r][1] += w * v.y;
-                        acc[r][2] += w * v.z; acc[r][3] += w * v.w;
-                    }
-                    Mr[r] = bm;
-                }
-                named_bar_sync(1, kT);  // the staging is rewritten by the next round
-            }
-            // normalised outputs
-#pragma unroll
-            for (int r = 0; r < kMergeOuts; ++r) {
-                const int o = tid + r * kT;
-                if (o >= (k1 - k) * outs_run) continue;
-                const int q = k + o / outs_run;
-                const int row = (o % outs_run) / kVec, c4 = o % kVec;
-                const int rk = l_key[q];
-                const int i = rk / a.Hkv, h = (rk % a.Hkv) * G + row;
-                const float inv = 1.f / Lr[r];
-                const size_t ob = ((size_t)i * a.Hq + h) * D + c4 * 4;
-                if (a.out_f32) {
-                    *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + ob) = make_float4(
-                        acc[r][0] * inv, acc[r][1] * inv, acc[r][2] * inv, acc[r][3] * inv);
-                } else {
-                    uint2 u;
-                    u.x = pack_bf16x2(acc[r][0] * inv, acc[r][1] * inv);
-                    u.y = pack_bf16x2(acc[r][2] * inv, acc[r][3] * inv);
-                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + ob) = u;
-                }
-            }
-            k = k1;
+        if (on && !share) {
+            MergeAcc other;
+            const float2 ml = x_ml[tid + kT / 2];
+            other.M = ml.x;
+            other.L = ml.y;
+            other.o = x_o[tid + kT / 2];
+            merge_finish<D>(a, run, row, c4, acc, other);
         }
-        named_bar_sync(1, kT);  // the list is rewritten by the next batch of arrivals
+        named_bar_sync(1, kT);
     }
 }
 
 template <int D>
-__global__ void __launch_bounds__(DecCfg<D>::kThreads, 2)
-    sq_decode_splitk_kernel(const __grid_constant__ CUtensorMap tmap, const DecodeArgs a) {
+__global__ void __launch_bounds__(DecCfg<D>::kThreads, 1)
+    sq_decode_splitk_kernel(const __grid_constant__ CUtensorMap tmap,
+                            const __grid_constant__ DecodeArgs a) {
     using C = DecCfg<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * C::kStages);
-    float* merge = reinterpret_cast<float*>(smem + C::kStages * C::kStageBytes + 256);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + C::kBarRuns + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < C::kStages; ++s) {
-            mbar_init(smem_addr(&bars[s]), 1);
-            mbar_init(smem_addr(&bars[C::kStages + s]), kDecodeConsumerWarps);
-        }
+        // per group: full [kStages], empty [kStages]
+        for (int s = 0; s < kDecodeGroups * 2 * C::kStages; ++s)
+            mbar_init(smem_addr(&bars[s]),
+                      s / C::kStages % 2 ? kDecodeConsumerWarps / kDecodeGroups : 1);
+        mbar_init(smem_addr(&bars[C::kBarOut]), kDecodeConsumerWarps);
+        mbar_init(smem_addr(&bars[C::kBarOutFree]), C::kClosers / 32);
+        mbar_init(smem_addr(&bars[C::kBarRuns]), 1);
+        reinterpret_cast<int*>(smem + C::kOffRuns)[1] = 0;
         *abort_flag = 0;
         fence_mbar_init();
     }
-    // A reused plan is read before the wait: the producer keeps its item range
-    // and first stages in registers and warms L2 with the first stages' rows.
-    FastStart fs;
-    fs.n = 0;
-    fs.early = 0;
-    int p_it0 = 0, p_it1 = 0;
-    if (warp == kDecodeConsumerWarps && lane == 0) {
-        prefetch_tmap(&tmap);
-        if (a.plan_ready) {
-            p_it0 = a.cta_begin[blockIdx.x];
-            p_it1 = a.cta_begin[blockIdx.x + 1];
-            if (a.P >= kStageTokens && (int)blockIdx.x != a.debug_drop_cta)
-                fast_start(a, p_it0, p_it1, fs);
-            prefetch_first_stages<D>(&tmap, a, p_it0, p_it1);
-        }
+    const int group = warp - kDecodeConsumerWarps;
+    if (group >= 0 && group < kDecodeGroups) {
+        if (threadIdx.x == C::kConsumers) prefetch_tmap(&tmap);
+        Producer<D> pr{&tmap, a, smem + group * C::kStages * C::kStageBytes,
+                       bars + group * 2 * C::kStages, abort_flag, group, lane};
+        // A reused plan is read before the wait.  Pages no in-flight work writes
+        // (the host checked every library write to them is complete; the kernels
+        // before this one write no other pool memory) are loaded before it too:
+        // the first stages stream in while the previous kernel finishes.
+        if (a.plan_ready) pr.init();
+        named_bar_sync(2, C::kThreads);  // (the barriers are initialised)
+        if (a.plan_ready) pr.early();
+        grid_dependency_wait();
+        grid_launch_dependents();  // the next kernel may be scheduled as CTAs retire
+        if (!a.plan_ready) pr.init();
+        pr.run();
+        return;
     }
-    __syncthreads();
-    // Pages no in-flight work writes (the host checked every library write to
-    // them is complete; the kernels before this one write no other pool
-    // memory) may be loaded before the wait: the first stages stream in while
-    // the previous kernel finishes.  Stop at the first stage in a page that
-    // may still be written; the rest go out after the wait, in order.
-    if (warp == kDecodeConsumerWarps && lane == 0 && a.kv_early && fs.n > 0) {
-        for (int k = 0; k < fs.n; ++k) {
-            bool unsafe = false;
-            for (int u = 0; u < a.n_unsafe; ++u) unsafe |= a.unsafe[u] == fs.pid[k];
-            if (unsafe) break;
-            issue_fast_stage<D>(&tmap, a, fs, k, smem, bars);
-            fs.early = k + 1;
-        }
-    }
+    const bool closer = group >= kDecodeGroups;
+    const int j0 = (lane >> 2) / a.G, j1 = ((lane >> 2) + 8) / a.G;
+    int it0 = 0, it1 = 0;
+    ItemHead head{};
+    auto read_plan = [&]() {
+        it0 = a.cta_begin[blockIdx.x];
+        it1 = a.cta_begin[blockIdx.x + 1];
+        if (it0 < it1 && !closer) head.read(a, it0, j0, j1);
+    };
+    if (a.plan_ready) read_plan();
+    named_bar_sync(2, C::kThreads);
     // Launched as a programmatic dependent: the set-up above overlapped the
     // previous kernel's tail; nothing else it may have written is read before here.
     grid_dependency_wait();
-    grid_launch_dependents();  // the next kernel may be scheduled as CTAs retire
-    if (warp == kDecodeConsumerWarps) {
-        if (lane == 0) {
-            if (!a.plan_ready) {
-                p_it0 = a.cta_begin[blockIdx.x];
-                p_it1 = a.cta_begin[blockIdx.x + 1];
-            }
-            produce<D>(&tmap, a, p_it0, p_it1, fs, smem, bars, abort_flag);
-        }
+    grid_launch_dependents();
+    if (!a.plan_ready) read_plan();
+    if (it0 == it1) return;
+    if (closer) {
+        close_items<D>(a, it0, it1, smem, bars, abort_flag,
+                       threadIdx.x - C::kConsumers - kDecodeGroups * 32);
         return;
     }
-    const int it0 = a.cta_begin[blockIdx.x], it1 = a.cta_begin[blockIdx.x + 1];
-    consume<D>(a, it0, it1, smem, bars, abort_flag, merge, warp, lane);
-    // the ring and the merge buffers are free again (every stage consumed, the
-    // last item ended on a barrier)
-    arrive_and_merge<D>(a, it0, it1, smem, reinterpret_cast<int*>(merge), warp);
+    consume<D>(a, it0, it1, head, smem, bars, abort_flag, warp, lane);
+    merge_last_runs<D>(a, smem, bars, abort_flag, lane);
 }
 
 }  // namespace
@@ -879,7 +915,7 @@ static cudaError_t prepare_one() {
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          DecCfg<D>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    // the largest shared-memory carveout, so that two CTAs fit on an SM
+    // the largest shared-memory carveout
     return cudaFuncSetAttribute(sq_decode_splitk_kernel<D>,
                                 cudaFuncAttributePreferredSharedMemoryCarveout,
                                 cudaSharedmemCarveoutMaxShared);
