@@ -136,9 +136,10 @@ struct sq_cache {
     // prefill split-K partials, reused by every call (grown on demand)
     float* pre_part = nullptr;
     size_t pre_part_cap = 0;
-    cudaEvent_t pre_ev = nullptr;
-    bool pre_ev_recorded = false;
-    cudaStream_t pre_ev_stream = nullptr;
+    // the plan whose launches used them last: its event (recorded after its last
+    // launch, and ordered after the ones before whatever becomes of the entry)
+    // covers that use
+    PrefillPlanEntry* pre_last = nullptr;
     PlanEntry plans[kPlanCacheEntries];
     PrefillPlanEntry pre_plans[kPrefillPlanEntries];
     uint64_t use_clock = 0;
@@ -536,7 +537,6 @@ int sq_cache_destroy(sq_cache* c) {
     for (auto& w : c->write_pending) cudaEventDestroy(w.second);
     for (cudaEvent_t ev : c->write_events) cudaEventDestroy(ev);
     if (c->pre_part) cudaFree(c->pre_part);
-    if (c->pre_ev) cudaEventDestroy(c->pre_ev);
     if (c->d_err) cudaFree(c->d_err);
     if (c->own_pool) cudaFree(c->pool);
     delete c;
@@ -1228,22 +1228,17 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     if (plan.n_parts > 0) {
         const size_t need =
             (size_t)plan.n_parts * kPrefillQTiles * kPrefillRows * (g.D + 1) * sizeof(float);
-        if (!c->pre_ev) {
-            e = cudaEventCreateWithFlags(&c->pre_ev, cudaEventDisableTiming);
-            if (e != cudaSuccess) return cuda_status(e);
-        }
+        const PrefillPlanEntry* last = c->pre_last;
         if (need > c->pre_part_cap) {
-            if (c->pre_ev_recorded) cudaEventSynchronize(c->pre_ev);
+            if (last && last->ev_recorded) cudaEventSynchronize(last->ev);
             if (c->pre_part) cudaFree(c->pre_part);
             c->pre_part = nullptr;
             c->pre_part_cap = 0;
             e = cudaMalloc(&c->pre_part, need * 5 / 4);
             if (e != cudaSuccess) return cuda_status(e);
             c->pre_part_cap = need * 5 / 4;
-            c->pre_ev_recorded = false;
-        }
-        if (c->pre_ev_recorded && c->pre_ev_stream != st) {
-            e = cudaStreamWaitEvent(st, c->pre_ev, 0);
+        } else if (last && last->ev_recorded && last->ev_stream != st) {
+            e = cudaStreamWaitEvent(st, last->ev, 0);
             if (e != cudaSuccess) return cuda_status(e);
         }
     }
@@ -1307,10 +1302,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         ca.BP = plan.BP;
         e = launch_prefill_combine(ca, g.D, st);
         if (e != cudaSuccess) return cuda_status(e);
-        e = cudaEventRecord(c->pre_ev, st);
-        if (e != cudaSuccess) return cuda_status(e);
-        c->pre_ev_recorded = true;
-        c->pre_ev_stream = st;
+        c->pre_last = hit;
     }
     e = cudaEventRecord(hit->ev, st);
     if (e != cudaSuccess) return cuda_status(e);

@@ -267,10 +267,6 @@ int HostCache::evict(int32_t h, const int32_t* starts, const int32_t* ends,
     plan->ragged = ragged;
     plan->n_old = n;
     plan->n_new = n;
-    plan->old_pages = s->pages;
-    plan->old_fill = s->fill;
-    plan->new_pages = s->pages;
-    plan->new_fill = s->fill;
     if (n_spans == 0) return kOk;
     if (!starts || !ends) return kInvalidArg;
 
@@ -403,16 +399,18 @@ int HostCache::evict(int32_t h, const int32_t* starts, const int32_t* ends,
             q = w.qb + 1;
             ++wi;
         } else {
-            pages.push_back(s->pages[q]);
-            fill.push_back(s->fill[q]);
-            ++q;
+            const int32_t e = wi < win.size() ? win[wi].qa : np;  // up to the next window
+            pages.insert(pages.end(), s->pages.begin() + q, s->pages.begin() + e);
+            fill.insert(fill.end(), s->fill.begin() + q, s->fill.begin() + e);
+            q = e;
         }
     }
-    plan->new_pages = pages;
-    plan->new_fill = fill;
     plan->n_new = (int32_t)(n - removed);
     plan->evicted = (int32_t)removed;
     plan->windows = ragged ? (int32_t)win.size() : 1;
+    // the old table goes to the plan, for an undo
+    plan->old_pages = std::move(s->pages);
+    plan->old_fill = std::move(s->fill);
     s->pages = std::move(pages);
     s->fill = std::move(fill);
     s->n = plan->n_new;
@@ -429,7 +427,7 @@ void HostCache::undo_evict(int32_t h, const EvictPlan& plan) {
         if (alloc_.refcount(p) == 0) alloc_.take(p);
         else alloc_.add_ref(p);
     }
-    for (int32_t p : plan.new_pages) alloc_.drop_ref(p);
+    for (int32_t p : s->pages) alloc_.drop_ref(p);  // the table after
     s->pages = plan.old_pages;
     s->fill = plan.old_fill;
     s->n = plan.n_old;

@@ -126,8 +126,7 @@ struct EvictMove {
 struct EvictPlan {
     int32_t n_old = 0, n_new = 0;
     bool ragged = false;
-    std::vector<int32_t> old_pages, old_fill;   // page table before
-    std::vector<int32_t> new_pages, new_fill;   // page table after
+    std::vector<int32_t> old_pages, old_fill;   // page table before (rows removed: n_new < n_old)
     // Row movement in increasing destination (slot-space) order.  Every
     // source of a move lies at a slot-space position >= its destination's,
     // inside the same window, so performing the moves in order (each one's

@@ -57,3 +57,35 @@ def test_split_last_round(D, n, n_q):
         check_budget_rows(p, h, 0, q, out, spans, scale, rows)
     finally:
         p.close()
+
+
+def test_split_partials_across_streams():
+    # six split plans in four plan entries, on three streams in turn: the
+    # partials and the entries that every call shares pass from stream to stream
+    p = Pair(1, 8, 2, 64, 64, num_pages=6 * 70 + 4, seed=11)
+    try:
+        hs = [p.seq_new() for _ in range(6)]
+        for i, h in enumerate(hs):
+            p.append(h, 4000 + 37 * i)
+        g = torch.Generator(device="cuda").manual_seed(5)
+        q = torch.randn(6, 16, 8, 64, device="cuda", generator=g).to(torch.bfloat16)
+        n_q = [16, 9, 16, 3, 12, 16]
+
+        def one(i, out, stream):
+            p.cache.prefill_attention(hs[i], 0, n_q[i], q[i], out, sq.SQ_OUT_F32, None, 0.125,
+                                      (), stream)
+        want = torch.zeros(6, 16, 8, 64, device="cuda")
+        for i in range(6):
+            one(i, want[i], None)
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        order = [(7 * k + k // 5) % 6 for k in range(60)]
+        got = torch.zeros(len(order), 16, 8, 64, device="cuda")
+        torch.cuda.synchronize()
+        for k, i in enumerate(order):
+            one(i, got[k], streams[k % 3].cuda_stream)
+        torch.cuda.synchronize()
+        for k, i in enumerate(order):
+            assert torch.equal(got[k], want[i]), (k, i)
+    finally:
+        p.close()
