@@ -34,6 +34,15 @@ struct TraceRange {
 constexpr int kPlanCacheEntries = 8;
 constexpr int kUploadSlots = 8;
 
+// Write tickets of a plan's pages (fixed while the plan is valid: a write to a
+// page changes the version of every sequence holding it): the kMaxUnsafe
+// newest (ticket, page) pairs and the newest ticket of all other pages.
+// Writes known complete when the plan was made are left out.
+struct WriteTickets {
+    std::vector<std::pair<uint64_t, int32_t>> top;
+    uint64_t rest = 0;
+};
+
 struct PlanEntry {
     bool valid = false;
     int32_t n_ctas = 0;
@@ -42,12 +51,7 @@ struct PlanEntry {
     DecodePlanLayout lay{};
     int64_t unique_tokens = 0, logical_tokens = 0;
     int32_t first_busy_cta = 0;  // lowest CTA with work (target of the test hook)
-    // write tickets of the plan's pages (fixed while the plan is valid: a
-    // write to a page changes the version of every sequence holding it): the
-    // kDecodeMaxUnsafe newest (ticket, page) pairs and the newest ticket of
-    // all other pages
-    std::vector<std::pair<uint64_t, int32_t>> tick_top;
-    uint64_t tick_rest = 0;
+    WriteTickets writes;
     // per call-local sequence: the segment holding its last page when that
     // segment has it alone (else -1), the slot-space start of that run, and
     // the last page's entry in page_fill (plans with page fills)
@@ -76,6 +80,7 @@ struct PrefillPlanEntry {
     size_t o_items = 0, o_merges = 0, o_pages = 0;  // byte offsets of the parts of d
     int32_t n_tiles = 0, n_pieces = 0, BP = 0, n_items = 0, n_merges = 0, n_parts = 0;
     int64_t visible_pairs = 0;
+    WriteTickets writes;   // of the sequence's pages, as a decode plan has them
     uint8_t* d = nullptr;  // [tiles][items][merges][tile_pages]
     size_t cap = 0;
     cudaEvent_t ev = nullptr;  // recorded after the last launch that used it
@@ -307,6 +312,34 @@ void poll_writes(sq_cache* c) {
         c->write_events.push_back(c->write_pending.front().second);
         c->write_pending.pop_front();
     }
+}
+
+// The write tickets of a new plan's pages.
+void list_writes(sq_cache* c, const int32_t* pages, size_t n, WriteTickets* w) {
+    w->top.clear();
+    w->rest = 0;
+    for (size_t i = 0; i < n; ++i)
+        if (c->page_ticket[pages[i]] > c->write_done)
+            w->top.push_back({c->page_ticket[pages[i]], pages[i]});
+    if (w->top.size() <= (size_t)kMaxUnsafe) return;
+    std::partial_sort(w->top.begin(), w->top.begin() + kMaxUnsafe, w->top.end(),
+                      [](const std::pair<uint64_t, int32_t>& x,
+                         const std::pair<uint64_t, int32_t>& y) { return x.first > y.first; });
+    for (size_t i = kMaxUnsafe; i < w->top.size(); ++i) w->rest = std::max(w->rest, w->top[i].first);
+    w->top.resize(kMaxUnsafe);
+}
+
+// Whether every write to a plan's pages outside its newest few is complete: a
+// kernel may then load its first K/V before its dependency wait, except from
+// the pages whose writes may still be running (listed in `unsafe`).
+bool early_writes(sq_cache* c, const WriteTickets& w, int32_t* unsafe, int32_t* n_unsafe) {
+    *n_unsafe = 0;
+    if (!c->early_ok) return false;
+    poll_writes(c);
+    if (w.rest > c->write_done) return false;
+    for (const auto& tp : w.top)
+        if (tp.first > c->write_done) unsafe[(*n_unsafe)++] = tp.second;
+    return true;
 }
 
 // Asynchronous host -> device copy of `bytes` from `src` through a pinned
@@ -625,21 +658,21 @@ static void plan_len_apply(sq_cache* c, const LenUpdate& u, uint64_t new_version
     e.logical_tokens += n_new;
     const uint64_t t = c->page_ticket[page];
     bool found = false;
-    for (auto& tp : e.tick_top)
+    for (auto& tp : e.writes.top)
         if (tp.second == page) {
             tp.first = std::max(tp.first, t);
             found = true;
         }
     if (!found) {
-        e.tick_top.push_back({t, page});
-        if (e.tick_top.size() > (size_t)kDecodeMaxUnsafe) {
+        e.writes.top.push_back({t, page});
+        if (e.writes.top.size() > (size_t)kMaxUnsafe) {
             auto oldest = std::min_element(
-                e.tick_top.begin(), e.tick_top.end(),
+                e.writes.top.begin(), e.writes.top.end(),
                 [](const std::pair<uint64_t, int32_t>& x, const std::pair<uint64_t, int32_t>& y) {
                     return x.first < y.first;
                 });
-            e.tick_rest = std::max(e.tick_rest, oldest->first);
-            e.tick_top.erase(oldest);
+            e.writes.rest = std::max(e.writes.rest, oldest->first);
+            e.writes.top.erase(oldest);
         }
     }
     // the plan's buffer is written by this append: it is reused (or replaced)
@@ -919,18 +952,7 @@ int sq_decode_attention(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, int32_t
         while (victim->first_busy_cta + 1 < (int32_t)plan.cta_begin.size() &&
                plan.cta_begin[victim->first_busy_cta + 1] == plan.cta_begin[victim->first_busy_cta])
             ++victim->first_busy_cta;
-        {
-            std::vector<std::pair<uint64_t, int32_t>> tk(plan.page_ids.size());
-            for (size_t i = 0; i < tk.size(); ++i)
-                tk[i] = {c->page_ticket[plan.page_ids[i]], plan.page_ids[i]};
-            const size_t top = std::min<size_t>(kDecodeMaxUnsafe, tk.size());
-            std::partial_sort(tk.begin(), tk.begin() + top, tk.end(),
-                              [](const std::pair<uint64_t, int32_t>& x,
-                                 const std::pair<uint64_t, int32_t>& y) { return x.first > y.first; });
-            victim->tick_top.assign(tk.begin(), tk.begin() + top);
-            victim->tick_rest = 0;
-            for (size_t i = top; i < tk.size(); ++i) victim->tick_rest = std::max(victim->tick_rest, tk[i].first);
-        }
+        list_writes(c, plan.page_ids.data(), plan.page_ids.size(), &victim->writes);
         hit = victim;
     } else if (hit->ev_recorded && hit->ev_stream != st) {
         e = cudaStreamWaitEvent(st, hit->ev, 0);
@@ -966,20 +988,10 @@ int sq_decode_attention(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, int32_t
     a.num_pages = g.num_pages;
     a.scale_log2 = sm_scale * 1.4426950408889634f;
     a.debug_drop_cta = (c->debug_flags & SQ_DEBUG_DROP_DECODE_STAGE) ? hit->first_busy_cta : -1;
-    a.kv_early = 0;
-    a.n_unsafe = 0;
-    if (plan_ready && c->early_ok) {
-        // every write to the plan's pages outside its newest few is complete:
-        // the kernel may load its first stages before its dependency wait,
-        // except from the pages whose writes may still be running
-        poll_writes(c);
-        if (hit->tick_rest <= c->write_done) {
-            a.kv_early = 1;
-            for (const auto& tp : hit->tick_top)
-                if (tp.first > c->write_done) a.unsafe[a.n_unsafe++] = tp.second;
-            c->stats.decode_early_calls += 1;
-            c->stats.decode_early_held += a.n_unsafe;
-        }
+    a.kv_early = plan_ready && early_writes(c, hit->writes, a.unsafe, &a.n_unsafe) ? 1 : 0;
+    if (a.kv_early) {
+        c->stats.decode_early_calls += 1;
+        c->stats.decode_early_held += a.n_unsafe;
     }
     c->debug_flags &= ~SQ_DEBUG_DROP_DECODE_STAGE;
     a.err = c->d_err;
@@ -1214,6 +1226,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         victim->n_merges = (int32_t)plan.merges.size();
         victim->n_parts = plan.n_parts;
         victim->visible_pairs = plan.visible_pairs;
+        list_writes(c, s->pages.data(), s->pages.size(), &victim->writes);
         victim->valid = true;
         hit = victim;
     } else if (hit->ev_recorded && hit->ev_stream != st) {
@@ -1221,7 +1234,12 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         e = cudaStreamWaitEvent(st, hit->ev, 0);
         if (e != cudaSuccess) return cuda_status(e);
     } else {
-        plan_ready = 1;
+        // (a captured launch may run after any work, also work that writes what
+        // this one would read ahead of its dependency wait)
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(st, &capture);
+        if (e != cudaSuccess) return cuda_status(e);
+        plan_ready = capture == cudaStreamCaptureStatusNone;
     }
     hit->last_use = ++c->use_clock;
     const PrefillPlanEntry& plan = *hit;
@@ -1256,7 +1274,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return SQ_ERR_INVALID_ARG;
     }
-    PrefillArgs a;
+    PrefillShortArgs a;
     a.tiles = reinterpret_cast<const PrefillTile*>(plan.d);
     a.items = reinterpret_cast<const PrefillItem*>(plan.d + plan.o_items);
     a.tile_pages = reinterpret_cast<const int32_t*>(plan.d + plan.o_pages);
@@ -1273,6 +1291,11 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     a.BP = plan.BP;
     a.n_items = plan.n_items;
     a.plan_ready = plan_ready;
+    a.n_unsafe = 0;
+    a.kv_early = plan_ready && g.P >= kPrefillKeys / 2 &&
+                         early_writes(c, plan.writes, a.unsafe, &a.n_unsafe)
+                     ? 1
+                     : 0;
     // the kernel keeps the scale inside the exponent (s * scale - m); a zero
     // scale runs as 1e-30, whose weights 2^(s * 1e-30 - m) are exactly 1
     a.scale_log2 = std::max(sm_scale * 1.4426950408889634f, 1e-30f);
@@ -1300,6 +1323,8 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         ca.Hkv = g.Hkv;
         ca.G = g.G();
         ca.BP = plan.BP;
+        // (a call whose queries all fit in tile a has only their rows)
+        ca.rows = n_q <= plan.BP ? n_q * g.G() : kPrefillQTiles * kPrefillRows;
         e = launch_prefill_combine(ca, g.D, st);
         if (e != cudaSuccess) return cuda_status(e);
         c->pre_last = hit;

@@ -11,9 +11,9 @@
 namespace sq {
 
 // ---- decode attention -------------------------------------------------------
-// Pages whose K/V may still be being written when a decode call starts, at
+// Pages whose K/V may still be being written when an attention call starts, at
 // most this many per call (see DecodeArgs::kv_early).
-constexpr int kDecodeMaxUnsafe = 32;
+constexpr int kMaxUnsafe = 32;
 
 struct DecodeArgs {
     const DecodeSeg* segs;
@@ -42,7 +42,7 @@ struct DecodeArgs {
     // kernel's tail, up to its first stage in one of those pages
     int32_t kv_early;
     int32_t n_unsafe;
-    int32_t unsafe[kDecodeMaxUnsafe];
+    int32_t unsafe[kMaxUnsafe];
     int* err;
 };
 
@@ -76,6 +76,16 @@ struct PrefillArgs {
     int* err;
 };
 
+// The arguments of a call; those past the base concern calls whose queries fit
+// in one query tile (kept apart: the two-tile kernel, whose issuing lane is
+// bound by its instructions, ran 2% slower with them in its parameters).
+struct PrefillShortArgs : PrefillArgs {
+    // 1: as DecodeArgs::kv_early (plan_ready, pages of 64 tokens or more)
+    int32_t kv_early;
+    int32_t n_unsafe;
+    int32_t unsafe[kMaxUnsafe];
+};
+
 struct PrefillCombineArgs {
     const PrefillMerge* merges;
     int32_t n_merges;
@@ -85,6 +95,7 @@ struct PrefillCombineArgs {
     int32_t out_f32;
     float* lse;
     int32_t n_q, Hq, Hkv, G, BP;
+    int32_t rows;  // rows of a unit that can hold queries (of kPrefillQTiles * kPrefillRows)
 };
 
 // Dynamic shared memory of the prefill kernel.
@@ -92,7 +103,7 @@ int prefill_smem_bytes(int D);
 cudaError_t prefill_prepare(int D);
 // qmap: 3-D map of the queries {D, Hq, n_q}, box {64, G, BP}, 128-byte swizzle.
 cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
-                           const PrefillArgs& a, int D, cudaStream_t st);
+                           const PrefillShortArgs& a, int D, cudaStream_t st);
 cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStream_t st);
 
 // ---- append / copy-on-write / eviction --------------------------------------

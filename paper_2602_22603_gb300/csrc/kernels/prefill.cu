@@ -42,7 +42,7 @@
 //
 // Work items: the host lists (CTA tile, KV head, key range) items, longest
 // first, and the grid has one CTA per item, of which an SM holds one.  A CTA
-// that has issued the loads of its item asks the launch hardware for the next
+// that has issued most loads of its item asks the launch hardware for the next
 // CTA not started yet (clusterlaunchcontrol.try_cancel) and takes over its
 // item, so the ring, the barriers' phases and tensor memory run on from item
 // to item and the next item's first keys and queries load while the last one's
@@ -53,6 +53,17 @@
 // that would leave most SMs idle) leaves normalised partial results that a
 // second kernel merges.
 //
+// Calls whose queries fit in one query tile (kOne: the 8-query calls of an
+// auxiliary thread, every item dual-key) run an instance without the two-tile
+// path.  HBM bounds them, so, when the plan was on the device before, their
+// producer loads its item's first keys, up to the ring's depth, before the
+// dependency wait, while the previous launch's last CTAs finish and are merged:
+// 8 queries over 131,080 tokens, 87.0 -> 85.0 us a layer (79 at the read
+// probe's rate).  Loading early in the two-tile instance gained nothing (the
+// issuing lane bounds it) and lost 1 to 2% to the code generated around it; a
+// ring one slot longer (the second query tile's space), or L2 prefetches beyond
+// the ring, slow the CTAs still at work by more than they save the next ones.
+//
 // Warp roles (320 threads): warp 0 loads (lanes 0 and 1 issue the TMA copies,
 // two loads at a time), lane 0 of warp 1 issues the MMAs and warp 1 owns the
 // TMEM allocation, warps 2-5
@@ -60,6 +71,8 @@
 // reads TMEM lanes 32 (w mod 4) .. +31, one row per thread).  Every wait is
 // bounded; a wait that runs out sets the error word and the CTA winds down
 // after its copies and MMAs in flight have completed.
+#include <type_traits>
+
 #include "launch.hpp"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -73,7 +86,7 @@ namespace {
 constexpr int kItemSlots = 4;
 constexpr int kItemReaders = 9;
 
-template <int D>
+template <int D, bool kOne>
 struct PreCfg {
     static constexpr int kThreads = 320;
     static constexpr int kColBlocks = D / 64;                  // 64-column (128-byte) blocks
@@ -82,7 +95,7 @@ struct PreCfg {
     static constexpr int kSlotBytes = kColBlocks * kBlockBytes;  // 128 keys of K or of V
     static constexpr int kSlots = D == 128 ? 5 : 12;
     static constexpr int kOffQ = 0;
-    static constexpr int kOffRing = kOffQ + kPrefillQTiles * kQBytes;
+    static constexpr int kOffRing = kOffQ + (kOne ? 1 : kPrefillQTiles) * kQBytes;
     static constexpr int kOffBar = kOffRing + kSlots * kSlotBytes;
     static constexpr int kBarQ = 0;
     static constexpr int kBarFull = 1;                  // [kSlots] tile landed (V: and ready)
@@ -118,9 +131,9 @@ struct PreCfg {
 struct Smem {
     uint32_t base;  // shared address of the 1024-aligned region
     uint8_t* ptr;
-    template <int D>
+    template <int D, bool kOne>
     __device__ uint32_t bar(int i) const {
-        return base + PreCfg<D>::kOffBar + 8 * i;
+        return base + PreCfg<D, kOne>::kOffBar + 8 * i;
     }
 };
 
@@ -131,6 +144,7 @@ struct Item {
     bool dual;  // tile b takes every other key tile of tile a's rows
 };
 
+template <bool kOne>
 __device__ __forceinline__ Item make_item(const PrefillArgs& a, int4 raw) {
     Item it;
     const int qt = raw.x / a.Hkv;
@@ -140,7 +154,7 @@ __device__ __forceinline__ Item make_item(const PrefillArgs& a, int4 raw) {
     it.T = raw.z;
     it.part = raw.w;
     // tile b is empty when every query of the CTA tile fits in tile a
-    it.two = it.pos_lo + a.BP < a.n_q;
+    it.two = !kOne && it.pos_lo + a.BP < a.n_q;
     it.dual = !it.two && it.T >= 2;
     return it;
 }
@@ -173,17 +187,18 @@ __device__ __forceinline__ int clc_answer(uint32_t src) {
 
 // The reading side of the item ring: item k of the CTA is in slot k mod
 // kItemSlots until every reader has freed it.
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ bool item_wait(const Smem& sm, uint32_t k, const volatile int* abort_flag) {
-    return mbar_wait(sm.bar<D>(PreCfg<D>::kBarItem + k % kItemSlots), (k / kItemSlots) & 1, abort_flag);
+    return mbar_wait(sm.bar<D, kOne>(PreCfg<D, kOne>::kBarItem + k % kItemSlots),
+                     (k / kItemSlots) & 1, abort_flag);
 }
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ int4 item_read(const Smem& sm, uint32_t k) {
-    return *reinterpret_cast<const int4*>(sm.ptr + PreCfg<D>::kOffItems + k % kItemSlots * 16);
+    return *reinterpret_cast<const int4*>(sm.ptr + PreCfg<D, kOne>::kOffItems + k % kItemSlots * 16);
 }
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ void item_free(const Smem& sm, uint32_t k) {
-    mbar_arrive(sm.bar<D>(PreCfg<D>::kBarItemFree + k % kItemSlots));
+    mbar_arrive(sm.bar<D, kOne>(PreCfg<D, kOne>::kBarItemFree + k % kItemSlots));
 }
 
 // Bits 0 .. x of a word (x < 0: none; x >= 31: all).
@@ -238,6 +253,54 @@ struct FirstItem {
     }
 };
 
+// The first loads of a CTA's own item before the grid-dependency wait: pairs of
+// loads, as the producer's, as many as the ring takes and `limit` allows, up to
+// the first key tile with a page that may still be being written or with rows
+// past the sequence's end.  Returns the loads issued.
+template <int D, bool kOne>
+__device__ __forceinline__ int early_loads(const CUtensorMap* pool_map, const PrefillShortArgs& a,
+                                           const Smem& sm, const FirstItem& start, const Item& it,
+                                           int limit, int lane) {
+    using C = PreCfg<D, kOne>;
+    const int32_t unsafe = lane < a.n_unsafe ? a.unsafe[lane] : -1;
+    const int j_tail = it.t0 + it.T == a.n_tiles ? it.T - 1 : it.T;
+    int u0 = 0;
+    __syncwarp();  // (lane 0 initialised the barriers)
+    for (; u0 + 2 <= C::kSlots && u0 < limit; u0 += 2) {
+        int j0, kv0, j1, kv1;
+        load_of(u0, it.T, it.dual, j0, kv0);
+        load_of(u0 + 1, it.T, it.dual, j1, kv1);
+        const int j = (lane & 1) ? j1 : j0, kv = (lane & 1) ? kv1 : kv0;
+        const int key0 = __shfl_sync(0xffffffffu, start.rec.x, j);
+        const int pg0 = __shfl_sync(0xffffffffu, start.rec.y, j);
+        const int pg1 = __shfl_sync(0xffffffffu, start.rec.z, j);
+        const int key0b = __shfl_sync(0xffffffffu, start.rec.w, j);
+        bool safe = j < j_tail && (uint32_t)pg0 < (uint32_t)a.num_pages &&
+                    (uint32_t)pg1 < (uint32_t)a.num_pages;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {  // (lanes 0 and 1 hold the pair's pages)
+            const int p0 = __shfl_sync(0xffffffffu, pg0, x), p1 = __shfl_sync(0xffffffffu, pg1, x);
+            safe = safe && !(unsafe >= 0 && (unsafe == p0 || unsafe == p1));
+        }
+        if (!__all_sync(0xffffffffu, safe)) break;
+        if (lane < 2) {
+            const int slot = u0 + lane;
+            const uint32_t fb = sm.bar<D, kOne>(C::kBarFull + slot);
+            const uint32_t dst = sm.base + C::kOffRing + slot * C::kSlotBytes;
+            const int head_row = (kv ? a.Hkv + it.g : it.g) * a.P;
+            mbar_arrive_expect_tx(fb, C::kSlotBytes);
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int cb = 0; cb < C::kColBlocks; ++cb)
+                    tma_load_4d(dst + cb * C::kBlockBytes + b * 64 * 128, pool_map, fb, cb * 64,
+                                head_row + ((b ? key0b : key0) & (a.P - 1)), b ? pg1 : pg0, a.layer);
+        }
+    }
+    __syncwarp();
+    return u0;
+}
+
 // The producer warp, item by item: the query tiles, then the K and V tiles of
 // every key tile into the ring in the order of load_of, two loads at a time:
 // the whole warp waits for both slots, then lanes 0 and 1 arm their barriers
@@ -251,11 +314,11 @@ struct FirstItem {
 // moved into place a few tiles before it, an item's first batch while the item
 // before it runs.  Boxes past the second (pages of fewer than 64 tokens) take
 // their page from global memory.
-template <int D>
+template <int D, bool kOne>
 __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* qmap,
                                 const PrefillArgs& a, const Smem& sm, const FirstItem& start,
-                                volatile int* abort_flag, int lane) {
-    using C = PreCfg<D>;
+                                int u_early, volatile int* abort_flag, int lane) {
+    using C = PreCfg<D, kOne>;
     const int br = a.P < 64 ? a.P : 64;  // rows of one TMA box
     const int n_pieces = a.n_pieces;      // <= 16
     auto load_rec = [&](int t0, int T, int tb) { return tile_record(a, t0, T, tb, lane); };
@@ -265,28 +328,28 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
     uint32_t ub = 0;          // loads issued before this item (even)
     uint32_t n_queries = 0;   // items whose queries were loaded
     uint32_t n_fix = 0;       // uses of the fix-up barrier
-    uint32_t issued = 0;
+    uint32_t issued = u_early;
     // Slots are freed by the MMA warp's commits: one for every V tile, which
     // covers the K tile loaded right after it too, and one for each item's
     // first K tile; in dual-key mode one for every tile.  Bit i of `own`: the
     // load i + 1 before the next one has a commit of its own; bit s of `par`:
     // parity of slot s's next commit.
     uint32_t own = 0, par = 0;
-    uint32_t slot0 = 0;       // slot of the next load
+    uint32_t slot0 = u_early % C::kSlots;  // slot of the next load
     uint32_t tail_u = 0;      // the load that used the fix-up barrier last
     bool tail_open = false;   // ... and was not handed over on its slot's barrier
     bool ok = true;
     auto load_queries = [&](const Item& it) {
         if (n_queries > 0)
-            ok = mbar_wait(sm.bar<D>(C::kBarQFree), (n_queries - 1) & 1, abort_flag);
+            ok = mbar_wait(sm.bar<D, kOne>(C::kBarQFree), (n_queries - 1) & 1, abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         if (ok && lane == 0) {
             const int nq = it.two ? 2 : 1;  // tile b is loaded only when it holds queries
-            mbar_arrive_expect_tx(sm.bar<D>(C::kBarQ), nq * C::kColBlocks * a.BP * a.G * 128);
+            mbar_arrive_expect_tx(sm.bar<D, kOne>(C::kBarQ), nq * C::kColBlocks * a.BP * a.G * 128);
             for (int t = 0; t < nq; ++t)
                 for (int cb = 0; cb < C::kColBlocks; ++cb)
                     tma_load_3d(sm.base + C::kOffQ + t * C::kQBytes + cb * C::kBlockBytes, qmap,
-                                sm.bar<D>(C::kBarQ), cb * 64, it.g * a.G, it.pos_lo + t * a.BP);
+                                sm.bar<D, kOne>(C::kBarQ), cb * 64, it.g * a.G, it.pos_lo + t * a.BP);
         }
         if (ok) ++n_queries;
     };
@@ -295,26 +358,28 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
         const int slot = n_items % kItemSlots;
         if (n_items >= kItemSlots)
             ok = __all_sync(0xffffffffu,
-                            mbar_wait(sm.bar<D>(C::kBarItemFree + slot),
+                            mbar_wait(sm.bar<D, kOne>(C::kBarItemFree + slot),
                                       (n_items / kItemSlots - 1) & 1, abort_flag));
         if (ok && lane == 0) {
             *reinterpret_cast<int4*>(sm.ptr + C::kOffItems + slot * 16) = r;
-            mbar_arrive(sm.bar<D>(C::kBarItem + slot));
+            mbar_arrive(sm.bar<D, kOne>(C::kBarItem + slot));
         }
         if (ok) ++n_items;
     };
-    // The next item: requested when an item's first loads have gone out, taken in
-    // a few loads later, with its first batch of records.
+    // The next item: requested six key tiles before an item's end, as late as
+    // the answer and its records allow, so that the SMs that are ahead take the
+    // items left (asking with the first loads gave them out an item early: 3,001
+    // queries over 33,001 tokens 841 -> 835 us); taken in with the last loads.
     int4 next = make_int4(0, 0, -1, 0);
     auto request = [&]() {
         if (lane == 0) {
-            mbar_arrive_expect_tx(sm.bar<D>(C::kBarClc), 16);
-            clc_request(sm.base + C::kOffClc, sm.bar<D>(C::kBarClc));
+            mbar_arrive_expect_tx(sm.bar<D, kOne>(C::kBarClc), 16);
+            clc_request(sm.base + C::kOffClc, sm.bar<D, kOne>(C::kBarClc));
         }
         asked = true;
     };
     auto take_next = [&](uint32_t parity) {
-        ok = __all_sync(0xffffffffu, mbar_wait(sm.bar<D>(C::kBarClc), parity, abort_flag));
+        ok = __all_sync(0xffffffffu, mbar_wait(sm.bar<D, kOne>(C::kBarClc), parity, abort_flag));
         if (!ok) return;
         asked = false;
         const int cta = clc_answer(sm.base + C::kOffClc);
@@ -326,15 +391,19 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
         fence_proxy_async_smem();
         __syncwarp();
     };
+    if (u_early > 0)  // (`own` after the first loads, as the loop below keeps it)
+        own = make_item<kOne>(a, raw).dual ? (1u << u_early) - 1u
+                                     : (3u << (u_early - 2)) | (0x55555555u & ((1u << (u_early - 2)) - 1u));
     while (ok && raw.z >= 0) {
-        const Item it = make_item(a, raw);
+        const Item it = make_item<kOne>(a, raw);
         const uint32_t clc_parity = (n_items - 1) & 1;
         int4 rec = first, pend = first;
         const int T = it.T;
         const int n_units = 2 * T;
-        const int take_at = n_units > 10 ? 8 : n_units - 2;
+        const int take_at = n_units - 2, ask_at = n_units > 14 ? n_units - 12 : 0;
         const bool late_queries = ub > 0;
         if (T > 0 && !late_queries) load_queries(it);
+        if (u_early > ask_at) request();
         if (T == 0) {
             request();
             take_next(clc_parity);
@@ -343,7 +412,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
         int merge_b = -1;  // the batch read into `pend`, not yet in place
         // only the sequence's last key tile has rows past its end
         const int j_tail = it.t0 + T == a.n_tiles ? T - 1 : T;
-        for (int u0 = 0; ok && u0 < n_units; u0 += 2) {  // n_units is even
+        for (int u0 = u_early; ok && u0 < n_units; u0 += 2) {  // n_units is even
             int j0, kv0, j1, kv1;
             load_of(u0, T, it.dual, j0, kv0);
             load_of(u0 + 1, T, it.dual, j1, kv1);
@@ -369,12 +438,12 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
             // every lane polls the slots' barriers in turn: warp-uniform waits,
             // so no lane waits at the vote below for two polling lanes
             if (U0 >= C::kSlots && ((own >> (C::kSlots - 1)) & 1u)) {
-                ok = mbar_wait(sm.bar<D>(C::kBarEmpty + slot0), (par >> slot0) & 1u, abort_flag);
+                ok = mbar_wait(sm.bar<D, kOne>(C::kBarEmpty + slot0), (par >> slot0) & 1u, abort_flag);
                 par ^= 1u << slot0;
             }
             if (U0 + 1 >= C::kSlots && ((own >> (C::kSlots - 2)) & 1u)) {
                 if (ok)
-                    ok = mbar_wait(sm.bar<D>(C::kBarEmpty + slot1), (par >> slot1) & 1u, abort_flag);
+                    ok = mbar_wait(sm.bar<D, kOne>(C::kBarEmpty + slot1), (par >> slot1) & 1u, abort_flag);
                 par ^= 1u << slot1;
             }
             own = own << 2 | (it.dual || j0 == 0 ? 3u : 1u);  // K_j0, V_j1 but in dual-key mode
@@ -398,7 +467,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
             if (n_pieces == 2 && jmax < j_tail) {
                 // two whole boxes of 64 rows, as almost every tile has
                 if (lane < 2) {
-                    const uint32_t fb = sm.bar<D>(C::kBarFull + slot);
+                    const uint32_t fb = sm.bar<D, kOne>(C::kBarFull + slot);
                     mbar_arrive_expect_tx(fb, C::kSlotBytes);
                     load_box(fb, 0, key0, checked(pg0));
                     load_box(fb, 1, key0b, checked(pg1));
@@ -411,7 +480,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
                 const bool vfix = lane < 2 && kv == 1 && rows < kPrefillKeys;
                 if (lane < 2) {
                     const int nv = (rows + br - 1) / br;  // boxes inside the sequence (a prefix)
-                    const uint32_t fb = vfix ? sm.bar<D>(C::kBarVfix) : sm.bar<D>(C::kBarFull + slot);
+                    const uint32_t fb = vfix ? sm.bar<D, kOne>(C::kBarVfix) : sm.bar<D, kOne>(C::kBarFull + slot);
                     mbar_arrive_expect_tx(fb, (uint32_t)nv * br * 128 * C::kColBlocks);
                     const int half = n_pieces / 2;
 #pragma unroll 1
@@ -436,7 +505,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
                     tail_u = U0 + src;
                     tail_open = true;
                     issued = U0 + 2;
-                    if (lane == 0) ok = mbar_wait(sm.bar<D>(C::kBarVfix), n_fix & 1, abort_flag);
+                    if (lane == 0) ok = mbar_wait(sm.bar<D, kOne>(C::kBarVfix), n_fix & 1, abort_flag);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0);
                     if (!ok) break;
                     ++n_fix;
@@ -449,19 +518,18 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
                                 make_uint4(0, 0, 0, 0);
                     fence_proxy_async_smem();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(sm.bar<D>(C::kBarFull + fslot));
+                    if (lane == 0) mbar_arrive(sm.bar<D, kOne>(C::kBarFull + fslot));
                     tail_open = false;
                 }
             }
             issued = U0 + 2;
             slot0 = slot1 + 1 == C::kSlots ? 0 : slot1 + 1;
-            if (u0 == 0) {
-                request();
-                if (late_queries) load_queries(it);
-            }
+            if (u0 == ask_at) request();
+            if (u0 == 0 && late_queries) load_queries(it);
             if (ok && u0 == take_at) take_next(clc_parity);
         }
         ub += n_units;
+        u_early = 0;
         raw = next;
         if (ok) publish(raw);  // an item, or the end mark
     }
@@ -472,11 +540,11 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
     // Drain: every copy this CTA issued lands before the CTA exits (immediate
     // unless a consumer gave up early).
     if (lane == 0) {
-        if (asked) mbar_wait(sm.bar<D>(C::kBarClc), (n_items - 1) & 1);
-        if (n_queries > 0) mbar_wait(sm.bar<D>(C::kBarQ), (n_queries - 1) & 1);
+        if (asked) mbar_wait(sm.bar<D, kOne>(C::kBarClc), (n_items - 1) & 1);
+        if (n_queries > 0) mbar_wait(sm.bar<D, kOne>(C::kBarQ), (n_queries - 1) & 1);
         for (uint32_t u = issued > C::kSlots ? issued - C::kSlots : 0; u < issued; ++u) {
-            if (u == tail_u && tail_open) mbar_wait(sm.bar<D>(C::kBarVfix), n_fix & 1);
-            else mbar_wait(sm.bar<D>(C::kBarFull + u % C::kSlots), (u / C::kSlots) & 1);
+            if (u == tail_u && tail_open) mbar_wait(sm.bar<D, kOne>(C::kBarVfix), n_fix & 1);
+            else mbar_wait(sm.bar<D, kOne>(C::kBarFull + u % C::kSlots), (u / C::kSlots) & 1);
         }
     }
 }
@@ -489,9 +557,9 @@ struct MmaDesc {
     uint32_t k_hi, v_hi;      // high words (the queries' is the K tile's)
     uint32_t tmem;
 };
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ MmaDesc mma_desc(const Smem& sm, uint32_t tmem) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     static_assert(C::kBlockBytes == 16384, "the K-major steps' block stride");
     const uint64_t q = smem_desc_sw128(sm.base + C::kOffQ, 16, 1024);
     const uint64_t k = smem_desc_sw128(sm.base + C::kOffRing, 16, 1024);
@@ -509,17 +577,17 @@ __device__ __forceinline__ MmaDesc mma_desc(const Smem& sm, uint32_t tmem) {
 
 // S_t = Q_q K^T for the K tile in `slot`, into TMEM columns 128 t (q = t
 // except in dual-key mode, where both tiles use query tile 0).
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ void issue_qk(const MmaDesc& d, int t, int q, uint32_t slot) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     mma_bf16_ss_steps<D / 16>(d.tmem + C::kColS + (uint32_t)t * kPrefillKeys, d.q[q],
                               d.k + slot * (C::kSlotBytes >> 4), d.k_hi, C::kIdescQK);
 }
 
 // O_t += P_t V for the V tile in `slot`; P_t from TMEM over the first half of S_t.
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ void issue_pv(const MmaDesc& d, int t, uint32_t slot, bool first) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     static_assert(kPrefillKeys == 128, "8 steps of 16 keys");
     mma_bf16_ts_steps8(d.tmem + C::kColO + (uint32_t)t * 128,
                        d.tmem + C::kColS + (uint32_t)t * kPrefillKeys,
@@ -549,15 +617,15 @@ struct MmaPhase {
 // odd ones, and the two results are merged at the end.  Key tile j's PV and
 // the QK of key tile j + 2 (into the same S columns) are issued in the order
 // of the loads, each as soon as its tile has landed.
-template <int D>
+template <int D, bool kOne>
 __device__ bool prefill_mma_dual(const Smem& sm, const MmaDesc& d, int T, MmaPhase& ph,
                                  volatile int* abort_flag) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     // the tiles are used in the order of their loads: K_0, K_1, V_0, K_2, V_1, ...
     uint32_t slot = ph.slot, full = (ph.ub / C::kSlots) & 1;
-    auto landed = [&]() { return mbar_wait(sm.bar<D>(C::kBarFull + slot), full, abort_flag); };
+    auto landed = [&]() { return mbar_wait(sm.bar<D, kOne>(C::kBarFull + slot), full, abort_flag); };
     auto used = [&]() {
-        mma_commit(sm.bar<D>(C::kBarEmpty + slot));
+        mma_commit(sm.bar<D, kOne>(C::kBarEmpty + slot));
         if (++slot == C::kSlots) {
             slot = 0;
             full ^= 1;
@@ -566,28 +634,28 @@ __device__ bool prefill_mma_dual(const Smem& sm, const MmaDesc& d, int T, MmaPha
     for (int t = 0; t < 2; ++t) {
         // S_t = Q_a K_t
         if (!landed()) return false;
-        issue_qk<D>(d, t, 0, slot);
-        mma_commit(sm.bar<D>(C::kBarS + t));
+        issue_qk<D, kOne>(d, t, 0, slot);
+        mma_commit(sm.bar<D, kOne>(C::kBarS + t));
         used();
     }
-    if (T == 2) mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
+    if (T == 2) mma_commit(sm.bar<D, kOne>(C::kBarQFree));  // the item's last QK
     for (int j = 0; j < T; ++j) {
         const int t = j & 1;
         if (!landed()) return false;
-        if (!mbar_wait(sm.bar<D>(C::kBarP + t), (ph.p >> t) & 1, abort_flag)) return false;
+        if (!mbar_wait(sm.bar<D, kOne>(C::kBarP + t), (ph.p >> t) & 1, abort_flag)) return false;
         ph.p ^= 1u << t;
         tc_fence_after();
-        issue_pv<D>(d, t, slot, j < 2);
+        issue_pv<D, kOne>(d, t, slot, j < 2);
         used();
         if (j + 2 >= T) {  // the last key tile of tile t
-            mma_commit(sm.bar<D>(C::kBarO + t));
+            mma_commit(sm.bar<D, kOne>(C::kBarO + t));
             continue;
         }
         if (!landed()) return false;
-        issue_qk<D>(d, t, 0, slot);
-        mma_commit(sm.bar<D>(C::kBarS + t));
+        issue_qk<D, kOne>(d, t, 0, slot);
+        mma_commit(sm.bar<D, kOne>(C::kBarS + t));
         used();
-        if (j + 3 == T) mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
+        if (j + 3 == T) mma_commit(sm.bar<D, kOne>(C::kBarQFree));  // the item's last QK
     }
     ph.slot = slot;
     return true;
@@ -595,69 +663,69 @@ __device__ bool prefill_mma_dual(const Smem& sm, const MmaDesc& d, int T, MmaPha
 
 // One step of the two-tile path: O_t += P_t V_j, then S_t for the next key tile,
 // for tile a and then tile b.
-template <int D, bool kFirst, bool kMore>
+template <int D, bool kOne, bool kFirst, bool kMore>
 __device__ __forceinline__ bool prefill_mma_step(const Smem& sm, const MmaDesc& d, uint32_t vslot,
                                                  uint32_t kslot, uint32_t pa, uint32_t pb,
                                                  const volatile int* abort_flag) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-        if (!mbar_wait(sm.bar<D>(C::kBarP + t), t ? pb : pa, abort_flag)) return false;
+        if (!mbar_wait(sm.bar<D, kOne>(C::kBarP + t), t ? pb : pa, abort_flag)) return false;
         tc_fence_after();
-        issue_pv<D>(d, t, vslot, kFirst);
-        if (kMore) issue_qk<D>(d, t, t, kslot);
-        mma_commit(sm.bar<D>(kMore ? C::kBarS + t : C::kBarO + t));
+        issue_pv<D, kOne>(d, t, vslot, kFirst);
+        if (kMore) issue_qk<D, kOne>(d, t, t, kslot);
+        mma_commit(sm.bar<D, kOne>(kMore ? C::kBarS + t : C::kBarO + t));
     }
-    mma_commit(sm.bar<D>(C::kBarEmpty + vslot));  // V_j, and K_{j+1} with it
+    mma_commit(sm.bar<D, kOne>(C::kBarEmpty + vslot));  // V_j, and K_{j+1} with it
     return true;
 }
 
 // `two`: tile b holds query rows (false for an item of one key tile whose rows
 // all fit in tile a; tile b's products are then skipped).
-template <int D>
+template <int D, bool kOne>
 __device__ bool prefill_mma_item(const Smem& sm, const MmaDesc& d, int T, bool two, MmaPhase& ph,
                                  volatile int* abort_flag) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     auto after = [](uint32_t slot) { return slot + 1 == C::kSlots ? 0u : slot + 1; };
     uint32_t slot = ph.slot;
-    if (!mbar_wait(sm.bar<D>(C::kBarFull + slot), (ph.ub / C::kSlots) & 1, abort_flag)) return false;
-    issue_qk<D>(d, 0, 0, slot);
-    mma_commit(sm.bar<D>(C::kBarS + 0));
+    if (!mbar_wait(sm.bar<D, kOne>(C::kBarFull + slot), (ph.ub / C::kSlots) & 1, abort_flag)) return false;
+    issue_qk<D, kOne>(d, 0, 0, slot);
+    mma_commit(sm.bar<D, kOne>(C::kBarS + 0));
     if (two) {
-        issue_qk<D>(d, 1, 1, slot);
-        mma_commit(sm.bar<D>(C::kBarS + 1));
+        issue_qk<D, kOne>(d, 1, 1, slot);
+        mma_commit(sm.bar<D, kOne>(C::kBarS + 1));
     }
-    mma_commit(sm.bar<D>(C::kBarEmpty + slot));
+    mma_commit(sm.bar<D, kOne>(C::kBarEmpty + slot));
     uint32_t vslot = after(slot), kslot = after(vslot);
-    if (!two) {
-        mma_commit(sm.bar<D>(C::kBarQFree));
-        if (!mbar_wait(sm.bar<D>(C::kBarP + 0), ph.p & 1, abort_flag)) return false;
+    if (kOne || !two) {
+        mma_commit(sm.bar<D, kOne>(C::kBarQFree));
+        if (!mbar_wait(sm.bar<D, kOne>(C::kBarP + 0), ph.p & 1, abort_flag)) return false;
         tc_fence_after();
-        issue_pv<D>(d, 0, vslot, true);
-        mma_commit(sm.bar<D>(C::kBarO + 0));
-        mma_commit(sm.bar<D>(C::kBarEmpty + vslot));
+        issue_pv<D, kOne>(d, 0, vslot, true);
+        mma_commit(sm.bar<D, kOne>(C::kBarO + 0));
+        mma_commit(sm.bar<D, kOne>(C::kBarEmpty + vslot));
         ph.p ^= 1u;
         ph.slot = kslot;
         return true;
     }
     uint32_t pa = ph.p & 1, pb = (ph.p >> 1) & 1;
     if (T == 1) {
-        mma_commit(sm.bar<D>(C::kBarQFree));
-        if (!prefill_mma_step<D, true, false>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
+        mma_commit(sm.bar<D, kOne>(C::kBarQFree));
+        if (!prefill_mma_step<D, kOne, true, false>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
     } else {
-        if (!prefill_mma_step<D, true, true>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
+        if (!prefill_mma_step<D, kOne, true, true>(sm, d, vslot, kslot, pa, pb, abort_flag)) return false;
         for (int j = 1; j + 1 < T; ++j) {
             vslot = after(kslot);
             kslot = after(vslot);
             pa ^= 1;
             pb ^= 1;
-            if (!prefill_mma_step<D, false, true>(sm, d, vslot, kslot, pa, pb, abort_flag))
+            if (!prefill_mma_step<D, kOne, false, true>(sm, d, vslot, kslot, pa, pb, abort_flag))
                 return false;
         }
-        mma_commit(sm.bar<D>(C::kBarQFree));  // the item's last QK
+        mma_commit(sm.bar<D, kOne>(C::kBarQFree));  // the item's last QK
         vslot = after(kslot);
         kslot = after(vslot);
-        if (!prefill_mma_step<D, false, false>(sm, d, vslot, kslot, pa ^ 1, pb ^ 1, abort_flag))
+        if (!prefill_mma_step<D, kOne, false, false>(sm, d, vslot, kslot, pa ^ 1, pb ^ 1, abort_flag))
             return false;
     }
     ph.p ^= (T & 1) ? 3u : 0u;
@@ -669,26 +737,26 @@ __device__ bool prefill_mma_item(const Smem& sm, const MmaDesc& d, int T, bool t
 // while the softmax warps still write out this one's O: S has columns of its
 // own, and the first PV, which overwrites O, waits for a P that each softmax
 // thread hands over only after it has read its O.
-template <int D>
+template <int D, bool kOne>
 __device__ void prefill_mma(const PrefillArgs& a, const Smem& sm, uint32_t tmem,
                             volatile int* abort_flag) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     MmaPhase ph = {0, 0, 0, 0};
-    const MmaDesc d = mma_desc<D>(sm, tmem);
+    const MmaDesc d = mma_desc<D, kOne>(sm, tmem);
     bool ok = true, any = false;
     for (uint32_t k = 0;; ++k) {
-        if (!(ok = item_wait<D>(sm, k, abort_flag))) break;
-        const int4 raw = item_read<D>(sm, k);
-        item_free<D>(sm, k);
+        if (!(ok = item_wait<D, kOne>(sm, k, abort_flag))) break;
+        const int4 raw = item_read<D, kOne>(sm, k);
+        item_free<D, kOne>(sm, k);
         if (raw.z < 0) break;
         if (raw.z == 0) continue;
-        const Item it = make_item(a, raw);
-        if (!(ok = mbar_wait(sm.bar<D>(C::kBarQ), ph.q & 1, abort_flag))) break;
+        const Item it = make_item<kOne>(a, raw);
+        if (!(ok = mbar_wait(sm.bar<D, kOne>(C::kBarQ), ph.q & 1, abort_flag))) break;
         tc_fence_after();
         ++ph.q;
         any = true;
-        ok = it.dual ? prefill_mma_dual<D>(sm, d, it.T, ph, abort_flag)
-                     : prefill_mma_item<D>(sm, d, it.T, it.two, ph, abort_flag);
+        ok = it.dual ? prefill_mma_dual<D, kOne>(sm, d, it.T, ph, abort_flag)
+                     : prefill_mma_item<D, kOne>(sm, d, it.T, it.two, ph, abort_flag);
         if (!ok) break;
         ph.ub += 2 * it.T;
     }
@@ -698,8 +766,8 @@ __device__ void prefill_mma(const PrefillArgs& a, const Smem& sm, uint32_t tmem,
     }
     if (any) {
         // every MMA issued here completes before TMEM is released
-        mma_commit(sm.bar<D>(C::kBarDone));
-        mbar_wait(sm.bar<D>(C::kBarDone), 0);
+        mma_commit(sm.bar<D, kOne>(C::kBarDone));
+        mbar_wait(sm.bar<D, kOne>(C::kBarDone), 0);
     }
 }
 
@@ -748,11 +816,11 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const v
 
 // Normalises and writes one row of O_t (with tile b's part in dual-key mode) to
 // the outputs, or to the item's partial result.
-template <int D>
+template <int D, bool kOne>
 __device__ __forceinline__ void prefill_write(const PrefillArgs& a, const Item& it, uint32_t tl,
                                               uint32_t col_o, int t, int row, bool valid,
                                               float m_run, float l, float wa, float wb) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     const bool dual = it.dual, any_keys = it.T > 0;
     const int qi = it.pos_lo + (dual ? 0 : t) * a.BP + row / a.G;
     const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -825,14 +893,14 @@ constexpr uint32_t kParS = 1, kParO = 2, kParX = 4;  // S_t, O_t, dual-key excha
 
 // Softmax warpgroup of query tile t (one row per thread) and its epilogue,
 // for one item.  False: a wait ran out.
-template <int D>
+template <int D, bool kOne>
 __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t tmem, int t,
                                 uint32_t k, SoftmaxPhase& ph, volatile int* abort_flag, int warp,
                                 int lane) {
-    using C = PreCfg<D>;
+    using C = PreCfg<D, kOne>;
     const int wq = warp & 3;
     const int row = wq * 32 + lane;
-    const Item it = make_item(a, item_read<D>(sm, k));
+    const Item it = make_item<kOne>(a, item_read<D, kOne>(sm, k));
     const bool dual = it.dual;
     const int T_cta = it.T, t0 = it.t0;
     // dual-key mode: both tiles hold tile a's queries, tile t takes key tiles
@@ -847,16 +915,16 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
     // and O are never read back).
     if (!__any_sync(0xffffffffu, valid)) {
         for (int j = 0; j < T; ++j) {
-            if (!warp_wait(sm.bar<D>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
+            if (!warp_wait(sm.bar<D, kOne>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
             ph.par ^= kParS;
             tc_fence_before();
-            mbar_arrive(sm.bar<D>(C::kBarP + t));
+            mbar_arrive(sm.bar<D, kOne>(C::kBarP + t));
         }
         if (T > 0) ph.par ^= kParO;
         if (dual) {
-            mbar_arrive(sm.bar<D>(t == 1 ? C::kBarX : C::kBarXFree));
+            mbar_arrive(sm.bar<D, kOne>(t == 1 ? C::kBarX : C::kBarXFree));
             // (tile b's next P waits for tile a's reads also here)
-            if (t == 1 && !warp_wait(sm.bar<D>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag))
+            if (t == 1 && !warp_wait(sm.bar<D, kOne>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag))
                 return false;
             ph.par ^= kParX;
         }
@@ -888,7 +956,7 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
             nk = __ldg(reinterpret_cast<const int2*>(tp + kstep));
             nb = __ldg(&tp[kstep].key0b);
         }
-        if (!warp_wait(sm.bar<D>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
+        if (!warp_wait(sm.bar<D, kOne>(C::kBarS + t), ph.par & kParS, abort_flag)) return false;
         ph.par ^= kParS;
         tc_fence_after();
         // Raw logits q.k (the scale is applied inside the exponent; it is > 0),
@@ -1017,9 +1085,9 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
         uint32_t fv = 0, fk = 0, pv = 0, pk = 0;
         if (wq == 0 && t == 0 && !dual) {
             const uint32_t uv = ph.ub + 2 * j + 1, uk = uv + 1;
-            fv = sm.bar<D>(C::kBarFull + uv % C::kSlots);
+            fv = sm.bar<D, kOne>(C::kBarFull + uv % C::kSlots);
             pv = (uv / C::kSlots) & 1;
-            fk = j + 1 < T ? sm.bar<D>(C::kBarFull + uk % C::kSlots) : fv;
+            fk = j + 1 < T ? sm.bar<D, kOne>(C::kBarFull + uk % C::kSlots) : fv;
             pk = j + 1 < T ? (uk / C::kSlots) & 1 : pv;
             landed = mbar_try_wait(fv, pv) & mbar_try_wait(fk, pk);
         }
@@ -1030,11 +1098,11 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
             if (!warp_wait(fv, pv, abort_flag) || !warp_wait(fk, pk, abort_flag)) return false;
         }
         tc_fence_before();
-        mbar_arrive(sm.bar<D>(C::kBarP + t));
+        mbar_arrive(sm.bar<D, kOne>(C::kBarP + t));
         tp += kstep;
     }
     if (T > 0) {
-        if (!warp_wait(sm.bar<D>(C::kBarO + t), (ph.par & kParO) != 0, abort_flag)) return false;
+        if (!warp_wait(sm.bar<D, kOne>(C::kBarO + t), (ph.par & kParO) != 0, abort_flag)) return false;
         ph.par ^= kParO;
     }
     // dual-key mode: tile b hands its (max, normaliser) to tile a, which
@@ -1046,16 +1114,16 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
         xchg[2 * row] = m_run;
         xchg[2 * row + 1] = l;
         tc_fence_before();
-        mbar_arrive(sm.bar<D>(C::kBarX));
+        mbar_arrive(sm.bar<D, kOne>(C::kBarX));
         // tile b's next P (and with it the products that overwrite O_b) waits
         // until tile a has read O_b
-        if (!warp_wait(sm.bar<D>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag)) return false;
+        if (!warp_wait(sm.bar<D, kOne>(C::kBarXFree), (ph.par & kParX) != 0, abort_flag)) return false;
         ph.par ^= kParX;
         tc_fence_after();
         return true;
     }
     if (dual) {
-        if (!warp_wait(sm.bar<D>(C::kBarX), (ph.par & kParX) != 0, abort_flag)) return false;
+        if (!warp_wait(sm.bar<D, kOne>(C::kBarX), (ph.par & kParX) != 0, abort_flag)) return false;
         ph.par ^= kParX;
         tc_fence_after();
         const float mb = xchg[2 * row], lb = xchg[2 * row + 1];
@@ -1066,20 +1134,21 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
         m_run = M;
     }
     // the item again, from its slot
-    const int4 raw = item_read<D>(sm, k);
-    prefill_write<D>(a, make_item(a, raw), tl, col_o, t, row, valid, m_run, l, wa, wb);
+    const int4 raw = item_read<D, kOne>(sm, k);
+    prefill_write<D, kOne>(a, make_item<kOne>(a, raw), tl, col_o, t, row, valid, m_run, l, wa, wb);
     if (dual) {
         tc_fence_before();
-        mbar_arrive(sm.bar<D>(C::kBarXFree));
+        mbar_arrive(sm.bar<D, kOne>(C::kBarXFree));
     }
     return true;
 }
 
-template <int D>
+template <int D, typename Args>
 __global__ void __launch_bounds__(320, 1)
     sq_prefill_kernel(const __grid_constant__ CUtensorMap pool_map,
-                      const __grid_constant__ CUtensorMap qmap, const PrefillArgs a) {
-    using C = PreCfg<D>;
+                      const __grid_constant__ CUtensorMap qmap, const Args a) {
+    constexpr bool kOne = std::is_same<Args, PrefillShortArgs>::value;
+    using C = PreCfg<D, kOne>;
     extern __shared__ uint8_t smem_raw[];
     Smem sm;
     sm.ptr = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -1091,26 +1160,26 @@ __global__ void __launch_bounds__(320, 1)
     // the split-merging kernel that follows may be scheduled from here on
     grid_launch_dependents();
     if (threadIdx.x == 0) {
-        mbar_init(sm.bar<D>(C::kBarQ), 1);
+        mbar_init(sm.bar<D, kOne>(C::kBarQ), 1);
         for (int s = 0; s < C::kSlots; ++s) {
-            mbar_init(sm.bar<D>(C::kBarFull + s), 1);
-            mbar_init(sm.bar<D>(C::kBarEmpty + s), 1);
+            mbar_init(sm.bar<D, kOne>(C::kBarFull + s), 1);
+            mbar_init(sm.bar<D, kOne>(C::kBarEmpty + s), 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(sm.bar<D>(C::kBarS + b), 1);
-            mbar_init(sm.bar<D>(C::kBarP + b), 128);
-            mbar_init(sm.bar<D>(C::kBarO + b), 1);
+            mbar_init(sm.bar<D, kOne>(C::kBarS + b), 1);
+            mbar_init(sm.bar<D, kOne>(C::kBarP + b), 128);
+            mbar_init(sm.bar<D, kOne>(C::kBarO + b), 1);
         }
-        mbar_init(sm.bar<D>(C::kBarVfix), 1);
-        mbar_init(sm.bar<D>(C::kBarQFree), 1);
-        mbar_init(sm.bar<D>(C::kBarDone), 1);
+        mbar_init(sm.bar<D, kOne>(C::kBarVfix), 1);
+        mbar_init(sm.bar<D, kOne>(C::kBarQFree), 1);
+        mbar_init(sm.bar<D, kOne>(C::kBarDone), 1);
         for (int s = 0; s < kItemSlots; ++s) {
-            mbar_init(sm.bar<D>(C::kBarItem + s), 1);
-            mbar_init(sm.bar<D>(C::kBarItemFree + s), kItemReaders);
+            mbar_init(sm.bar<D, kOne>(C::kBarItem + s), 1);
+            mbar_init(sm.bar<D, kOne>(C::kBarItemFree + s), kItemReaders);
         }
-        mbar_init(sm.bar<D>(C::kBarClc), 1);
-        mbar_init(sm.bar<D>(C::kBarX), 128);
-        mbar_init(sm.bar<D>(C::kBarXFree), 128);
+        mbar_init(sm.bar<D, kOne>(C::kBarClc), 1);
+        mbar_init(sm.bar<D, kOne>(C::kBarX), 128);
+        mbar_init(sm.bar<D, kOne>(C::kBarXFree), 128);
         fence_mbar_init();
         *abort_flag = 0;
     }
@@ -1119,22 +1188,31 @@ __global__ void __launch_bounds__(320, 1)
         tmem_relinquish();
     }
     FirstItem start;
+    int u_early = 0;
     if (warp == 0) {
         if (lane == 0) {
             prefetch_tmap(&pool_map);
             prefetch_tmap(&qmap);
         }
         if (a.plan_ready) start.read(a, lane);
+        if constexpr (kOne) {
+            if (a.kv_early) {
+                const Item it = make_item<kOne>(a, start.raw);
+                // (the pair with which the next item is taken in stays with the loop)
+                u_early = early_loads<D, kOne>(&pool_map, a, sm, start, it, 2 * it.T - 2, lane);
+            }
+        }
     }
     // Launched as a programmatic dependent: the set-up above overlapped the
     // preceding kernel's tail; the queries and the pool, and a plan that was
-    // not on the device before that kernel, are read only from here on.
+    // not on the device before that kernel, are read only from here on (but for
+    // the first K/V tiles of early_loads).
     grid_dependency_wait();
     if (warp == 0) {
         if (!a.plan_ready) start.read(a, lane);
         if (lane == 0) {  // the thread that initialised the barriers
             *reinterpret_cast<int4*>(sm.ptr + C::kOffItems) = start.raw;
-            mbar_arrive(sm.bar<D>(C::kBarItem));
+            mbar_arrive(sm.bar<D, kOne>(C::kBarItem));
         }
     }
     tc_fence_before();
@@ -1142,27 +1220,27 @@ __global__ void __launch_bounds__(320, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     if (warp == 0) {
-        prefill_produce<D>(&pool_map, &qmap, a, sm, start, abort_flag, lane);
+        prefill_produce<D, kOne>(&pool_map, &qmap, a, sm, start, u_early, abort_flag, lane);
     } else if (warp == 1) {
-        if (lane == 0) prefill_mma<D>(a, sm, tmem, abort_flag);
+        if (lane == 0) prefill_mma<D, kOne>(a, sm, tmem, abort_flag);
         __syncwarp();
     } else {
         const int t = (warp - 2) >> 2;
         SoftmaxPhase ph = {0, 0};
         bool ok;
         for (uint32_t k = 0;; ++k) {
-            ok = __all_sync(0xffffffffu, item_wait<D>(sm, k, abort_flag));
+            ok = __all_sync(0xffffffffu, item_wait<D, kOne>(sm, k, abort_flag));
             if (!ok) break;
-            const int4 raw = item_read<D>(sm, k);
+            const int4 raw = item_read<D, kOne>(sm, k);
             if (raw.z < 0) break;
-            const Item it = make_item(a, raw);
+            const Item it = make_item<kOne>(a, raw);
             if (t == 0 || it.two || it.dual) {
-                ok = prefill_softmax<D>(a, sm, tmem, t, k, ph, abort_flag, warp, lane);
+                ok = prefill_softmax<D, kOne>(a, sm, tmem, t, k, ph, abort_flag, warp, lane);
                 if (!ok) break;
             }
             ph.ub += 2 * raw.z;
             __syncwarp();
-            if (lane == 0) item_free<D>(sm, k);
+            if (lane == 0) item_free<D, kOne>(sm, k);
         }
         if (!ok && lane == 0) {
             if (!*abort_flag) set_error(a.err, kErrTimeout);
@@ -1178,32 +1256,37 @@ __global__ void __launch_bounds__(320, 1)
 }
 
 // Merges the key-range splits of each query row: weights 2^(lse_s - max).
-// One warp per (split unit, query tile, row); the lanes take the splits' log-sum-
+// One warp per (split unit, row, 64 columns); the lanes take the splits' log-sum-
 // exps (up to 64 splits).  The partial outputs of the first 24 splits are
 // loaded together with them, so a row of up to 24 splits costs one round trip;
 // an empty split's partial (never written) is read but selected away.
+//
+// Two warps a row keep its loads in few registers, so that a batch of short
+// rows (an 8-query call: 256 rows of 19 splits) spreads over the SMs.  The
+// kernel lets the next one be scheduled at once: a next layer's prefill CTAs
+// take the SMs as this layer's leave.
+constexpr int kCombineThreads = 128;
 template <int D>
-__global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCombineArgs a) {
-    constexpr int V = D / 32;  // output elements per lane
+__global__ void __launch_bounds__(kCombineThreads, 6)
+    sq_prefill_combine_kernel(const PrefillCombineArgs a) {
+    constexpr int V = 2;        // output elements per lane
+    constexpr int kParts = D / (32 * V);
     constexpr int U = 24;      // splits per batch of loads
+    grid_launch_dependents();
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     constexpr int kRowsPerUnit = kPrefillQTiles * kPrefillRows;
-    if (gw >= a.n_merges * kRowsPerUnit) {
-        grid_dependency_wait();
-        return;
-    }
-    const int tr = gw % kRowsPerUnit;
+    const int m = gw / (a.rows * kParts);
+    if (m >= a.n_merges) return;
+    const int tr = (gw / kParts) % a.rows, col = (gw % kParts) * 32 * V + lane * V;
     // the plan was uploaded before the prefill kernel started
-    const PrefillMerge mg = a.merges[gw / kRowsPerUnit];
+    const PrefillMerge mg = a.merges[m];
     const int n_split = mg.n;
     const int t = tr / kPrefillRows, row = tr % kPrefillRows;
     const int qt = mg.unit / a.Hkv, g = mg.unit % a.Hkv;
     const int qi = (qt * kPrefillQTiles + t) * a.BP + row / a.G;
-    // programmatic dependent of the prefill kernel: wait for its partials;
-    // the next layer's prefill may then be scheduled
+    // programmatic dependent of the prefill kernel: wait for its partials
     grid_dependency_wait();
-    grid_launch_dependents();
     if (row >= a.BP * a.G || qi >= a.n_q) return;
     const int h = g * a.G + row % a.G;
     // partial row of split s: part0 + s * kRowsPerUnit
@@ -1211,23 +1294,15 @@ __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCo
     const float ml0 = lane < n_split ? a.part_ml[part0 + (size_t)lane * kRowsPerUnit] : -INFINITY;
     const float ml1 =
         lane + 32 < n_split ? a.part_ml[part0 + (size_t)(lane + 32) * kRowsPerUnit] : -INFINITY;
-    float vals[U][V];
+    float2 vals[U];
     auto load = [&](int s0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int s = s0 + u;  // the same in every lane
-#pragma unroll
-            for (int e = 0; e < V; ++e) vals[u][e] = 0.f;
-            if (s < n_split) {
-                const float* po = a.part_o + (part0 + (size_t)s * kRowsPerUnit) * D + lane * V;
-                if constexpr (V == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(po);
-                    vals[u][0] = v.x; vals[u][1] = v.y; vals[u][2] = v.z; vals[u][3] = v.w;
-                } else {
-                    const float2 v = *reinterpret_cast<const float2*>(po);
-                    vals[u][0] = v.x; vals[u][1] = v.y;
-                }
-            }
+            vals[u] = make_float2(0.f, 0.f);
+            if (s < n_split)
+                vals[u] = *reinterpret_cast<const float2*>(
+                    a.part_o + (part0 + (size_t)s * kRowsPerUnit) * D + col);
         }
     };
     load(0);
@@ -1242,9 +1317,7 @@ __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCo
     float W = w0 + w1;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) W += __shfl_xor_sync(0xffffffffu, W, off);
-    float acc[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) acc[e] = 0.f;
+    float acc[V] = {0.f, 0.f};
     for (int s0 = 0; W > 0.f && s0 < n_split; s0 += U) {
         if (s0 > 0) load(s0);
 #pragma unroll
@@ -1252,54 +1325,50 @@ __global__ void __launch_bounds__(256) sq_prefill_combine_kernel(const PrefillCo
             const int s = s0 + u;
             const float ws = __shfl_sync(0xffffffffu, s < 32 ? w0 : w1, s & 31);
             if (s < n_split && ws > 0.f) {
-#pragma unroll
-                for (int e = 0; e < V; ++e) acc[e] += ws * vals[u][e];
+                acc[0] += ws * vals[u].x;
+                acc[1] += ws * vals[u].y;
             }
         }
     }
     const float inv = W > 0.f ? 1.f / W : 0.f;
-    const size_t o = ((size_t)qi * a.Hq + h) * D + lane * V;
-    if (a.out_f32) {
-        float* out = reinterpret_cast<float*>(a.out) + o;
-        if constexpr (V == 4)
-            *reinterpret_cast<float4*>(out) =
-                make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
-        else
-            *reinterpret_cast<float2*>(out) = make_float2(acc[0] * inv, acc[1] * inv);
-    } else {
-        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + o;
-        if constexpr (V == 4) {
-            uint2 u;
-            u.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
-            u.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-            *reinterpret_cast<uint2*>(out) = u;
-        } else {
-            *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
-        }
-    }
-    if (lane == 0 && a.lse)
+    const size_t o = ((size_t)qi * a.Hq + h) * D + col;
+    if (a.out_f32)
+        *reinterpret_cast<float2*>(reinterpret_cast<float*>(a.out) + o) =
+            make_float2(acc[0] * inv, acc[1] * inv);
+    else
+        *reinterpret_cast<uint32_t*>(reinterpret_cast<__nv_bfloat16*>(a.out) + o) =
+            pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    if (lane == 0 && col == 0 && a.lse)
         a.lse[(size_t)qi * a.Hq + h] = W > 0.f ? (M + __log2f(W)) * 0.69314718055994531f : -INFINITY;
 }
 
 }  // namespace
 }  // namespace dev
 
-int prefill_smem_bytes(int D) {
-    return D == 128 ? dev::PreCfg<128>::kSmemBytes : dev::PreCfg<64>::kSmemBytes;
+template <int D>
+static cudaError_t prepare() {
+    cudaError_t e = cudaFuncSetAttribute(dev::sq_prefill_kernel<D, PrefillArgs>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         dev::PreCfg<D, false>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(dev::sq_prefill_kernel<D, PrefillShortArgs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             dev::PreCfg<D, true>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    // the same split of L1 and shared memory as the prefill kernel's: the two
+    // take turns on every SM
+    return cudaFuncSetAttribute(dev::sq_prefill_combine_kernel<D>,
+                                cudaFuncAttributePreferredSharedMemoryCarveout,
+                                cudaSharedmemCarveoutMaxShared);
 }
 
-cudaError_t prefill_prepare(int D) {
-    if (D == 128)
-        return cudaFuncSetAttribute(dev::sq_prefill_kernel<128>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    dev::PreCfg<128>::kSmemBytes);
-    return cudaFuncSetAttribute(dev::sq_prefill_kernel<64>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                dev::PreCfg<64>::kSmemBytes);
+int prefill_smem_bytes(int D) {
+    return D == 128 ? dev::PreCfg<128, false>::kSmemBytes : dev::PreCfg<64, false>::kSmemBytes;
 }
+
+cudaError_t prefill_prepare(int D) { return D == 128 ? prepare<128>() : prepare<64>(); }
 
 cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
-                           const PrefillArgs& a, int D, cudaStream_t st) {
+                           const PrefillShortArgs& a, int D, cudaStream_t st) {
     const unsigned grid = (unsigned)a.n_items;
     if (grid == 0) return cudaSuccess;
     // a programmatic dependent of whatever precedes it: its barrier and tensor
@@ -1312,19 +1381,25 @@ cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    if (D == 128) {
-        cfg.blockDim = dim3(dev::PreCfg<128>::kThreads);
-        cfg.dynamicSmemBytes = dev::PreCfg<128>::kSmemBytes;
-        return cudaLaunchKernelEx(&cfg, dev::sq_prefill_kernel<128>, pool_map, qmap, a);
-    }
-    cfg.blockDim = dim3(dev::PreCfg<64>::kThreads);
-    cfg.dynamicSmemBytes = dev::PreCfg<64>::kSmemBytes;
-    return cudaLaunchKernelEx(&cfg, dev::sq_prefill_kernel<64>, pool_map, qmap, a);
+    auto launch = [&](auto cfg_of, auto kernel, const auto& args) {
+        using C = decltype(cfg_of);
+        cfg.blockDim = dim3(C::kThreads);
+        cfg.dynamicSmemBytes = C::kSmemBytes;
+        return cudaLaunchKernelEx(&cfg, kernel, pool_map, qmap, args);
+    };
+    const PrefillArgs& base = a;
+    const bool one = a.n_q <= a.BP;  // every query in tile a of the only CTA tile
+    if (D == 128)
+        return one ? launch(dev::PreCfg<128, true>{}, dev::sq_prefill_kernel<128, PrefillShortArgs>, a)
+                   : launch(dev::PreCfg<128, false>{}, dev::sq_prefill_kernel<128, PrefillArgs>, base);
+    return one ? launch(dev::PreCfg<64, true>{}, dev::sq_prefill_kernel<64, PrefillShortArgs>, a)
+               : launch(dev::PreCfg<64, false>{}, dev::sq_prefill_kernel<64, PrefillArgs>, base);
 }
 
 cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStream_t st) {
-    const int64_t warps = (int64_t)a.n_merges * kPrefillQTiles * kPrefillRows;
-    const unsigned grid = (unsigned)((warps * 32 + 255) / 256);
+    const int64_t warps = (int64_t)a.n_merges * a.rows * (D / 64);
+    const int per = dev::kCombineThreads / 32;
+    const unsigned grid = (unsigned)((warps + per - 1) / per);
     if (grid == 0) return cudaSuccess;
     // scheduled while the prefill kernel's last CTAs run; waits for them
     cudaLaunchAttribute at;
@@ -1332,7 +1407,7 @@ cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStrea
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(dev::kCombineThreads);
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;

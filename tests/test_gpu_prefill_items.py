@@ -89,3 +89,97 @@ def test_split_partials_across_streams():
             assert torch.equal(got[k], want[i]), (k, i)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("D,P,n,new,n_q,grow", [
+    (128, 64, 9000, 3000, 8, True),     # one tile of queries, keys split over the SMs
+    (128, 64, 9000, 40, 8, False),
+    (64, 128, 5000, 1000, 12, True),
+    (128, 256, 300, 200, 150, True),    # few key tiles: the ring holds an item's all
+    (64, 64, 100, 1, 1, False),         # one key tile
+    (128, 64, 6000, 2500, 2500, True),  # two-tile items, several per SM
+    (64, 32, 3000, 600, 9, True),       # small pages: nothing is loaded early
+])
+def test_layers_right_after_appends(D, P, n, new, n_q, grow):
+    """The calls after the first reuse its plan and load keys before the work
+    before them is done: never from pages whose rows are still being written."""
+    L = 3
+    p = Pair(L, 8, 2, D, P, num_pages=6 * ((n + 8 * new) // P + 4), seed=n + new)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(n)
+
+        def rand(*shape):
+            return torch.randn(*shape, device="cuda", generator=g).to(torch.bfloat16)
+        kv = [(rand(L, m, 2, D), rand(L, m, 2, D)) for m in [n] + [new] * 8]
+        q = rand(8, L, n_q, 8, D)
+        filler = rand(L, 20000, 2, D)   # (keeps the stream busy while the calls are issued)
+        spare = sq.Cache(L, 8, 2, D, 64, 340)
+
+        def steps(sync):
+            h = p.cache.seq_new()
+            p.cache.append_kv(h, n, *kv[0])
+            outs = []
+            for i in range(8):
+                if not sync:
+                    x = spare.seq_new()
+                    spare.append_kv(x, 20000, filler, filler)
+                    spare.release(x)
+                target = h if grow else p.cache.fork_aux(h)
+                p.cache.append_kv(target, new, *kv[1 + i])
+                for layer in range(L):
+                    out = torch.empty(n_q, 8, D, device="cuda")
+                    if sync:
+                        torch.cuda.synchronize()
+                    p.cache.prefill_attention(target, layer, n_q, q[i, layer], out, sq.SQ_OUT_F32,
+                                              None, 0.1, ())
+                    outs.append(out)
+                if not grow:
+                    p.cache.release(target)
+            p.cache.release(h)
+            torch.cuda.synchronize()
+            assert p.cache.sync_status() == sq.SQ_OK
+            return outs
+        want, got = steps(True), steps(False)
+        for i, (x, y) in enumerate(zip(want, got)):
+            assert torch.isfinite(x).all() and torch.equal(x, y), (i // L, i % L)
+        spare.close()
+    finally:
+        p.close()
+
+
+def test_prefill_replayed_from_a_cuda_graph():
+    p = Pair(2, 8, 2, 128, 64, num_pages=200, seed=3)
+    try:
+        h, other = p.seq_new(), p.seq_new()
+        p.append(h, 6000)
+        q = torch.zeros(2, 16, 8, 128, dtype=torch.bfloat16, device="cuda")
+        outs = torch.zeros(2, 16, 8, 128, device="cuda")
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+
+        def layers():
+            for layer in range(2):
+                p.cache.prefill_attention(h, layer, 16, q[layer], outs[layer], sq.SQ_OUT_F32, None,
+                                          0.1, ())
+        qs = [torch.randn(2, 16, 8, 128, device="cuda").to(torch.bfloat16) for _ in range(3)]
+        want = []
+        with torch.cuda.stream(s):
+            for x in qs:
+                q.copy_(x)
+                layers()
+                want.append(outs.clone())
+            p.append(other, 100)   # a write that no call has found complete yet
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            layers()
+        for x, w in zip(qs, want):
+            q.copy_(x)
+            outs.fill_(float("nan"))
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.isfinite(w).all() and torch.equal(outs, w)
+        assert p.cache.sync_status() == sq.SQ_OK
+        del g
+    finally:
+        p.close()
