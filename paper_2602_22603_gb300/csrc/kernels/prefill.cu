@@ -26,7 +26,8 @@
 // warpgroup may rescale O_t then without another wait.  The running maximum
 // is raised lazily: a key tile's weights are taken with the current maximum
 // and accepted while every row's sum of them stays at most 2^16 (so does each
-// weight); only then is a maximum raised and O rescaled.  K and V stream through
+// weight; 2^8 in warps with rows that are no query); only then is a maximum
+// raised and O rescaled.  K and V stream through
 // one ring of shared-memory slots (K_0, V_0, K_1, ...); V_j and K_{j+1} are
 // released together, after the products PV_b(j) and S_b(j+1).
 //
@@ -938,6 +939,14 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
     const uint32_t col_s = C::kColS + (uint32_t)t * kPrefillKeys;
     const uint32_t col_o = C::kColO + (uint32_t)t * 128;
     const float sc = a.scale_log2;  // > 0 (the host raises a zero scale to a tiny one)
+    // most that a row's weights of one tile may sum to without a look at their
+    // maximum (a power of two above the running one).  A warp with rows that are
+    // no query raises its maxima where a weight passes 2^8, as such warps did
+    // when every tile of theirs took the path with the maximum: the largest
+    // weight of a row is then more often exactly 1, and not rounded (with 2^16
+    // the log-sum-exp of 3 queries over 9,892 tokens was off by 2.4e-5 instead
+    // of 1.3e-5 of its size).
+    const float accept = __all_sync(0xffffffffu, valid) ? 65536.f : 256.f;
     float m_run = -INFINITY, l = 0.f;
     // {first keys, flags} of the next key tile; its visibility bits are read
     // only where a tile is masked (they would hold eight registers of the loop)
@@ -1009,7 +1018,7 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
         };
         // The maximum is raised lazily, so most tiles keep it: take the
         // weights with the current maximum and accept them when no row's sum
-        // exceeds 2^16, which bounds every weight; no maximum is needed for
+        // exceeds `accept`, which bounds every weight; no maximum is needed for
         // that.  Otherwise (or when a row has seen no key yet) find the tile's
         // maximum and redo the tile with it wherever it exceeds the running
         // one by more than 2^8.
@@ -1017,7 +1026,7 @@ __device__ bool prefill_softmax(const PrefillArgs& a, const Smem& sm, uint32_t t
         bool done = false;
         if (__all_sync(0xffffffffu, m_run != -INFINITY || !valid)) {
             weights(m_run, tsum);
-            done = !__any_sync(0xffffffffu, valid && tsum > 65536.f);
+            done = !__any_sync(0xffffffffu, valid && tsum > accept);
         }
         if (!done) {
             // row maximum: three-input max over four independent chains

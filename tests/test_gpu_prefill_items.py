@@ -183,3 +183,41 @@ def test_prefill_replayed_from_a_cuda_graph():
         del g
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,n,n_q,rise", [
+    (320, 160, 1000, 3, 9.0),      # 6 rows of a warp hold queries
+    (320, 160, 1000, 3, 15.0),
+    (480, 160, 1000, 200, 12.0),   # G = 3: two rows of every tile hold none
+])
+def test_dominant_key_in_a_partly_filled_warp(Hq, Hkv, n, n_q, rise):
+    """A key of an item's later tiles whose weight passes the running maximum
+    by 2^9 .. 2^15 sets the maximum in warps with rows that are no query, so its
+    weight is exactly 1 and the log-sum-exp is off by the rounding of the other
+    weights alone: n of them, 2^-rise each, every one off by an independent 2^-9
+    at most, so by less than 6 sqrt(n) 2^-rise 2^-9 together.  Rounded to bf16
+    the large weight itself (2^(rise + 0.40625)) would be off by 0.0022."""
+    p = Pair(1, Hq, Hkv, 64, 64, num_pages=n // 64 + 4, seed=1)
+    try:
+        h = p.seq_new()
+        scale = math.log(2.0)      # logits in powers of two
+        k = torch.zeros(1, n, Hkv, 64, dtype=torch.bfloat16, device="cuda")
+        k[..., 1] = 0.11 * torch.randn(n, device="cuda").to(torch.bfloat16)[None, :, None]
+        k[0, 700 if n_q < 10 else 500, :, 0] = rise + 0.40625   # (not near a power of two)
+        v = torch.randn(1, n, Hkv, 64, device="cuda").to(torch.bfloat16)
+        p.cache.append_kv(h, n, k, v)
+        q = torch.zeros(n_q, Hq, 64, dtype=torch.bfloat16, device="cuda")
+        q[..., :2] = 1
+        out = torch.empty(n_q, Hq, 64, device="cuda")
+        lse = torch.empty(n_q, Hq, device="cuda")
+        p.cache.prefill_attention(h, 0, n_q, q, out, sq.SQ_OUT_F32, lse, scale, ())
+        x = (k[0, :, 0, 0].double() + k[0, :, 0, 1].double()) * scale
+        want = torch.stack([torch.logsumexp(x[:n - n_q + i + 1], 0) for i in range(n_q)])
+        # the queries of the warp of 32 rows that ends a tile of BP positions
+        bp = 128 // (Hq // Hkv)
+        at = [i for i in range(n_q) if n_q < bp or i % bp >= 96 * Hkv // Hq]
+        assert at
+        err = (lse.double() - want[:, None]).abs()[at].max().item()
+        assert err <= 6 * math.sqrt(n) * 2.0 ** (-rise - 9) + 2e-5, err
+    finally:
+        p.close()
