@@ -23,13 +23,17 @@
 // item's partial and merge what it completes.
 //
 // What bounds it: HBM in long calls (the read probe's rate at 128k); in short
-// ones the chain after the last stage (add, partial, arrival, merge, ~6 us) and
-// the start.  Two CTAs per SM with the same ring space, each closing its items
-// itself, left twice the entries per run and stalled at every item's end.  Per
-// call at 32q/8kv, d = 128, before and after: one sequence of 32,768 tokens
-// 27.5 and 25.1 us, 36 sequences of 250 .. 6,000 tokens 51.4 and 47.0 us, four
-// agents and their forks at 20,000 .. 60,000 tokens with partial pages 54.6 and
-// 46.4 us; eight of 131,072 and their forks 604 us either way.
+// ones the chain after the last stage (add, partial, arrival, merge: 5 us from
+// the slowest CTA's last stage to the next call's start) and the SMs' unequal
+// shares of HBM (2 us between most and the slowest).  Two CTAs per SM with the
+// same ring space, each closing its items itself, left twice the entries per
+// run and stalled at every item's end.  Per call at 32q/8kv, d = 128, so and
+// now: one sequence of 32,768 tokens 27.5 and 24.6 us, 36 sequences of 250 ..
+// 6,000 tokens 51.4 and 46.4 us, four agents and their forks at 20,000 ..
+// 60,000 tokens with partial pages 54.6 and 45.6 us; eight of 131,072 and their
+// forks 600 us either way.  Prefetching stages past the ring into L2 while the
+// previous call ends gains nothing: 6 instead of 4 stages 795 -> 810 us for 32
+// layers of the 32k sequence.
 //
 // Merge: an item leaves one partial (max, sum, unnormalised output) per group
 // member, in that (sequence, KV head)'s contiguous run of entries; a member
@@ -296,6 +300,62 @@ __device__ __forceinline__ int out_pos(int row, int col) {
     return row * D + ((((col >> 3) ^ row) & (D / 8 - 1)) << 3) + (col & 7);
 }
 
+// Four consecutive output elements from element `at`: v * inv.
+__device__ __forceinline__ void write_out(const DecodeArgs& a, size_t at, const float4& v, float inv) {
+    if (a.out_f32) {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + at) =
+            make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+    } else {
+        uint2 u;
+        u.x = pack_bf16x2(v.x * inv, v.y * inv);
+        u.y = pack_bf16x2(v.z * inv, v.w * inv);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + at) = u;
+    }
+}
+
+// Adds the consumer warps' rows rb .. rb + 7 of an item (weights 2^(m_w - M),
+// warps in order) and writes its partials or outputs: `n` threads, `v0` = which.
+template <int D>
+__device__ __forceinline__ void close_rows(const DecodeArgs& a, const DecodeItem* item,
+                                           const DecodeSeg* seg, int head, int sole, int rows, int rb,
+                                           const uint8_t* smem, int v0, int n) {
+    using C = DecCfg<D>;
+    constexpr int kVec = D / 4;  // float4 per output row
+    const int G = a.G;
+    const float* red_m = reinterpret_cast<const float*>(smem + C::kOffRed);
+    const float* red_l = red_m + kDecodeConsumerWarps * kRowsPerTile;
+    const float* red_o = reinterpret_cast<const float*>(smem + C::kOffOut);
+    const int n_out = min(rows - rb, (int)C::kPassRows) * kVec;
+    for (int v = v0; v < n_out; v += n) {
+        const int pr = v / kVec, c4 = v % kVec, r = rb + pr, j = r / G;
+        // a member whose run is this item alone gets its normalised output
+        const bool alone = (sole >> j) & 1;
+        const int to = alone ? seg->grp_seq[j] : item->ent[j];
+        float M = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kDecodeConsumerWarps; ++w) M = fmaxf(M, red_m[w * kRowsPerTile + r]);
+        const float Ms = M == -INFINITY ? 0.f : M;
+        float L = 0.f;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < kDecodeConsumerWarps; ++w) {
+            const float f = exp2f(red_m[w * kRowsPerTile + r] - Ms);
+            L += red_l[w * kRowsPerTile + r] * f;
+            const float4 x =
+                *reinterpret_cast<const float4*>(red_o + w * C::kPassRows * D + out_pos<D>(pr, c4 * 4));
+            sum.x += x.x * f; sum.y += x.y * f; sum.z += x.z * f; sum.w += x.w * f;
+        }
+        if (alone) {
+            write_out(a, ((size_t)to * a.Hq + head * G + r % G) * D + c4 * 4, sum, 1.f / L);
+        } else {
+            const size_t pe = (size_t)to * G + r % G;
+            *reinterpret_cast<float4*>(a.part_o + pe * D + c4 * 4) = sum;
+            if (c4 == 0)
+                *reinterpret_cast<float4*>(a.part_ml + pe * 4) = make_float4(M, L, 0.f, 0.f);
+        }
+    }
+}
+
 template <int D>
 __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, uint8_t* smem,
                         uint64_t* all_bars, volatile int* abort_flag, int warp, int lane) {
@@ -503,9 +563,10 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, ui
         l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
         l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
         const int rows = n_grp * G;
+        const bool last = it + 1 == it1;
         for (int rb = 0; rb < rows; rb += C::kPassRows, ++n_pass) {
             // the previous pass's rows have been read
-            if (!dead && n_pass > 0) {
+            if (!dead && n_pass > 0 && !(last && rb > 0)) {
                 const bool ok =
                     mbar_wait(smem_addr(&all_bars[C::kBarOutFree]), (n_pass - 1) & 1, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) {
@@ -514,7 +575,7 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, ui
                     dead = true;
                 }
             }
-            if (dead) continue;
+            if (dead && !last) continue;
             const int r = rb + gid;  // this lane's row of the pass: r0, then r1
             if (tig == 0) {
                 red_m[warp * kRowsPerTile + r] = rb ? m1 : m0;
@@ -527,8 +588,20 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, ui
                     *reinterpret_cast<float2*>(wo + out_pos<D>(gid, nd * 8 + tig * 2)) =
                         rb ? make_float2(o[nd][2], o[nd][3]) : make_float2(o[nd][0], o[nd][1]);
             }
+            if (last) {
+                // nothing is left to stream: the consumers add the rows themselves
+                // (every warp gets here, also after a wait ran out)
+                const int sole = a.items[it].sole;
+                named_bar_sync(1, C::kConsumers);
+                close_rows<D>(a, a.items + it, seg, item.head, sole, rows, rb, smem, threadIdx.x,
+                              C::kConsumers);
+                if (rb + C::kPassRows < rows) {
+                    named_bar_sync(1, C::kConsumers);
+                    continue;
+                }
+            }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_addr(&all_bars[C::kBarOut]));
+            if (lane == 0 && !dead) mbar_arrive(smem_addr(&all_bars[C::kBarOut]));
         }
     }
 }
@@ -538,28 +611,32 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, ui
 // the consumer warps' rows (weights 2^(m_w - M), warps in order), write the
 // item's partials or outputs, arrive on the runs it belongs to and merge those
 // it completes.  (With the consumers doing this between items, a batch of 36
-// short sequences, ~3 items per CTA, stalled at every end: 51 us per call
-// against TODO.)  The runs that the CTA's last item completes are merged by the
-// consumers, which have nothing else to do by then.
+// short sequences, ~3 items per CTA, stalled at every end: 51.4 us per call
+// against 46.9.)  Of a CTA's last item the consumers add and write the rows
+// themselves and merge the runs it completes, since nothing is left to stream;
+// the closing warps only arrive.  That shortens the chain after the last stage,
+// which a call cannot hide: one sequence of 32,768 tokens 25.1 -> 24.6 us per
+// call, the 36 short ones 46.9 -> 46.4.
 //
 // The arrival word of a run holds two counts.  Its low half counts the items
-// that finished (a relaxed add, the claim); the claim that brings it to the
+// that finished (an acquire add, the claim); the claim that brings it to the
 // run's length makes its CTA the merger.  Every other CTA then publishes its
 // partial with a release add to the high half, and the merger, instead of
 // releasing its own partial first (a GPU-scope fence on its critical path),
-// waits with acquire loads until the high half counts the other entries (their
-// claims came first, so their releases are under way: the wait depends on
-// nothing this CTA still has to do); its own partial it reads back within the
-// CTA.  The merger sets the word back to zero.  Every CTA claims once per
+// reads whether the high half counts the other entries: in the claim's own
+// answer, as a rule (the last one to finish), else in acquire loads until it
+// does (their claims came first, so their releases are under way: the wait
+// depends on nothing this CTA still has to do); its own partial it reads back
+// within the CTA.  The merger sets the word back to zero.  Every CTA claims once per
 // (item, group member), also after a wait ran out, so every call leaves every
 // word at zero, and a plan upload writes zeros; the word therefore always
 // starts a call at zero.  A run holds at most 65,535 entries (the planner's
 // limit), so the halves never carry.
 
 // GPU-scope atomics of the arrival protocol.
-__device__ __forceinline__ unsigned atom_add_relaxed_gpu(unsigned* p, unsigned v) {
+__device__ __forceinline__ unsigned atom_add_acquire_gpu(unsigned* p, unsigned v) {
     unsigned old;
-    asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    asm volatile("atom.acquire.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
 __device__ __forceinline__ void red_add_release_gpu(unsigned* p, unsigned v) {
@@ -569,19 +646,6 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-
-// Four consecutive output elements from element `at`: v * inv.
-__device__ __forceinline__ void write_out(const DecodeArgs& a, size_t at, const float4& v, float inv) {
-    if (a.out_f32) {
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + at) =
-            make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
-    } else {
-        uint2 u;
-        u.x = pack_bf16x2(v.x * inv, v.y * inv);
-        u.y = pack_bf16x2(v.z * inv, v.w * inv);
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + at) = u;
-    }
 }
 
 // (max, sum, weighted output) of one output float4.
@@ -674,9 +738,6 @@ __device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem
     using C = DecCfg<D>;
     constexpr int kVec = D / 4;  // float4 per output row
     const int G = a.G, lane = et & 31;
-    const float* red_m = reinterpret_cast<const float*>(smem + C::kOffRed);
-    const float* red_l = red_m + kDecodeConsumerWarps * kRowsPerTile;
-    const float* red_o = reinterpret_cast<const float*>(smem + C::kOffOut);
     int* n_runs = reinterpret_cast<int*>(smem + C::kOffRuns);
     RunRef* runs = reinterpret_cast<RunRef*>(n_runs + 4);
     uint32_t n_pass = 0;
@@ -706,36 +767,8 @@ __device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem
                 }
             }
             if (dead) continue;
-            const int n_out = min(rows - rb, (int)C::kPassRows) * kVec;
-            for (int v = et; v < n_out; v += C::kClosers) {
-                const int pr = v / kVec, c4 = v % kVec, r = rb + pr;
-                float M = -INFINITY;
-#pragma unroll
-                for (int w = 0; w < kDecodeConsumerWarps; ++w)
-                    M = fmaxf(M, red_m[w * kRowsPerTile + r]);
-                const float Ms = M == -INFINITY ? 0.f : M;
-                float L = 0.f;
-                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int w = 0; w < kDecodeConsumerWarps; ++w) {
-                    const float f = exp2f(red_m[w * kRowsPerTile + r] - Ms);
-                    L += red_l[w * kRowsPerTile + r] * f;
-                    const float4 x = *reinterpret_cast<const float4*>(
-                        red_o + w * C::kPassRows * D + out_pos<D>(pr, c4 * 4));
-                    sum.x += x.x * f; sum.y += x.y * f; sum.z += x.z * f; sum.w += x.w * f;
-                }
-                // a member whose run is this item alone gets its normalised output
-                const int j = r / G;
-                if ((sole >> j) & 1) {
-                    write_out(a, ((size_t)seg->grp_seq[j] * a.Hq + head * G + r % G) * D + c4 * 4, sum,
-                              1.f / L);
-                } else {
-                    const size_t pe = (size_t)item->ent[j] * G + r % G;
-                    *reinterpret_cast<float4*>(a.part_o + pe * D + c4 * 4) = sum;
-                    if (c4 == 0)
-                        *reinterpret_cast<float4*>(a.part_ml + pe * 4) = make_float4(M, L, 0.f, 0.f);
-                }
-            }
+            if (it + 1 == it1) break;  // the consumers have added and written its rows
+            close_rows<D>(a, item, seg, head, sole, rows, rb, smem, et, C::kClosers);
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_addr(&bars[C::kBarOutFree]));
         }
@@ -744,11 +777,11 @@ __device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem
         if (et < 32) {
             bool merger = false;
             if (key >= 0) {
-                const unsigned old = atom_add_relaxed_gpu(a.arrive + key, 1u);
+                const unsigned old = atom_add_acquire_gpu(a.arrive + key, 1u);
                 merger = (old & 0xffffu) + 1u == (unsigned)mine.n;
                 if (!merger) {
                     red_add_release_gpu(a.arrive + key, 0x10000u);
-                } else {
+                } else if ((old >> 16) != (unsigned)(mine.n - 1)) {
                     const uint64_t t0 = globaltimer_ns();
                     for (uint32_t spin = 1;; ++spin) {
                         if ((ld_acquire_gpu(a.arrive + key) >> 16) == (unsigned)(mine.n - 1)) break;
@@ -757,8 +790,8 @@ __device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem
                             break;
                         }
                     }
-                    a.arrive[key] = 0u;
                 }
+                if (merger) a.arrive[key] = 0u;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, merger);
             if (merger) runs[__popc(mask & ((1u << lane) - 1u))] = mine;
