@@ -1045,36 +1045,49 @@ int evict_impl(sq_cache* c, sq_seq seq, const sq_span* spans, int32_t n_spans, v
         const int64_t resident = c->evict_resident;
         const int32_t max_chunks = (int32_t)std::max<int64_t>(1, 4 * resident / planes);
         evict_chunks(window_tile, (int32_t)tiles.size(), max_chunks, 4, &chunk);
-        const size_t tb = tiles.size() * sizeof(EvictTile);
-        const size_t pcb = pieces.size() * sizeof(EvictPiece);
-        std::vector<uint8_t> buf(tb + pcb + chunk.size() * sizeof(int32_t));
-        std::memcpy(buf.data(), tiles.data(), tb);
-        std::memcpy(buf.data() + tb, pieces.data(), pcb);
-        std::memcpy(buf.data() + tb + pcb, chunk.data(), chunk.size() * sizeof(int32_t));
-        UploadSlot& s = c->slots[c->next_slot];
-        c->next_slot = (c->next_slot + 1) % kUploadSlots;
-        rc = upload(c, s, buf.data(), buf.size(), stream);
-        if (rc != SQ_OK) return undo(rc);
-        EvictArgs ea;
+        EvictInlineArgs ea;
         ea.pool = c->pool;
         ea.num_pages = g.num_pages;
         ea.L = g.L; ea.Hkv = g.Hkv; ea.P = g.P; ea.D = g.D;
-        ea.tiles = reinterpret_cast<const EvictTile*>(s.d);
-        ea.pieces = reinterpret_cast<const EvictPiece*>(s.d + tb);
         ea.n_tiles = (int32_t)tiles.size();
         ea.n_pieces = (int32_t)pieces.size();
         ea.tile_rows = c->evict_tile_rows;
         ea.stages = c->evict_stages;
         ea.zero_tiles = plan.zeroed_rows > 0 ? 1 : 0;
         ea.n_chunks = (int32_t)chunk.size() - 1;
-        ea.chunk = ea.n_chunks > 1 ? reinterpret_cast<const int32_t*>(s.d + tb + pcb) : nullptr;
+        ea.tiles = nullptr;
+        ea.pieces = nullptr;
+        ea.chunk = nullptr;
         ea.err = c->d_err;
-        cudaError_t e = launch_evict(ea, st);
-        if (e != cudaSuccess) return undo(cuda_status(e));
-        e = cudaEventRecord(s.ev, st);
-        if (e != cudaSuccess) return cuda_status(e);
-        s.ev_recorded = true;
-        s.ev_stream = st;
+        const size_t tb = tiles.size() * sizeof(EvictTile);
+        const size_t pcb = pieces.size() * sizeof(EvictPiece);
+        const size_t cb = chunk.size() * sizeof(int32_t);
+        if (tiles.size() + pieces.size() <= (size_t)kEvictInline &&
+            ea.n_chunks <= kEvictInlineChunks) {
+            std::memcpy(ea.rec, tiles.data(), tb);
+            std::memcpy(ea.rec + tiles.size(), pieces.data(), pcb);
+            std::memcpy(ea.inline_chunk, chunk.data(), cb);
+            cudaError_t e = launch_evict_inline(ea, st);
+            if (e != cudaSuccess) return undo(cuda_status(e));
+        } else {
+            std::vector<uint8_t> buf(tb + pcb + cb);
+            std::memcpy(buf.data(), tiles.data(), tb);
+            std::memcpy(buf.data() + tb, pieces.data(), pcb);
+            std::memcpy(buf.data() + tb + pcb, chunk.data(), cb);
+            UploadSlot& s = c->slots[c->next_slot];
+            c->next_slot = (c->next_slot + 1) % kUploadSlots;
+            rc = upload(c, s, buf.data(), buf.size(), stream);
+            if (rc != SQ_OK) return undo(rc);
+            ea.tiles = reinterpret_cast<const EvictTile*>(s.d);
+            ea.pieces = reinterpret_cast<const EvictPiece*>(s.d + tb);
+            ea.chunk = reinterpret_cast<const int32_t*>(s.d + tb + pcb);
+            cudaError_t e = launch_evict(ea, st);
+            if (e != cudaSuccess) return undo(cuda_status(e));
+            e = cudaEventRecord(s.ev, st);
+            if (e != cudaSuccess) return cuda_status(e);
+            s.ev_recorded = true;
+            s.ev_stream = st;
+        }
         std::vector<int32_t> written;
         for (const EvictMove& m : plan.moves)
             if (written.empty() || written.back() != m.dst_page) written.push_back(m.dst_page);

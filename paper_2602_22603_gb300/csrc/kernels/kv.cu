@@ -4,6 +4,9 @@
 // Pool layout: [L][num_pages][2 (K, V)][Hkv][P][D] bf16, so the rows of one
 // (layer, page, K/V, head) are P*D contiguous elements and one token row is
 // D*2 bytes.  Appends move 16-byte vectors, evictions whole runs of rows.
+#include <algorithm>
+#include <type_traits>
+
 #include "launch.hpp"
 #include "ptx.cuh"
 
@@ -200,8 +203,35 @@ __global__ void __launch_bounds__(kAppendThreads)
 // zeros: the unused slots of a page that a ragged eviction leaves partial.  Its store reads a zero tile that the
 // CTA's warp clears once; it writes only past the rows its window kept, and
 // later tiles read only later windows' pages.
-template <int S>  // ring slots
-__global__ void __launch_bounds__(32) sq_evict_compact_kernel(const EvictArgs a) {
+//
+// What bounds it: latency.  A CTA moves a few tiles, and every record it reads
+// from memory is a round trip ahead of its first load.  A plan of up to
+// kEvictInline records therefore comes with the launch's arguments (read from
+// the constant bank, with no upload before the launch): 25 spans of a context
+// of 98,304 tokens, 8 layers of 8 heads, d = 128: 29.7 -> 24.8 us, the call with
+// its fork and release 39.8 -> 33.8 us (the 115 MB moved allow 17).  Longer
+// plans than fit the 4 KB of arguments are read from memory: their CTAs move
+// many tiles each, which hides the records' latency.
+template <int S, typename Args>  // ring slots; EvictArgs or EvictInlineArgs
+__global__ void __launch_bounds__(32)
+    sq_evict_compact_kernel(const __grid_constant__ Args a) {
+    constexpr bool kInline = std::is_same<Args, EvictInlineArgs>::value;
+    auto tile_at = [&](int g) {
+        int4 r;
+        if constexpr (kInline) r = a.rec[g];
+        else r = __ldg(reinterpret_cast<const int4*>(a.tiles) + g);
+        return EvictTile{r.x, r.y, r.z, r.w};
+    };
+    auto piece_at = [&](int k) {
+        int4 r;
+        if constexpr (kInline) r = a.rec[a.n_tiles + k];
+        else r = __ldg(reinterpret_cast<const int4*>(a.pieces) + k);
+        return EvictPiece{r.x, r.y, r.z, r.w};
+    };
+    auto chunk_at = [&](int c) {
+        if constexpr (kInline) return a.inline_chunk[c];
+        else return __ldg(&a.chunk[c]);
+    };
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -220,8 +250,8 @@ __global__ void __launch_bounds__(32) sq_evict_compact_kernel(const EvictArgs a)
     const int planes = a.L * 2 * a.Hkv;
     const int plane = blockIdx.x % planes;
     const int ch = blockIdx.x / planes;
-    const int tb = a.chunk ? __ldg(&a.chunk[ch]) : 0;
-    const int te = a.chunk ? __ldg(&a.chunk[ch + 1]) : a.n_tiles;
+    const int tb = a.n_chunks > 1 ? chunk_at(ch) : 0;
+    const int te = a.n_chunks > 1 ? chunk_at(ch + 1) : a.n_tiles;
     if (tb < 0 || te > a.n_tiles || tb > te) {
         set_error(a.err, kErrBounds);
         return;
@@ -240,11 +270,11 @@ __global__ void __launch_bounds__(32) sq_evict_compact_kernel(const EvictArgs a)
         const int g = tb + t;
         const uint32_t bar = smem_addr(&full[slot]);
         const uint32_t dst0 = smem_addr(smem + slot * tile_bytes);
-        const int pb = __ldg(&a.tiles[g].piece_begin);
-        const int pe = g + 1 < a.n_tiles ? __ldg(&a.tiles[g + 1].piece_begin) : a.n_pieces;
+        const int pb = tile_at(g).piece_begin;
+        const int pe = g + 1 < a.n_tiles ? tile_at(g + 1).piece_begin : a.n_pieces;
         uint32_t bytes = 0;
         for (int k = pb; k < pe; ++k) {
-            const EvictPiece pc = a.pieces[k];
+            const EvictPiece pc = piece_at(k);
             if ((uint64_t)pc.src_page >= (uint64_t)a.num_pages || pc.src_slot < 0 ||
                 pc.n_rows <= 0 || pc.src_slot + pc.n_rows > a.P || pc.dst_row < 0 ||
                 pc.dst_row + pc.n_rows > a.tile_rows)
@@ -257,7 +287,7 @@ __global__ void __launch_bounds__(32) sq_evict_compact_kernel(const EvictArgs a)
             mbar_arrive_expect_tx(bar, bytes);
         }
         for (int k = pb; k < pe; ++k) {
-            const EvictPiece pc = a.pieces[k];
+            const EvictPiece pc = piece_at(k);
             if ((uint64_t)pc.src_page >= (uint64_t)a.num_pages || pc.src_slot < 0 ||
                 pc.n_rows <= 0 || pc.src_slot + pc.n_rows > a.P || pc.dst_row < 0 ||
                 pc.dst_row + pc.n_rows > a.tile_rows) {
@@ -281,8 +311,8 @@ __global__ void __launch_bounds__(32) sq_evict_compact_kernel(const EvictArgs a)
         }
         fence_proxy_async_smem();
         const int g = tb + t;
-        const EvictTile tl = a.tiles[g];
-        const int pe = g + 1 < a.n_tiles ? __ldg(&a.tiles[g + 1].piece_begin) : a.n_pieces;
+        const EvictTile tl = tile_at(g);
+        const int pe = g + 1 < a.n_tiles ? tile_at(g + 1).piece_begin : a.n_pieces;
         const bool zeros = tl.piece_begin == pe;  // no pieces: a tile of zeros
         if ((uint64_t)tl.dst_page < (uint64_t)a.num_pages && tl.dst_slot >= 0 && tl.n_rows > 0 &&
             tl.n_rows <= a.tile_rows && tl.dst_slot + tl.n_rows <= a.P && (!zeros || a.zero_tiles)) {
@@ -349,19 +379,19 @@ int evict_smem_bytes(int tile_rows, int D, int stages, bool zero_tiles) {
 }
 
 // The ring depths built: 3, 4 and 6 slots (the host's choices).
-template <typename F>
+template <typename Args, typename F>
 static cudaError_t with_evict_kernel(int stages, F f) {
     switch (stages) {
-        case 3: return f(sq_evict_compact_kernel<3>);
-        case 4: return f(sq_evict_compact_kernel<4>);
-        case 6: return f(sq_evict_compact_kernel<6>);
+        case 3: return f(sq_evict_compact_kernel<3, Args>);
+        case 4: return f(sq_evict_compact_kernel<4, Args>);
+        case 6: return f(sq_evict_compact_kernel<6, Args>);
         default: return cudaErrorInvalidValue;
     }
 }
 
 int evict_ctas_per_sm(int tile_rows, int D, int stages) {
     int n = 0;
-    const cudaError_t e = with_evict_kernel(stages, [&](auto kernel) {
+    const cudaError_t e = with_evict_kernel<EvictArgs>(stages, [&](auto kernel) {
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, 32,
                                                              evict_smem_bytes(tile_rows, D, stages));
     });
@@ -370,24 +400,33 @@ int evict_ctas_per_sm(int tile_rows, int D, int stages) {
 
 cudaError_t evict_prepare() {
     for (int stages : {3, 4, 6}) {
-        const cudaError_t e = with_evict_kernel(stages, [&](auto kernel) {
+        auto raise = [&](auto kernel) {
             return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         evict_smem_bytes(kStageTokens, 128, stages, true));
-        });
+        };
+        cudaError_t e = with_evict_kernel<EvictArgs>(stages, raise);
+        if (e == cudaSuccess) e = with_evict_kernel<EvictInlineArgs>(stages, raise);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t launch_evict(const EvictArgs& a, cudaStream_t st) {
-    const int blocks = a.L * 2 * a.Hkv * (a.chunk ? a.n_chunks : 1);
+template <typename Args>
+static cudaError_t launch_evict_kernel(const Args& a, cudaStream_t st) {
+    const int blocks = a.L * 2 * a.Hkv * std::max(a.n_chunks, 1);
     if (blocks == 0 || a.n_tiles == 0) return cudaSuccess;
     const int smem = evict_smem_bytes(a.tile_rows, a.D, a.stages, a.zero_tiles != 0);
-    const cudaError_t e = with_evict_kernel(a.stages, [&](auto kernel) {
+    const cudaError_t e = with_evict_kernel<Args>(a.stages, [&](auto kernel) {
         kernel<<<blocks, 32, smem, st>>>(a);
         return cudaSuccess;
     });
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_evict(const EvictArgs& a, cudaStream_t st) { return launch_evict_kernel(a, st); }
+
+cudaError_t launch_evict_inline(const EvictInlineArgs& a, cudaStream_t st) {
+    return launch_evict_kernel(a, st);
 }
 
 }  // namespace sq

@@ -183,6 +183,15 @@ struct EvictArgs {
     int* err;
 };
 
+// A plan of few tiles and pieces goes with the launch.
+constexpr int kEvictInline = 224;       // tiles and pieces together
+constexpr int kEvictInlineChunks = 64;
+struct EvictInlineArgs : EvictArgs {
+    int4 rec[kEvictInline];             // the tiles, then the pieces
+    int32_t inline_chunk[kEvictInlineChunks + 1];
+};
+static_assert(sizeof(EvictInlineArgs) <= 4096, "launch arguments");
+
 cudaError_t launch_append(AppendArgs& a, cudaStream_t st);
 cudaError_t launch_append_batch(AppendBatchArgs& a, cudaStream_t st);
 // Shared memory of one eviction CTA for a tile size and ring depth (plus one
@@ -192,6 +201,7 @@ int evict_smem_bytes(int tile_rows, int D, int stages, bool zero_tiles = false);
 int evict_ctas_per_sm(int tile_rows, int D, int stages);
 cudaError_t evict_prepare();  // raises the dynamic shared-memory limit once
 cudaError_t launch_evict(const EvictArgs& a, cudaStream_t st);
+cudaError_t launch_evict_inline(const EvictInlineArgs& a, cudaStream_t st);
 
 // Read-only streaming probe over `bytes` (multiple of 16) at `buf`.
 cudaError_t launch_read_probe(const void* buf, size_t bytes, unsigned int* sink, int num_sms,
