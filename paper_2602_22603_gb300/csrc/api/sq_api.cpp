@@ -79,6 +79,7 @@ struct PrefillPlanEntry {
     std::vector<int32_t> spans;  // start, end pairs as passed
     size_t o_items = 0, o_merges = 0, o_pages = 0;  // byte offsets of the parts of d
     int32_t n_tiles = 0, n_pieces = 0, BP = 0, n_items = 0, n_merges = 0, n_parts = 0;
+    int32_t max_splits = 0;
     int64_t visible_pairs = 0;
     WriteTickets writes;   // of the sequence's pages, as a decode plan has them
     uint8_t* d = nullptr;  // [tiles][items][merges][tile_pages]
@@ -1238,6 +1239,9 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         victim->n_items = (int32_t)plan.items.size();
         victim->n_merges = (int32_t)plan.merges.size();
         victim->n_parts = plan.n_parts;
+        victim->max_splits = 0;
+        for (const PrefillMerge& m : plan.merges)
+            victim->max_splits = std::max(victim->max_splits, m.n);
         victim->visible_pairs = plan.visible_pairs;
         list_writes(c, s->pages.data(), s->pages.size(), &victim->writes);
         victim->valid = true;
@@ -1326,6 +1330,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         PrefillCombineArgs ca;
         ca.merges = reinterpret_cast<const PrefillMerge*>(plan.d + plan.o_merges);
         ca.n_merges = plan.n_merges;
+        ca.max_splits = plan.max_splits;
         ca.part_o = a.part_o;
         ca.part_ml = a.part_ml;
         ca.out = out;

@@ -95,6 +95,7 @@ struct PrefillCombineArgs {
     int32_t out_f32;
     float* lse;
     int32_t n_q, Hq, Hkv, G, BP;
+    int32_t max_splits;  // of any merge
     int32_t rows;  // rows of a unit that can hold queries (of kPrefillQTiles * kPrefillRows)
 };
 

@@ -1265,22 +1265,26 @@ __global__ void __launch_bounds__(320, 1)
 }
 
 // Merges the key-range splits of each query row: weights 2^(lse_s - max).
-// One warp per (split unit, row, 64 columns); the lanes take the splits' log-sum-
-// exps (up to 64 splits).  The partial outputs of the first 24 splits are
-// loaded together with them, so a row of up to 24 splits costs one round trip;
-// an empty split's partial (never written) is read but selected away.
-//
-// Two warps a row keep its loads in few registers, so that a batch of short
-// rows (an 8-query call: 256 rows of 19 splits) spreads over the SMs.  The
+// One warp per (split unit, row, 32 V columns); the lanes take the splits' log-
+// sum-exps (up to 64 splits).  The partial outputs of the first U splits are
+// loaded together with them, so a row of up to U splits costs one round trip;
+// an empty split's partial (never written) is read but selected away.  The
 // kernel lets the next one be scheduled at once: a next layer's prefill CTAs
 // take the SMs as this layer's leave.
+//
+// What bounds it: the loads in flight.  Many rows of few splits (a split last
+// round: 10,240 rows of 7) want many warps, each with a whole row in few
+// registers (V = D / 32, U = 8); few rows of many splits (an 8-query call: 256
+// rows of 19) one round trip, spread over the SMs (V = 2, U = 24).  With the
+// second form for both, a turn with four layers of the former took 2,500 us
+// instead of 2,484; with the first for both, an 8-query call needs three round
+// trips for its 19 splits.
 constexpr int kCombineThreads = 128;
-template <int D>
-__global__ void __launch_bounds__(kCombineThreads, 6)
+constexpr int kCombineFew = 8;  // splits up to which the first form is used
+template <int D, int V, int U>  // V: output elements per lane, U: splits per batch of loads
+__global__ void __launch_bounds__(kCombineThreads, U > kCombineFew ? 6 : 8)
     sq_prefill_combine_kernel(const PrefillCombineArgs a) {
-    constexpr int V = 2;        // output elements per lane
     constexpr int kParts = D / (32 * V);
-    constexpr int U = 24;      // splits per batch of loads
     grid_launch_dependents();
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -1303,15 +1307,22 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
     const float ml0 = lane < n_split ? a.part_ml[part0 + (size_t)lane * kRowsPerUnit] : -INFINITY;
     const float ml1 =
         lane + 32 < n_split ? a.part_ml[part0 + (size_t)(lane + 32) * kRowsPerUnit] : -INFINITY;
-    float2 vals[U];
+    float vals[U][V];
     auto load = [&](int s0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int s = s0 + u;  // the same in every lane
-            vals[u] = make_float2(0.f, 0.f);
-            if (s < n_split)
-                vals[u] = *reinterpret_cast<const float2*>(
-                    a.part_o + (part0 + (size_t)s * kRowsPerUnit) * D + col);
+            const float* po = a.part_o + (part0 + (size_t)s * kRowsPerUnit) * D + col;
+#pragma unroll
+            for (int e = 0; e < V; ++e) vals[u][e] = 0.f;
+            if (s >= n_split) continue;
+            if constexpr (V == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(po);
+                vals[u][0] = v.x; vals[u][1] = v.y; vals[u][2] = v.z; vals[u][3] = v.w;
+            } else {
+                const float2 v = *reinterpret_cast<const float2*>(po);
+                vals[u][0] = v.x; vals[u][1] = v.y;
+            }
         }
     };
     load(0);
@@ -1326,7 +1337,7 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
     float W = w0 + w1;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) W += __shfl_xor_sync(0xffffffffu, W, off);
-    float acc[V] = {0.f, 0.f};
+    float acc[V] = {};
     for (int s0 = 0; W > 0.f && s0 < n_split; s0 += U) {
         if (s0 > 0) load(s0);
 #pragma unroll
@@ -1334,19 +1345,31 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
             const int s = s0 + u;
             const float ws = __shfl_sync(0xffffffffu, s < 32 ? w0 : w1, s & 31);
             if (s < n_split && ws > 0.f) {
-                acc[0] += ws * vals[u].x;
-                acc[1] += ws * vals[u].y;
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[e] += ws * vals[u][e];
             }
         }
     }
     const float inv = W > 0.f ? 1.f / W : 0.f;
     const size_t o = ((size_t)qi * a.Hq + h) * D + col;
-    if (a.out_f32)
-        *reinterpret_cast<float2*>(reinterpret_cast<float*>(a.out) + o) =
-            make_float2(acc[0] * inv, acc[1] * inv);
-    else
-        *reinterpret_cast<uint32_t*>(reinterpret_cast<__nv_bfloat16*>(a.out) + o) =
-            pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    if (a.out_f32) {
+        float* out = reinterpret_cast<float*>(a.out) + o;
+        if constexpr (V == 4)
+            *reinterpret_cast<float4*>(out) =
+                make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
+        else
+            *reinterpret_cast<float2*>(out) = make_float2(acc[0] * inv, acc[1] * inv);
+    } else {
+        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + o;
+        if constexpr (V == 4) {
+            uint2 u;
+            u.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+            u.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+            *reinterpret_cast<uint2*>(out) = u;
+        } else {
+            *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+        }
+    }
     if (lane == 0 && col == 0 && a.lse)
         a.lse[(size_t)qi * a.Hq + h] = W > 0.f ? (M + __log2f(W)) * 0.69314718055994531f : -INFINITY;
 }
@@ -1363,9 +1386,13 @@ static cudaError_t prepare() {
     e = cudaFuncSetAttribute(dev::sq_prefill_kernel<D, PrefillShortArgs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              dev::PreCfg<D, true>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    // the same split of L1 and shared memory as the prefill kernel's: the two
-    // take turns on every SM
-    return cudaFuncSetAttribute(dev::sq_prefill_combine_kernel<D>,
+    // the same split of L1 and shared memory as the prefill kernel's: they take
+    // turns on every SM
+    e = cudaFuncSetAttribute(dev::sq_prefill_combine_kernel<D, 2, 24>,
+                             cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(dev::sq_prefill_combine_kernel<D, D / 32, dev::kCombineFew>,
                                 cudaFuncAttributePreferredSharedMemoryCarveout,
                                 cudaSharedmemCarveoutMaxShared);
 }
@@ -1406,7 +1433,8 @@ cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
 }
 
 cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStream_t st) {
-    const int64_t warps = (int64_t)a.n_merges * a.rows * (D / 64);
+    const bool few = a.max_splits <= dev::kCombineFew;
+    const int64_t warps = (int64_t)a.n_merges * a.rows * (few ? 1 : D / 64);
     const int per = dev::kCombineThreads / 32;
     const unsigned grid = (unsigned)((warps + per - 1) / per);
     if (grid == 0) return cudaSuccess;
@@ -1420,8 +1448,12 @@ cudaError_t launch_prefill_combine(const PrefillCombineArgs& a, int D, cudaStrea
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    if (D == 128) return cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<128>, a);
-    return cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<64>, a);
+    constexpr int kF = dev::kCombineFew;
+    if (D == 128)
+        return few ? cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<128, 4, kF>, a)
+                   : cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<128, 2, 24>, a);
+    return few ? cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<64, 2, kF>, a)
+               : cudaLaunchKernelEx(&cfg, dev::sq_prefill_combine_kernel<64, 2, 24>, a);
 }
 
 }  // namespace sq

@@ -42,6 +42,20 @@ def test_more_units_than_sms(Hq, Hkv, D, P, n, n_q, spans):
         p.close()
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("Hkv,G", [(152, 1), (76, 2), (21, 2), (19, 4), (16, 2), (2, 8)])
+def test_merges_of_few_and_many_splits(D, Hkv, G):
+    # 1, 2, 7, 8, 9 and 23 or more splits of every unit (8 and less merge a row a warp)
+    p = Pair(1, Hkv * G, Hkv, D, 64, num_pages=60, seed=D + Hkv)
+    try:
+        h = p.seq_new()
+        p.append(h, 3003)
+        check(p, h, 0, 5, [(100, 900)], seed=Hkv)
+        check(p, h, 0, 3, [], seed=Hkv, out_dtype=sq.SQ_OUT_BF16)
+    finally:
+        p.close()
+
+
 @pytest.mark.parametrize("D,n,n_q", [(64, 18000, 5120), (128, 18001, 5003)])
 def test_split_last_round(D, n, n_q):
     # 160 units on 152 SMs: the units of a second round are split in key ranges
