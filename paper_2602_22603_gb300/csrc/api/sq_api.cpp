@@ -8,6 +8,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <functional>
 #include <cstddef>
 #include <cstring>
 #include <deque>
@@ -315,19 +316,29 @@ void poll_writes(sq_cache* c) {
     }
 }
 
-// The write tickets of a new plan's pages.
+// The write tickets of a new plan's pages, in one pass (a new context's plan has
+// a page for every 64 tokens of it, all written lately): the newest kMaxUnsafe
+// are kept as a heap with the oldest of them in front.
 void list_writes(sq_cache* c, const int32_t* pages, size_t n, WriteTickets* w) {
     w->top.clear();
     w->rest = 0;
-    for (size_t i = 0; i < n; ++i)
-        if (c->page_ticket[pages[i]] > c->write_done)
-            w->top.push_back({c->page_ticket[pages[i]], pages[i]});
-    if (w->top.size() <= (size_t)kMaxUnsafe) return;
-    std::partial_sort(w->top.begin(), w->top.begin() + kMaxUnsafe, w->top.end(),
-                      [](const std::pair<uint64_t, int32_t>& x,
-                         const std::pair<uint64_t, int32_t>& y) { return x.first > y.first; });
-    for (size_t i = kMaxUnsafe; i < w->top.size(); ++i) w->rest = std::max(w->rest, w->top[i].first);
-    w->top.resize(kMaxUnsafe);
+    const std::greater<std::pair<uint64_t, int32_t>> newer;
+    const uint64_t* ticket = c->page_ticket.data();
+    uint64_t floor = c->write_done;  // tickets up to here are left out
+    for (size_t i = 0; i < n; ++i) {
+        const uint64_t t = ticket[pages[i]];
+        if (t <= floor) {
+            if (t > c->write_done) w->rest = std::max(w->rest, t);
+            continue;
+        }
+        w->top.push_back({t, pages[i]});
+        std::push_heap(w->top.begin(), w->top.end(), newer);
+        if (w->top.size() <= (size_t)kMaxUnsafe) continue;
+        std::pop_heap(w->top.begin(), w->top.end(), newer);
+        w->rest = std::max(w->rest, w->top.back().first);
+        w->top.pop_back();
+        floor = w->top.front().first;
+    }
 }
 
 // Whether every write to a plan's pages outside its newest few is complete: a
