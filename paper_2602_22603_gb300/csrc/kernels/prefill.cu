@@ -57,10 +57,9 @@
 // Calls whose queries fit in one query tile (kOne: the 8-query calls of an
 // auxiliary thread, every item dual-key) run an instance without the two-tile
 // path.  HBM bounds them, so, when the plan was on the device before, their
-// producer loads its item's first keys, up to the ring's depth, before the
-// dependency wait, while the previous launch's last CTAs finish and are merged:
-// 8 queries over 131,080 tokens, 87.0 -> 85.0 us a layer (79 at the read
-// probe's rate).  Loading early in the two-tile instance gained nothing (the
+// producer loads its item's first two key tiles before the dependency wait,
+// while the previous launch's last CTAs finish and are merged: 8 queries over
+// 131,080 tokens, 87.0 -> 85.4 us a layer (79 at the read probe's rate).  Loading early in the two-tile instance gained nothing (the
 // issuing lane bounds it) and lost 1 to 2% to the code generated around it; a
 // ring one slot longer (the second query tile's space), or L2 prefetches beyond
 // the ring, slow the CTAs still at work by more than they save the next ones.
@@ -254,52 +253,46 @@ struct FirstItem {
     }
 };
 
-// The first loads of a CTA's own item before the grid-dependency wait: pairs of
-// loads, as the producer's, as many as the ring takes and `limit` allows, up to
-// the first key tile with a page that may still be being written or with rows
-// past the sequence's end.  Returns the loads issued.
+// K_0 and K_1 of a CTA's own dual-key item, before the grid-dependency wait:
+// unless a page of theirs may still be being written, or one has rows past the
+// sequence's end.  Returns the loads issued (2 or 0).  Two of the ring's slots
+// and not all: where nothing precedes the launch, the queries, whose load waits
+// for the dependency, would queue behind the ring's 20 MB (8 queries over
+// 131,080 tokens: calls apart 90.4 us with four loads, 89.3 with two or none;
+// layers back to back 85.4, 85.4 and 86.3).
 template <int D, bool kOne>
 __device__ __forceinline__ int early_loads(const CUtensorMap* pool_map, const PrefillShortArgs& a,
                                            const Smem& sm, const FirstItem& start, const Item& it,
-                                           int limit, int lane) {
+                                           int lane) {
     using C = PreCfg<D, kOne>;
+    static_assert(C::kSlots > 2, "ring");
     const int32_t unsafe = lane < a.n_unsafe ? a.unsafe[lane] : -1;
     const int j_tail = it.t0 + it.T == a.n_tiles ? it.T - 1 : it.T;
-    int u0 = 0;
+    // lanes 0 and 1 have the records of key tiles 0 and 1
+    const int pg0 = start.rec.y, pg1 = start.rec.z;
+    bool safe = it.dual && j_tail > 1;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int p0 = __shfl_sync(0xffffffffu, pg0, x), p1 = __shfl_sync(0xffffffffu, pg1, x);
+        safe = safe && (uint32_t)p0 < (uint32_t)a.num_pages && (uint32_t)p1 < (uint32_t)a.num_pages;
+        safe = safe && !(unsafe >= 0 && (unsafe == p0 || unsafe == p1));
+    }
+    safe = __all_sync(0xffffffffu, safe);
     __syncwarp();  // (lane 0 initialised the barriers)
-    for (; u0 + 2 <= C::kSlots && u0 < limit; u0 += 2) {
-        int j0, kv0, j1, kv1;
-        load_of(u0, it.T, it.dual, j0, kv0);
-        load_of(u0 + 1, it.T, it.dual, j1, kv1);
-        const int j = (lane & 1) ? j1 : j0, kv = (lane & 1) ? kv1 : kv0;
-        const int key0 = __shfl_sync(0xffffffffu, start.rec.x, j);
-        const int pg0 = __shfl_sync(0xffffffffu, start.rec.y, j);
-        const int pg1 = __shfl_sync(0xffffffffu, start.rec.z, j);
-        const int key0b = __shfl_sync(0xffffffffu, start.rec.w, j);
-        bool safe = j < j_tail && (uint32_t)pg0 < (uint32_t)a.num_pages &&
-                    (uint32_t)pg1 < (uint32_t)a.num_pages;
+    if (safe && lane < 2) {
+        const uint32_t fb = sm.bar<D, kOne>(C::kBarFull + lane);
+        const uint32_t dst = sm.base + C::kOffRing + lane * C::kSlotBytes;
+        mbar_arrive_expect_tx(fb, C::kSlotBytes);
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {  // (lanes 0 and 1 hold the pair's pages)
-            const int p0 = __shfl_sync(0xffffffffu, pg0, x), p1 = __shfl_sync(0xffffffffu, pg1, x);
-            safe = safe && !(unsafe >= 0 && (unsafe == p0 || unsafe == p1));
-        }
-        if (!__all_sync(0xffffffffu, safe)) break;
-        if (lane < 2) {
-            const int slot = u0 + lane;
-            const uint32_t fb = sm.bar<D, kOne>(C::kBarFull + slot);
-            const uint32_t dst = sm.base + C::kOffRing + slot * C::kSlotBytes;
-            const int head_row = (kv ? a.Hkv + it.g : it.g) * a.P;
-            mbar_arrive_expect_tx(fb, C::kSlotBytes);
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int cb = 0; cb < C::kColBlocks; ++cb)
-                    tma_load_4d(dst + cb * C::kBlockBytes + b * 64 * 128, pool_map, fb, cb * 64,
-                                head_row + ((b ? key0b : key0) & (a.P - 1)), b ? pg1 : pg0, a.layer);
-        }
+            for (int cb = 0; cb < C::kColBlocks; ++cb)
+                tma_load_4d(dst + cb * C::kBlockBytes + b * 64 * 128, pool_map, fb, cb * 64,
+                            it.g * a.P + ((b ? start.rec.w : start.rec.x) & (a.P - 1)), b ? pg1 : pg0,
+                            a.layer);
     }
     __syncwarp();
-    return u0;
+    return safe ? 2 : 0;
 }
 
 // The producer warp, item by item: the query tiles, then the K and V tiles of
@@ -336,7 +329,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
     // load i + 1 before the next one has a commit of its own; bit s of `par`:
     // parity of slot s's next commit.
     uint32_t own = 0, par = 0;
-    uint32_t slot0 = u_early % C::kSlots;  // slot of the next load
+    uint32_t slot0 = u_early;  // slot of the next load
     uint32_t tail_u = 0;      // the load that used the fix-up barrier last
     bool tail_open = false;   // ... and was not handed over on its slot's barrier
     bool ok = true;
@@ -392,9 +385,7 @@ __device__ void prefill_produce(const CUtensorMap* pool_map, const CUtensorMap* 
         fence_proxy_async_smem();
         __syncwarp();
     };
-    if (u_early > 0)  // (`own` after the first loads, as the loop below keeps it)
-        own = make_item<kOne>(a, raw).dual ? (1u << u_early) - 1u
-                                     : (3u << (u_early - 2)) | (0x55555555u & ((1u << (u_early - 2)) - 1u));
+    if (u_early > 0) own = 3;  // as the loop below keeps it
     while (ok && raw.z >= 0) {
         const Item it = make_item<kOne>(a, raw);
         const uint32_t clc_parity = (n_items - 1) & 1;
@@ -1207,8 +1198,7 @@ __global__ void __launch_bounds__(320, 1)
         if constexpr (kOne) {
             if (a.kv_early) {
                 const Item it = make_item<kOne>(a, start.raw);
-                // (the pair with which the next item is taken in stays with the loop)
-                u_early = early_loads<D, kOne>(&pool_map, a, sm, start, it, 2 * it.T - 2, lane);
+                u_early = early_loads<D, kOne>(&pool_map, a, sm, start, it, lane);
             }
         }
     }
