@@ -131,8 +131,11 @@ SQ_API int sq_seq_new(sq_cache *cache, sq_seq *out);
 SQ_API int sq_append_kv(sq_cache *cache, sq_seq seq, int32_t n_tokens, const void *k,
                  const void *v, void *stream);
 
-/* Append one token to each of n_seqs sequences in one launch (a decode step
- * of a batch; Algorithm 1: C <- C + R one generated token at a time).
+/* Append one token to each of n_seqs sequences (a decode step of a batch;
+ * Algorithm 1: C <- C + R one generated token at a time).  One launch for up to
+ * 128 sequences; a new one starts at a sequence that writes in place to rows
+ * which an earlier one of the launch copies (holders of one last page, after
+ * an eviction of trailing rows from one of them).
  *   seqs: host, n_seqs distinct live handles
  *   k, v: device, bf16, contiguous [num_layers][n_seqs][num_kv_heads][head_dim]:
  *         row i belongs to seqs[i]

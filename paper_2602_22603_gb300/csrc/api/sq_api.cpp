@@ -795,7 +795,8 @@ int sq_append_kv_batch(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, const vo
         plan_len_updates(c, seqs[i], plans[i], old_versions[i], st, &ups[i]);
     int rc = fence_taken_pages(c, taken, stream);
     if (rc != SQ_OK) return undo(n_seqs, rc);
-    for (int32_t b = 0; b < n_seqs; b += kAppendBatchMax) {
+    for (int32_t b = 0, end; b < n_seqs; b = end) {
+        end = append_launch_end(plans, b, kAppendBatchMax);
         AppendBatchArgs a;
         a.pool = c->pool;
         a.k = reinterpret_cast<const __nv_bfloat16*>(k);
@@ -804,7 +805,7 @@ int sq_append_kv_batch(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, const vo
         a.L = g.L; a.Hkv = g.Hkv; a.P = g.P; a.D = g.D;
         a.n_total = n_seqs;
         a.row0 = b;
-        a.n = std::min(kAppendBatchMax, n_seqs - b);
+        a.n = end - b;
         AppendLens& l = a.lens;
         l.n = 0;
         a.n_cow = 0;

@@ -220,6 +220,21 @@ void HostCache::undo_append(int32_t h, const AppendPlan& plan) {
     s->version = g_version_counter++;
 }
 
+int32_t append_launch_end(const std::vector<AppendPlan>& plans, int32_t begin, int32_t most) {
+    const int32_t n = (int32_t)std::min<int64_t>(plans.size(), (int64_t)begin + most);
+    bool copies = false;
+    for (int32_t i = begin; i < n; ++i) {
+        const AppendPlan& p = plans[i];
+        if (copies && !p.cow && p.taken.empty())  // in place
+            for (int32_t j = begin; j < i; ++j)
+                // (its slot is its old fill)
+                if (plans[j].cow && plans[j].cow_old == p.pages[0] && p.last_fill0 < plans[j].cow_rows)
+                    return i;
+        copies |= p.cow;
+    }
+    return n;
+}
+
 bool has_partial_pages(const Seq& s, int32_t P) {
     for (size_t q = 0; q + 1 < s.fill.size(); ++q)
         if (s.fill[q] != P) return true;

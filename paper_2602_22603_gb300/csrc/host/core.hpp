@@ -115,6 +115,14 @@ struct AppendPlan {
     std::vector<int32_t> taken;    // pages newly taken (cow page first)
 };
 
+// Appends of one row each, planned one after the other: the end of the launch
+// that starts with plans[begin], at most `most` of them.  A launch's copies and
+// rows are in no order, so it ends before an append that writes in place to a
+// row which a copy of the same launch reads.  That takes two holders of a page
+// with different fills: an eviction of trailing rows moves nothing and leaves
+// the page shared, and the last holder left writes where its own rows end.
+int32_t append_launch_end(const std::vector<AppendPlan>& plans, int32_t begin, int32_t most);
+
 // One contiguous piece of an eviction's row movement: n rows from slots
 // src_slot .. of page src_page to slots dst_slot .. of page dst_page, or n
 // zero rows when src_page is -1.

@@ -38,9 +38,12 @@ __device__ __forceinline__ void write_lens(const AppendLens& l) {
 // 8 x 128 (6.3 GB moved) took 1,531 us in seven appends, now 930 (6.8 TB/s).
 //
 // Copy-on-write: the blocks after the append's copy the rows that a sequence
-// keeps of a shared last page to its fresh page, one plane each.  They read
-// slots below the old fill and the append writes slots from it on, so the two
-// parts of a launch never touch the same row.
+// keeps of a shared last page to its fresh page, one plane each, in no order
+// with the appended rows.  A sequence's copy reads slots below its fill and its
+// row goes to the slot at it.  Of two sequences of a batch that hold one page
+// with different fills, the shorter may write in place to a row that the longer
+// copies: the host ends the launch before such a write (append_launch_end), so
+// the two parts of a launch never touch the same row.
 constexpr int kAppendThreads = 256;
 constexpr int kAppendUnroll = 8;  // vectors a thread has in flight
 constexpr int kAppendVecs = kAppendThreads * kAppendUnroll;

@@ -1,7 +1,7 @@
 """Appends against the oracle, bit for bit, where the append kernels can go
 wrong: the edges of a block's chunk of tokens, head counts that do not divide a
-block's rows, page edges, more pages than one launch takes, and copy-on-write
-of the last page in the same launch."""
+block's rows, page edges, more pages than one launch takes, copy-on-write of the
+last page in the same launch, and batches whose holders of a page differ in fill."""
 import pytest
 import torch
 
@@ -44,6 +44,32 @@ def test_append_sizes_and_copy_on_write(Hkv, D, P, chunk):
     assert p.cache.sync_status() == sq.SQ_OK
     p.check_tables()
     for h in (a, b, c, d):
+        p.check_contents(h)
+    p.close()
+
+
+# Three holders of one last page with 5, 3 and 1 rows of it: whoever is left alone
+# with the page writes in place, in a longer holder's rows if it is a shorter one.
+# Enough planes (768 blocks a copy) that a launch's blocks overlap.
+@pytest.mark.parametrize("ragged", [False, True])
+@pytest.mark.parametrize("order", [(0, 1, 2), (2, 1, 0), (1, 0, 2), (0, 2), (2, 0)])
+def test_batch_of_holders_with_different_fills(order, ragged):
+    p = Pair(48, 8, 8, 128, 64, num_pages=60, seed=len(order) + 2 * ragged)
+    keep = []
+    for _ in range(3):
+        a = p.seq_new()
+        keep.append(p.append(a, 69))
+        hs = [a, p.fork(a), p.fork(a)]
+        p.evict(hs[1], [(67, 69)], ragged=ragged)
+        p.evict(hs[2], [(65, 69)], ragged=ragged)
+        if len(order) == 2:
+            p.release(hs.pop(1))
+            hs.insert(1, None)
+        keep.append(p.append_batch([hs[i] for i in order]))
+        keep.append(p.append_batch([hs[i] for i in order]))
+    assert p.cache.sync_status() == sq.SQ_OK
+    p.check_tables()
+    for h in p.o:
         p.check_contents(h)
     p.close()
 
