@@ -408,6 +408,22 @@ int upload(sq_cache* c, UploadSlot& s, const void* src, size_t bytes, void* stre
     return staged_copy(c, s.d, src, bytes, stream);
 }
 
+// A call fails after it has enqueued something that uses plan entry `p` on `st`
+// (its upload, a launch): the entry is not used again as it is, and its buffers
+// only after that work.
+template <typename Entry>
+int drop_plan(Entry& p, cudaStream_t st, int code) {
+    p.valid = false;
+    if (cudaEventRecord(p.ev, st) == cudaSuccess) {
+        p.ev_recorded = true;
+        p.ev_stream = st;
+    } else {
+        cudaStreamSynchronize(st);
+        cudaGetLastError();
+    }
+    return code;
+}
+
 void free_entry(PlanEntry& p) {
     if (p.d_plan) cudaFree(p.d_plan);
     if (p.d_part) cudaFree(p.d_part);
@@ -940,7 +956,7 @@ int sq_decode_attention(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, int32_t
         if (c->staging.size() < (size_t)lay.total) c->staging.resize(lay.total);
         plan_serialize(plan, lay, c->staging.data());
         int urc = staged_copy(c, victim->d_plan, c->staging.data(), lay.total, stream);
-        if (urc != SQ_OK) { victim->valid = false; return urc; }
+        if (urc != SQ_OK) return drop_plan(*victim, st, urc);
         c->stats.decode_plans_built += 1;
         victim->valid = true;
         victim->n_ctas = c->decode_ctas;
@@ -1009,9 +1025,9 @@ int sq_decode_attention(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, int32_t
     c->debug_flags &= ~SQ_DEBUG_DROP_DECODE_STAGE;
     a.err = c->d_err;
     e = launch_decode(c->tmap, a, L.n_ctas, g.D, st);
-    if (e != cudaSuccess) { hit->valid = false; return cuda_status(e); }
+    if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
     e = cudaEventRecord(hit->ev, st);
-    if (e != cudaSuccess) return cuda_status(e);
+    if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
     hit->ev_recorded = true;
     hit->ev_stream = st;
     for (int32_t i = 0; i < n_seqs; ++i) c->host->seq_mut(seqs[i])->last_stream = stream;
@@ -1236,7 +1252,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         put(o_merges, plan.merges.data(), o_pages - o_merges);
         put(o_pages, plan.tile_pages.data(), bytes - o_pages);
         rc = staged_copy(c, victim->d, c->staging.data(), bytes, stream);
-        if (rc != SQ_OK) return rc;
+        if (rc != SQ_OK) return drop_plan(*victim, st, rc);
         victim->seq = seq;
         victim->version = s->version;
         victim->n_q = n_q;
@@ -1282,12 +1298,13 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
             c->pre_part = nullptr;
             c->pre_part_cap = 0;
             e = cudaMalloc(&c->pre_part, need * 5 / 4);
-            if (e != cudaSuccess) return cuda_status(e);
+            if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
             c->pre_part_cap = need * 5 / 4;
         } else if (last && last->ev_recorded && last->ev_stream != st) {
             e = cudaStreamWaitEvent(st, last->ev, 0);
-            if (e != cudaSuccess) return cuda_status(e);
+            if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
         }
+        c->pre_last = hit;  // (its event is recorded whatever becomes of the call)
     }
     // queries: {D, Hq, n_q}, one box = the G heads of a KV head x BP positions
     CUtensorMap qmap;
@@ -1301,7 +1318,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
                             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return SQ_ERR_INVALID_ARG;
+        if (r != CUDA_SUCCESS) return drop_plan(*hit, st, SQ_ERR_INVALID_ARG);
     }
     PrefillShortArgs a;
     a.tiles = reinterpret_cast<const PrefillTile*>(plan.d);
@@ -1337,7 +1354,7 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
                     : nullptr;
     a.err = c->d_err;
     e = launch_prefill(c->tmap, qmap, a, g.D, st);
-    if (e != cudaSuccess) return cuda_status(e);
+    if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
     if (plan.n_merges > 0) {
         PrefillCombineArgs ca;
         ca.merges = reinterpret_cast<const PrefillMerge*>(plan.d + plan.o_merges);
@@ -1356,11 +1373,10 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         // (a call whose queries all fit in tile a has only their rows)
         ca.rows = n_q <= plan.BP ? n_q * g.G() : kPrefillQTiles * kPrefillRows;
         e = launch_prefill_combine(ca, g.D, st);
-        if (e != cudaSuccess) return cuda_status(e);
-        c->pre_last = hit;
+        if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
     }
     e = cudaEventRecord(hit->ev, st);
-    if (e != cudaSuccess) return cuda_status(e);
+    if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
     hit->ev_recorded = true;
     hit->ev_stream = st;
     c->host->seq_mut(seq)->last_stream = stream;
