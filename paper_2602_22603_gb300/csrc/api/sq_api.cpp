@@ -1289,17 +1289,18 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     hit->last_use = ++c->use_clock;
     const PrefillPlanEntry& plan = *hit;
     if (plan.n_parts > 0) {
-        const size_t need =
-            (size_t)plan.n_parts * kPrefillQTiles * kPrefillRows * (g.D + 1) * sizeof(float);
+        const size_t need = (size_t)plan.n_parts * prefill_part_bytes(g.D);
         const PrefillPlanEntry* last = c->pre_last;
         if (need > c->pre_part_cap) {
             if (last && last->ev_recorded) cudaEventSynchronize(last->ev);
             if (c->pre_part) cudaFree(c->pre_part);
             c->pre_part = nullptr;
             c->pre_part_cap = 0;
-            e = cudaMalloc(&c->pre_part, need * 5 / 4);
+            // (room for larger plans, up to the planner's limit)
+            const size_t cap = std::max(need, std::min(need * 5 / 4, (size_t)kPrefillPartLimit));
+            e = cudaMalloc(&c->pre_part, cap);
             if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
-            c->pre_part_cap = need * 5 / 4;
+            c->pre_part_cap = cap;
         } else if (last && last->ev_recorded && last->ev_stream != st) {
             e = cudaStreamWaitEvent(st, last->ev, 0);
             if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));

@@ -775,7 +775,8 @@ void plan_serialize(const DecodePlanHost& p, const DecodePlanLayout& L, uint8_t*
 // merge (a launch, and the partials written and read) + a quarter of a piece
 // for SMs of unequal speed.  Units of growing length (a whole trace) already
 // end with the short ones and are not split.
-static void list_prefill_items(int32_t Hkv, int32_t ctas, PrefillPlanHost* out) {
+// At most `max_parts` partial results.
+static void list_prefill_items(int32_t Hkv, int32_t ctas, int64_t max_parts, PrefillPlanHost* out) {
     constexpr double kItem = 2.0, kMergeLaunch = 4.0, kMergePiece = 0.032;
     constexpr int32_t kMaxPieces = 16;
     const int32_t n_qt = out->n_qt, units = n_qt * Hkv;
@@ -789,6 +790,7 @@ static void list_prefill_items(int32_t Hkv, int32_t ctas, PrefillPlanHost* out) 
             if (r > units) break;
             for (int32_t k = 2; k <= kMaxPieces && 4 * k <= T; ++k) {
                 const int64_t pieces = (int64_t)r * k;
+                if (pieces > max_parts) break;
                 const double cost = (double)((units - r) / ctas) * (T + kItem) +
                                     (double)((pieces + ctas - 1) / ctas) * ((T + k - 1) / k + kItem) +
                                     kMergeLaunch + kMergePiece * pieces + 0.25 * T / k;
@@ -841,7 +843,7 @@ static void list_prefill_items(int32_t Hkv, int32_t ctas, PrefillPlanHost* out) 
 // plan carries the span part as one bit per key, per key tile.
 int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* starts,
                  const int32_t* ends, int32_t n_spans, int32_t target_ctas,
-                 PrefillPlanHost* out, const int32_t* pages) {
+                 PrefillPlanHost* out, const int32_t* pages, int64_t part_limit) {
     *out = PrefillPlanHost();
     if (n < 1 || n_q < 1 || n_q > n) return kInvalidArg;
     std::vector<std::pair<int32_t, int32_t>> sp;
@@ -939,6 +941,7 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
     // fill the GPU: pick the split that minimises the estimated makespan,
     // rounds x (key tiles per item + a fixed cost per item), items running
     // `target_ctas` at a time.
+    const int64_t max_parts = part_limit / prefill_part_bytes(g.D);
     int32_t split = 1;
     if (units < target_ctas && n_tiles > 0 && target_ctas > 0) {
         constexpr double kItemCost = 4.0;  // prologue + epilogue, in key tiles
@@ -948,6 +951,7 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
         double best = 1e300;
         for (int32_t sp = 1; sp <= kPrefillMaxSplit && sp <= n_tiles; ++sp) {
             const int64_t ctas = units * sp;
+            if (sp > 1 && ctas > max_parts) break;
             const int64_t waves = (ctas + target_ctas - 1) / target_ctas;
             const double cost = (double)waves * (avg / sp + kItemCost);
             if (cost < best - 1e-9) {
@@ -957,7 +961,7 @@ int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* start
         }
     }
     out->n_split = split;
-    list_prefill_items(g.Hkv, std::max<int32_t>(1, target_ctas), out);
+    list_prefill_items(g.Hkv, std::max<int32_t>(1, target_ctas), max_parts, out);
     return kOk;
 }
 

@@ -271,13 +271,16 @@ struct PrefillPlanHost {
 // for `target_ctas` CTAs at a time.  Every unit's key range is split in
 // n_split parts when the units alone would fill fewer CTAs than that; with
 // more of them, the units of a last round that would leave CTAs idle may be.
+// The partial results of split units take at most `part_limit` bytes (0: no
+// unit is split).
 // `pages` (may be null) is the sequence's page table; with it the plan also
 // lists the page of every piece of every key tile.  Positions are slot-space
 // positions: for a sequence with partial pages, n is its slot-space end and
 // the spans include its unused slots (see prefill_slot_spans).
 int plan_prefill(const Geometry& g, int32_t n, int32_t n_q, const int32_t* starts,
                  const int32_t* ends, int32_t n_spans, int32_t target_ctas,
-                 PrefillPlanHost* out, const int32_t* pages = nullptr);
+                 PrefillPlanHost* out, const int32_t* pages = nullptr,
+                 int64_t part_limit = kPrefillPartLimit);
 
 // Slot-space form of a masked prefill over sequence `s`: validates the
 // logical spans against s.n, maps them to slot-space ranges, adds the unused

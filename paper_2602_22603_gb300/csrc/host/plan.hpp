@@ -123,6 +123,17 @@ struct PrefillMerge {
 };
 // Partial results one unit may have at most (a lane of the merge takes two).
 constexpr int32_t kPrefillMaxSplit = 64;
+// Bytes of one partial result (normalised outputs and log-sum-exps of the rows
+// of a unit, fp32), and of all that a plan may have: they are held for the
+// cache's life.  The limit is 1,016 partial results at d = 128.  By the planner's
+// model of the time, over 600 shapes drawn from 4k to 256k tokens and 8 to 16k
+// queries, it costs 11 of them up to 1.7% (unlimited, one wanted 2,272, 300 MB);
+// half of it would cost 49 of them up to 22%, such as 120 units whose five key
+// ranges each fill four rounds.
+constexpr int64_t prefill_part_bytes(int32_t D) {
+    return (int64_t)kPrefillQTiles * kPrefillRows * (D + 1) * (int64_t)sizeof(float);
+}
+constexpr int64_t kPrefillPartLimit = int64_t(128) << 20;
 
 // Byte offsets of the arrays of a decode plan inside one upload buffer.
 // Byte offsets of the serialised decode plan.  `arrive` holds one 32-bit

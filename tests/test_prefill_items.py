@@ -3,6 +3,7 @@ is in exactly one item, split units have contiguous partial results that tile
 their keys, and CTAs that take the items in order finish close together."""
 import ctypes
 import heapq
+import random
 
 import pytest
 
@@ -59,6 +60,27 @@ def test_items_cover_every_key_tile_once(Hq, Hkv, n, n_q, spans):
             assert [p for _, _, p in parts] == list(range(p0, p0 + k)) and 2 <= k <= 64
             used += range(p0, p0 + k)
     assert sorted(used) == list(range(n_parts))
+
+
+PART_LIMIT = 128 << 20           # bytes of partial results a plan may have
+PART_BYTES = 2 * 128 * (128 + 1) * 4
+
+
+def test_partial_results_are_bounded():
+    # without a limit 1,820 and 2,272 of 132 KB each (last rounds), 2,736 (few
+    # units), and 12 of the 400 drawn ones above the limit
+    shapes = [(32, 2, 236067, 5976), (32, 2, 197877, 10857), (32, 8, 250000, 1150)]
+    rng = random.Random(1)
+    for _ in range(400):
+        n = int(2 ** rng.uniform(12, 18))
+        shapes.append((*rng.choice([(32, 8), (64, 8), (16, 4), (32, 2), (8, 8), (32, 4)]), n,
+                       int(min(n, 2 ** rng.uniform(3, 14)))))
+    most = 0
+    for Hq, Hkv, n, n_q in shapes:
+        _, _, n_parts = items(Hq, Hkv, n, n_q, [])
+        assert n_parts * PART_BYTES <= PART_LIMIT, (Hq, Hkv, n, n_q, n_parts)
+        most = max(most, n_parts)
+    assert most > 700   # the limit is no tighter than it says
 
 
 @pytest.mark.parametrize("n,n_q,most", [
