@@ -424,6 +424,28 @@ int drop_plan(Entry& p, cudaStream_t st, int code) {
     return code;
 }
 
+// Room for `need` bytes of prefill partial results.  Where there is none, the
+// plans that had theirs in the buffer given up are dropped.
+int reserve_parts(sq_cache* c, size_t need) {
+    if (need <= c->pre_part_cap) return SQ_OK;
+    if (c->pre_last && c->pre_last->ev_recorded) cudaEventSynchronize(c->pre_last->ev);
+    if (c->pre_part) cudaFree(c->pre_part);
+    c->pre_part = nullptr;
+    c->pre_part_cap = 0;
+    // (room for larger plans, up to the planner's limit)
+    const size_t cap = std::max(need, std::min(need * 5 / 4, (size_t)kPrefillPartLimit));
+    const cudaError_t e = cudaMalloc(&c->pre_part, cap);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        c->pre_part = nullptr;
+        for (auto& p : c->pre_plans)
+            if (p.n_parts > 0) p.valid = false;
+        return cuda_status(e);
+    }
+    c->pre_part_cap = cap;
+    return SQ_OK;
+}
+
 void free_entry(PlanEntry& p) {
     if (p.d_plan) cudaFree(p.d_plan);
     if (p.d_part) cudaFree(p.d_part);
@@ -1197,19 +1219,26 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
         }
         PrefillPlanHost plan;
         int rc;
+        int32_t n_pos = s->n;
         if (has_partial_pages(*s, g.P)) {
             // slot space: the spans mapped through the page fills, plus the
             // unused slots of the partial pages
             std::vector<int32_t> xa, xb;
-            int32_t n_slots = 0;
             rc = prefill_slot_spans(*s, g.P, n_q, sa.data(), sb.data(), n_spans, &xa, &xb,
-                                    &n_slots);
+                                    &n_pos);
             if (rc != SQ_OK) return rc;
-            rc = plan_prefill(g, n_slots, n_q, xa.data(), xb.data(), (int32_t)xa.size(),
-                              c->num_sms, &plan, s->pages.data());
-        } else {
-            rc = plan_prefill(g, s->n, n_q, sa.data(), sb.data(), n_spans, c->num_sms, &plan,
-                              s->pages.data());
+            sa = std::move(xa);
+            sb = std::move(xb);
+        }
+        auto make_plan = [&](int64_t part_limit) {
+            return plan_prefill(g, n_pos, n_q, sa.data(), sb.data(), (int32_t)sa.size(),
+                                c->num_sms, &plan, s->pages.data(), part_limit);
+        };
+        rc = make_plan(kPrefillPartLimit);
+        if (rc == SQ_OK && plan.n_parts > 0) {
+            rc = reserve_parts(c, (size_t)plan.n_parts * prefill_part_bytes(g.D));
+            // no room for partial results: the plan without any
+            if (rc == SQ_ERR_NO_MEMORY) rc = make_plan(0);
         }
         if (rc != SQ_OK) return rc;
         // upload: key tiles, items, merges, then the page of every piece (the
@@ -1289,19 +1318,9 @@ int sq_prefill_attention(sq_cache* c, sq_seq seq, int32_t layer, int32_t n_q, co
     hit->last_use = ++c->use_clock;
     const PrefillPlanEntry& plan = *hit;
     if (plan.n_parts > 0) {
-        const size_t need = (size_t)plan.n_parts * prefill_part_bytes(g.D);
+        // (reserved when the plan was made)
         const PrefillPlanEntry* last = c->pre_last;
-        if (need > c->pre_part_cap) {
-            if (last && last->ev_recorded) cudaEventSynchronize(last->ev);
-            if (c->pre_part) cudaFree(c->pre_part);
-            c->pre_part = nullptr;
-            c->pre_part_cap = 0;
-            // (room for larger plans, up to the planner's limit)
-            const size_t cap = std::max(need, std::min(need * 5 / 4, (size_t)kPrefillPartLimit));
-            e = cudaMalloc(&c->pre_part, cap);
-            if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
-            c->pre_part_cap = cap;
-        } else if (last && last->ev_recorded && last->ev_stream != st) {
+        if (last && last->ev_recorded && last->ev_stream != st) {
             e = cudaStreamWaitEvent(st, last->ev, 0);
             if (e != cudaSuccess) return drop_plan(*hit, st, cuda_status(e));
         }

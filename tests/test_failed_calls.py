@@ -45,6 +45,25 @@ def test_streams_take_turns(cache, call):
     assert fakelib.lib().fake_races() == 0
 
 
+def test_prefill_without_room_for_partial_results(cache):
+    L = fakelib.lib()
+    a, b, c = seq(cache, 3000), seq(cache, 500), seq(cache, 9000)
+    prefill(cache, b, 1)                   # split in few pieces: a small workspace
+    assert L.fake_count(fakelib.COMBINE) == 1
+    L.fake_malloc_limit(1 << 20)
+    prefill(cache, a, 1)                   # no room for its pieces: not split
+    prefill(cache, a, 2)
+    prefill(cache, c, 2)
+    assert L.fake_count(fakelib.COMBINE) == 1
+    prefill(cache, b, 2)                   # ... nor the first call's any more
+    assert L.fake_count(fakelib.COMBINE) == 1 and L.fake_count(fakelib.PREFILL) == 5
+    L.fake_malloc_limit(-1)
+    prefill(cache, c, 3, n_q=9)            # room again
+    prefill(cache, b, 1)
+    assert L.fake_count(fakelib.COMBINE) == 2
+    assert L.fake_races() == 0
+
+
 @pytest.mark.parametrize("kind,call", [
     (fakelib.PREFILL, prefill), (fakelib.COMBINE, prefill), (fakelib.DECODE, decode)])
 @pytest.mark.parametrize("same", [True, False])
