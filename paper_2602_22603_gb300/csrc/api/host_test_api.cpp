@@ -147,6 +147,11 @@ int sqh_refcount(void* c, int32_t p) {
 
 int sqh_free_count(void* c) { return static_cast<HostCache*>(c)->alloc().free_count(); }
 
+// The merger's side of a run's arrival word: whether `word` counts every release,
+// and the word it leaves.
+int32_t sqh_arrive_complete(uint32_t word, uint32_t n) { return arrive_complete(word, n); }
+uint32_t sqh_arrive_leave(uint32_t word, uint32_t n) { return word + arrive_settle(n); }
+
 int64_t sqh_peak_live_pages(void* c) { return static_cast<HostCache*>(c)->peak_live_pages(); }
 
 // Plans a decode call.  layout_out receives 17 int64 values:

@@ -3,6 +3,12 @@
 #pragma once
 #include <stdint.h>
 
+#if defined(__CUDACC__)
+#define SQ_HOST_DEVICE __host__ __device__
+#else
+#define SQ_HOST_DEVICE
+#endif
+
 namespace sq {
 
 // Rows of one tensor-core tile: the query rows a decode work item serves
@@ -29,6 +35,21 @@ constexpr int kUnitCostStages = 2;
 constexpr int kShortUnitStages = 2;
 constexpr int kDecodeUnitCost = 4;
 constexpr int kDecodeShortUnitCost = 8;
+
+// The arrival word of a (sequence, KV head) run of n entries: one claim (1) for
+// each, and one release (kArriveRelease) for each but the last to claim, which
+// merges the run.
+constexpr uint32_t kArriveRelease = 0x10000u;
+// Whether a word counts the releases of all the other entries.
+SQ_HOST_DEVICE constexpr bool arrive_complete(uint32_t word, uint32_t n) {
+    return word >> 16 == n - 1;
+}
+// What the merger adds when it leaves: it takes back every claim and release of
+// the run, also the releases that come after it (its wait for them is bounded),
+// so that the word is zero when the call is done.
+SQ_HOST_DEVICE constexpr uint32_t arrive_settle(uint32_t n) {
+    return 0u - (n + (n - 1) * kArriveRelease);
+}
 
 // A run of logical pages read once for a group of sequences that hold the
 // same physical pages there (a main thread and its forks, Sec. 3.4).

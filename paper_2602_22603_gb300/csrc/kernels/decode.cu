@@ -627,11 +627,13 @@ __device__ void consume(const DecodeArgs& a, int it0, int it1, ItemHead next, ui
 // answer, as a rule (the last one to finish), else in acquire loads until it
 // does (their claims came first, so their releases are under way: the wait
 // depends on nothing this CTA still has to do); its own partial it reads back
-// within the CTA.  The merger sets the word back to zero.  Every CTA claims once per
-// (item, group member), also after a wait ran out, so every call leaves every
-// word at zero, and a plan upload writes zeros; the word therefore always
-// starts a call at zero.  A run holds at most 65,535 entries (the planner's
-// limit), so the halves never carry.
+// within the CTA.  The merger then takes all of the run's claims and releases off
+// the word, also the releases still due when its own wait ran out (a store of
+// zero would leave those to the next call, which could then merge too early).
+// Every CTA claims once per (item, group member), also after a wait ran out, so
+// every call leaves every word at zero, and a plan upload writes zeros; the word
+// therefore always starts a call at zero.  A run holds at most 65,535 entries
+// (the planner's limit), so the low half never carries.
 
 // GPU-scope atomics of the arrival protocol.
 __device__ __forceinline__ unsigned atom_add_acquire_gpu(unsigned* p, unsigned v) {
@@ -780,18 +782,18 @@ __device__ void close_items(const DecodeArgs& a, int it0, int it1, uint8_t* smem
                 const unsigned old = atom_add_acquire_gpu(a.arrive + key, 1u);
                 merger = (old & 0xffffu) + 1u == (unsigned)mine.n;
                 if (!merger) {
-                    red_add_release_gpu(a.arrive + key, 0x10000u);
-                } else if ((old >> 16) != (unsigned)(mine.n - 1)) {
+                    red_add_release_gpu(a.arrive + key, kArriveRelease);
+                } else if (!arrive_complete(old, mine.n)) {
                     const uint64_t t0 = globaltimer_ns();
                     for (uint32_t spin = 1;; ++spin) {
-                        if ((ld_acquire_gpu(a.arrive + key) >> 16) == (unsigned)(mine.n - 1)) break;
+                        if (arrive_complete(ld_acquire_gpu(a.arrive + key), mine.n)) break;
                         if ((spin & 31) == 0 && globaltimer_ns() - t0 > kWaitLimitNs) {
                             set_error(a.err, kErrTimeout);
                             break;
                         }
                     }
                 }
-                if (merger) a.arrive[key] = 0u;
+                if (merger) atomicAdd(a.arrive + key, arrive_settle(mine.n));
             }
             const unsigned mask = __ballot_sync(0xffffffffu, merger);
             if (merger) runs[__popc(mask & ((1u << lane) - 1u))] = mine;
