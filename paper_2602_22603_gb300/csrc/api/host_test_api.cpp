@@ -154,28 +154,21 @@ uint32_t sqh_arrive_leave(uint32_t word, uint32_t n) { return word + arrive_sett
 
 int64_t sqh_peak_live_pages(void* c) { return static_cast<HostCache*>(c)->peak_live_pages(); }
 
-// Plans a decode call.  layout_out receives 17 int64 values:
-//   offsets segs, items, cta_begin, page_ids, comb_off, arrive, total,
-//   counts n_segs, n_items, n_ctas, n_page_ids, n_comb_keys, n_comb_ent,
-//   unique_tokens, logical_tokens, sizeof(DecodeSeg), offset page_fill (-1: none).
-// If buf is non-NULL and buf_bytes >= total, the serialised plan is written.
 // The eviction CTA shape the library picks: tile rows for (P, D) and ring
 // slots for (planes, SMs).
 int32_t sqh_evict_tile_rows(int32_t P, int32_t D) { return evict_tile_rows_for(P, D); }
 int32_t sqh_evict_stages(int64_t planes, int32_t num_sms) { return evict_stages_for(planes, num_sms); }
 
-// `sqh_decode_costs` sets the units' start-up costs of the plans that follow
-// (negative: the library's own).
-static int32_t g_unit_cost = kUnitCostStages, g_short_cost = kUnitCostStages;
-void sqh_decode_costs(int32_t unit, int32_t small) {
-    g_unit_cost = unit < 0 ? kDecodeUnitCost : unit;
-    g_short_cost = small < 0 ? kDecodeShortUnitCost : small;
-}
+// Plans a decode call.  layout_out receives 17 int64 values:
+//   offsets segs, items, cta_begin, page_ids, comb_off, arrive, total,
+//   counts n_segs, n_items, n_ctas, n_page_ids, n_comb_keys, n_comb_ent,
+//   unique_tokens, logical_tokens, sizeof(DecodeSeg), offset page_fill (-1: none).
+// If buf is non-NULL and buf_bytes >= total, the serialised plan is written.
 int sqh_plan_decode(void* c, const int32_t* handles, int32_t n, int32_t n_ctas,
                     int64_t* layout_out, uint8_t* buf, int64_t buf_bytes) {
     HostCache* hc = static_cast<HostCache*>(c);
     DecodePlanHost p;
-    int rc = plan_decode(*hc, handles, n, n_ctas, &p, g_unit_cost, g_short_cost);
+    int rc = plan_decode(*hc, handles, n, n_ctas, &p);
     if (rc != kOk) return rc;
     DecodePlanLayout L = plan_layout(p, n, hc->geom().Hkv);
     int64_t v[17] = {L.segs, L.items, L.cta_begin, L.page_ids, L.comb_off, L.arrive, L.total,

@@ -937,8 +937,7 @@ int sq_decode_attention(sq_cache* c, const sq_seq* seqs, int32_t n_seqs, int32_t
     bool plan_ready = false;
     if (!hit) {
         DecodePlanHost plan;
-        int rc = plan_decode(*c->host, seqs, n_seqs, c->decode_ctas, &plan, kDecodeUnitCost,
-                             kDecodeShortUnitCost);
+        int rc = plan_decode(*c->host, seqs, n_seqs, c->decode_ctas, &plan);
         if (rc != SQ_OK) return rc;
         DecodePlanLayout lay = plan_layout(plan, n_seqs, g.Hkv);
         // least recently used entry
@@ -1551,8 +1550,7 @@ int sq_decode_attention_noalloc(sq_cache* c, const sq_seq* seqs, int32_t n_seqs,
     if (dev != c->device) return SQ_ERR_INVALID_ARG;
     if (c->noalloc_status != SQ_OK) return c->noalloc_status;
     DecodePlanHost plan;
-    int rc = plan_decode(*c->host, seqs, n_seqs, c->decode_ctas, &plan, kDecodeUnitCost,
-                             kDecodeShortUnitCost);
+    int rc = plan_decode(*c->host, seqs, n_seqs, c->decode_ctas, &plan);
     if (rc != SQ_OK) return rc;
     const DecodePlanLayout L = plan_layout(plan, n_seqs, g.Hkv);
     // scratch = [plan (with zeroed arrival words) | partial outputs | partial (max, sum)]

@@ -526,7 +526,7 @@ void evict_chunks(const std::vector<int32_t>& window_tile, int32_t n_tiles, int3
 // decode planning
 
 int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
-                int32_t n_ctas, DecodePlanHost* out, int32_t unit_cost, int32_t short_cost) {
+                int32_t n_ctas, DecodePlanHost* out) {
     *out = DecodePlanHost();
     const Geometry& g = c.geom();
     if (n_seqs < 1 || !handles || n_ctas < 1) return kInvalidArg;
@@ -671,7 +671,7 @@ int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
     int64_t total = 0, stages = 0;
     for (size_t v = 0; v < unit_seg.size(); ++v) {
         const int32_t n = ceil_div(out->segs[unit_seg[v]].n_tok, kStageTokens);
-        total += n <= kShortUnitStages ? short_cost : unit_cost;
+        total += n <= kShortUnitStages ? kDecodeShortUnitCost : kDecodeUnitCost;
         unit_start.push_back(total);
         total += n;
         stages += n;

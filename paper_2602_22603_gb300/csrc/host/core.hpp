@@ -236,11 +236,10 @@ constexpr int32_t kMaxRunEntries = 65535;
 // kStageTokens tokens and deals the stages out evenly to `n_ctas`
 // persistent CTAs.  kCapacity if a (sequence, KV head) would get more than
 // kMaxRunEntries partial results (more CTAs than that on one sequence).
-// On the line that is cut evenly a unit's start-up counts `unit_cost` stages,
-// `short_cost` for a unit of at most kShortUnitStages.
+// On the line that is cut evenly a unit's start-up counts kDecodeUnitCost
+// stages, kDecodeShortUnitCost for a unit of at most kShortUnitStages.
 int plan_decode(const HostCache& c, const int32_t* handles, int32_t n_seqs,
-                int32_t n_ctas, DecodePlanHost* out, int32_t unit_cost = kUnitCostStages,
-                int32_t short_cost = kUnitCostStages);
+                int32_t n_ctas, DecodePlanHost* out);
 
 // Serialises a plan into one buffer (8-byte aligned arrays).
 DecodePlanLayout plan_layout(const DecodePlanHost& p, int32_t n_seqs,

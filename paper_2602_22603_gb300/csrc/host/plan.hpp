@@ -24,9 +24,7 @@ constexpr int kDecodeConsumerWarps = 4 * kDecodeGroups;
 // Fixed cost of starting a work unit, in stages: its query reload and its
 // item-end merge.  The planner balances stages plus this cost per unit, so a
 // CTA that gets many short units (e.g. the few-token tails of several forks)
-// is not the one every other CTA waits for.
-constexpr int kUnitCostStages = 2;
-// The costs the decode calls plan with.  A stage passes in 0.7 us; a unit's
+// is not the one every other CTA waits for.  A stage passes in 0.7 us; a unit's
 // start and end hide behind the stages of its neighbours unless it is a stage
 // or two long.  Measured, us per pass for costs (2, 2) (4, 4) (4, 8) (6, 6):
 // 36 short sequences x 8 layers 379 376 376 383; four agents with forks and

@@ -1,11 +1,11 @@
-"""Decode plans with the units' start-up costs the library plans with (CPU): the
-items tile every (segment, KV head) once and in order, and the CTAs' shares of
-the cost line are even."""
+"""Decode plans and the units' start-up costs (CPU): the items tile every
+(segment, KV head) once and in order, and the CTAs' shares of the cost line are
+even."""
 import random
 
 import pytest
 
-from tests.hostlib import HostCache, lib
+from tests.hostlib import HostCache
 
 UNIT, SHORT, SHORT_STAGES = 4, 8, 2
 
@@ -25,11 +25,7 @@ def test_items_tile_the_cost_line(seed):
             assert hc.append(a, rng.randint(1, 64)) == 0
             seqs.append(a)
     n_ctas = rng.choice([1, 7, 152])
-    lib().sqh_decode_costs(-1, -1)
-    try:
-        rc, plan = hc.plan_decode(seqs, n_ctas)
-    finally:
-        lib().sqh_decode_costs(2, 2)
+    rc, plan = hc.plan_decode(seqs, n_ctas)
     assert rc == 0
     stages = [-(-s["n_tok"] // 64) for s in plan["segs"]]
     at = {}

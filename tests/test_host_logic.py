@@ -114,13 +114,15 @@ def _check_plan(hc, handles, plan, n_ctas, G):
     assert cb[0] == 0 and cb[-1] == len(items)
     assert all(cb[i] <= cb[i + 1] for i in range(len(cb) - 1))
     assert len(cb) - 1 <= n_ctas
-    # work per CTA (stages + a fixed cost per item) is balanced: within one
-    # unit start-up cost plus one stage
-    C = 2
-    per_cta = [sum(items[i][3] - items[i][2] + C for i in range(cb[c], cb[c + 1]))
+    # work per CTA (stages + a start-up cost per unit: 4 stages, 8 for a unit of
+    # one or two) is an even cut of the whole, but that the start-up costs at
+    # its two cuts may fall to either side
+    def cost(seg, s0, s1):
+        start = 8 if -(-segs[seg]["n_tok"] // 64) <= 2 else 4
+        return s1 - s0 + (start if s0 == 0 else 0)
+    per_cta = [sum(cost(*items[i][:1], *items[i][2:4]) for i in range(cb[c], cb[c + 1]))
                for c in range(len(cb) - 1)]
-    busy = [x for x in per_cta if x > 0]
-    assert max(busy) - min(busy) <= 2 * C + 1
+    assert max(per_cta) - min(per_cta) <= 2 * 8 + 1
     for s in segs:
         assert 1 <= s["n_grp"] <= 16 // G
         assert max(s["grp_lim"]) == s["n_tok"] and min(s["grp_lim"]) > 0
