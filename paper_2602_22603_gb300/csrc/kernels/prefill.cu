@@ -1398,7 +1398,9 @@ cudaError_t launch_prefill(const CUtensorMap& pool_map, const CUtensorMap& qmap,
     const unsigned grid = (unsigned)a.n_items;
     if (grid == 0) return cudaSuccess;
     // a programmatic dependent of whatever precedes it: its barrier and tensor
-    // memory set-up overlaps that work's tail (it waits before any read)
+    // memory set-up overlaps that work's tail.  Before its wait it reads only a
+    // plan that was on the device already (plan_ready), and, in the short
+    // instance, keys and values that no running work writes (kv_early).
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
