@@ -68,16 +68,25 @@ class Caches:
             assert np.array_equal(pool[:, page, 1, :, slot].transpose(1, 0, 2, 3), v), h
 
 
-@pytest.fixture(autouse=True)
-def _fake(monkeypatch):
+@pytest.fixture
+def caches(monkeypatch):
     monkeypatch.setattr(sq, "_lib", fakelib.lib())
+    made = []
+
+    def make(*args):
+        made.append(Caches(*args))
+        return made[-1]
+
+    yield make
+    for c in made:   # while the stand-in is the library
+        c.cache.close()
 
 
 @pytest.mark.parametrize("copies_last", [False, True])
 @pytest.mark.parametrize("ragged", [False, True])
 @pytest.mark.parametrize("order", [(0, 1, 2), (2, 1, 0), (1, 0, 2), (0, 2), (2, 0)])
-def test_holders_of_different_fills(order, ragged, copies_last):
-    c = Caches(64, 40, copies_last)
+def test_holders_of_different_fills(caches, order, ragged, copies_last):
+    c = caches(64, 40, copies_last)
     a = c.new(69)                       # last page: 5 rows
     hs = [a, c.fork(a), c.fork(a)]
     c.evict(hs[1], [(67, 69)], ragged)  # 3 rows, the page still shared
@@ -95,9 +104,9 @@ def test_holders_of_different_fills(order, ragged, copies_last):
 
 @pytest.mark.parametrize("copies_last", [False, True])
 @pytest.mark.parametrize("seed", range(6))
-def test_random_holders(seed, copies_last):
+def test_random_holders(caches, seed, copies_last):
     rng = random.Random(seed)
-    c = Caches(rng.choice([8, 64]), 900, copies_last)
+    c = caches(rng.choice([8, 64]), 900, copies_last)
     live = []
     for _ in range(rng.choice([3, 40])):
         live.append(c.new(rng.randint(1, 100)))
@@ -113,8 +122,8 @@ def test_random_holders(seed, copies_last):
         c.check()
 
 
-def test_equal_fills_take_one_launch():
-    c = Caches(64, 60, True)
+def test_equal_fills_take_one_launch(caches):
+    c = caches(64, 60, True)
     a = c.new(70)
     hs = [a] + [c.fork(a) for _ in range(9)]
     c.append_batch(hs)
